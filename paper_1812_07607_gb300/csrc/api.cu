@@ -17,6 +17,7 @@
 
 #include "checked.cuh"
 #include "kernels.h"
+#include "simt_tile.cuh"
 
 namespace dl {
 
@@ -550,8 +551,8 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
     } else if (hmetric) {
         // |D32 - D| <= g32 D + abs32 for the SIMT evaluation, |D64 - D| <= g64 D for the canonical sum
         const double g64 = (hmetric == 1) ? gamma64(d) : gamma64(d + 4);
-        const double g32 = (hmetric == 1) ? (d + 4) * 1.1920928955078125e-07 : (d + 16) * 1.1920928955078125e-07;
-        const double abs32 = (hmetric == 1) ? d * 7.52316384526264e-37 : d * 2.168404344971009e-19;   // d 2^-120, d 2^-62
+        const double g32 = (hmetric == 1) ? (d + 4) * 1.1920928955078125e-07 : chi2_g32(d);
+        const double abs32 = (hmetric == 1) ? d * 7.52316384526264e-37 : chi2_abs32(d);   // L1: d 2^-120
         c.t_acc = f32_rd(eps * (1.0 - g64) * (1.0 - g32) * (1.0 - 8.881784197001252e-16) - abs32);
         c.t_rej = f32_ru(eps * (1.0 + 2.0 * g64) * (1.0 + g32) * (1.0 + 8.881784197001252e-16) + abs32);
     } else {
