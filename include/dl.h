@@ -68,14 +68,18 @@ typedef enum dl_metric {
 } dl_metric;
 
 typedef enum dl_precision {
-    DL_PREC_AUTO = 0,       /* BF16 tensor-core path when d <= 512, else FP8 e4m3 (ε-join);
-                               top-k: BF16 when d <= 512, else FP32 */
+    DL_PREC_AUTO = 0,       /* ε-join: FP16 tensor-core path when d <= 512 (BF16 when a store's features
+                               span too wide a range), else FP8 e4m3, or FP16 for large joins;
+                               top-k: FP16 or BF16 when d <= 512, else FP32 */
     DL_PREC_BF16 = 1,       /* -2 q.x on tcgen05 tensor cores in BF16, FP32 accumulate; exact result */
     DL_PREC_FP8E4M3 = 2,    /* as BF16 but FP8 e4m3 with power-of-two scales (per 32-row chunk of
                                each store); exact result */
     DL_PREC_FP32 = 3,       /* FP32 SIMT distances + bound + FP64 recheck; exact result */
-    DL_PREC_FP32_PLAIN = 4  /* plain FP32 SIMT join D32 <= (float)(eps*eps): the comparison
+    DL_PREC_FP32_PLAIN = 4, /* plain FP32 SIMT join D32 <= (float)(eps*eps): the comparison
                                baseline, NOT exact near the threshold */
+    DL_PREC_FP16 = 5        /* as BF16 but FP16 with one power-of-two scale per store; exact result.
+                               DL_EUNSUPPORTED when a store's rows span more than a factor of 2^18 in
+                               their largest magnitudes (AUTO takes BF16 there) */
 } dl_precision;
 
 typedef enum dl_memkind {
@@ -124,7 +128,7 @@ void dl_join_opts_default(dl_join_opts *o);
  * Create a store of n patches with int64 `ids` [n] and float32 `feats` [n][d]
  * (row-major, contiguous). `where` tells whether both pointers are host or
  * device memory; the data are copied, then one pass (K1) derives the per-row
- * norms, the BF16 copy and the error-bound statistics the join kernels use.
+ * norms, the 16-bit copy and the error-bound statistics the join kernels use.
  * Requirements: 1 <= d <= 1024, 0 <= n < 2^31, every feature finite with
  * |x| <= 2^40 (else DL_EINVAL). Ids are opaque and may repeat. On success *out
  * owns device memory until dl_store_destroy. Ordered on `cuda_stream`; the
@@ -283,7 +287,7 @@ int dl_sim_join_noalloc(const float *R, const int64_t *r_ids, int64_t nR, const 
 /*
  * Diagnostics for the error bound of the low-precision stage (no counterpart in
  * the paper). Runs the tensor-core pass of an R x S join in `precision`
- * (DL_PREC_BF16 or DL_PREC_FP8E4M3) and writes, for every pair at the callers'
+ * (DL_PREC_BF16, DL_PREC_FP16 or DL_PREC_FP8E4M3) and writes, for every pair at the callers'
  * row order, the kernel's approximation h~ of h = q.x - ||x||^2/2 (so that
  * D = ||q||^2 - 2h) into h_out[|R|][|S|] and the bound E it uses into
  * e_out[|R|][|S|] (device memory, caller-owned). |R| |S| <= 2^28. A sound kernel

@@ -170,6 +170,8 @@ struct PassOut {
     int grid = 0;           // CTAs of the tensor-core launch
 };
 
+static bool tc_prec(int prec) { return prec == DL_PREC_BF16 || prec == DL_PREC_FP16 || prec == DL_PREC_FP8E4M3; }
+
 static int run_pass(const PassCfg &c, PassOut *po)
 {
     const dl_store *R = c.R, *S = c.S;
@@ -229,24 +231,29 @@ static int run_pass(const PassCfg &c, PassOut *po)
     int launches = 0;
     if (nR > 0 && nS > 0) {
         NvtxScope nvtx_pass("join pass: distances, bounds, compaction, recheck");
-        if (c.prec == DL_PREC_BF16 || c.prec == DL_PREC_FP8E4M3) {
+        if (tc_prec(c.prec)) {
             const bool fp8 = c.prec == DL_PREC_FP8E4M3;
+            const int fmt = c.prec == DL_PREC_FP16 ? kHalfF16 : kHalfBF16;
+            Half *hR = nullptr, *hS = nullptr;
             if (fp8) {
                 rc = ensure_fp8(const_cast<dl_store *>(R), st);
                 if (!rc) rc = ensure_fp8(const_cast<dl_store *>(S), st);
+            } else {
+                rc = get_half(const_cast<dl_store *>(R), fmt, st, &hR);
+                if (!rc) rc = get_half(const_cast<dl_store *>(S), fmt, st, &hS);
             }
             if (!rc && c.ip) rc = ensure_ip(const_cast<dl_store *>(S), st);
             if (!rc && c.ip)
-                rc = launch_rowpar_ip(R->rowb, nR, rows_pad, R->dp, c.e2, rowpar, st);
+                rc = launch_rowpar_ip(hR->rowb, nR, rows_pad, R->dp, c.e2, rowpar, st);
             else if (!rc)
-                rc = launch_rowpar(R->nq64, R->rowb, nR, rows_pad, R->dp, c.e2, nullptr, gamma64(d), rowpar, st,
-                                   fp8 ? R->rowb8 : nullptr);
+                rc = launch_rowpar(R->nq64, fp8 ? nullptr : hR->rowb, nR, rows_pad, R->dp, c.e2, nullptr, gamma64(d), rowpar,
+                                   st, fp8 ? R->rowb8 : nullptr);
             ++launches;
             const CUtensorMap *tmA = nullptr, *tmB = nullptr;
-            if (!rc) rc = fp8 ? get_tmap8(const_cast<dl_store *>(R), 128, &tmA) : get_tmap(const_cast<dl_store *>(R), 128, &tmA);
+            if (!rc) rc = fp8 ? get_tmap8(const_cast<dl_store *>(R), 128, &tmA) : get_tmap(const_cast<dl_store *>(R), hR, 128, &tmA);
             const int b_rows = c.cg2 ? c.BN / 2 : c.BN;   // an SM pair loads half of each S tile per SM
             if (!rc)
-                rc = fp8 ? get_tmap8(const_cast<dl_store *>(S), b_rows, &tmB) : get_tmap(const_cast<dl_store *>(S), b_rows, &tmB);
+                rc = fp8 ? get_tmap8(const_cast<dl_store *>(S), b_rows, &tmB) : get_tmap(const_cast<dl_store *>(S), hS, b_rows, &tmB);
             const int4 *units = nullptr;
             int n_units = 0;
             if (!rc && c.units) {
@@ -272,11 +279,13 @@ static int run_pass(const PassCfg &c, PassOut *po)
                 L.p.nR = (int)nR;
                 L.p.nS = (int)nS;
                 L.p.kc = fp8 ? R->dp8 / 128 : R->dp / 64;
+                L.p.fmt = fmt == kHalfBF16;
+                L.p.scale = fp8 ? 1.0f : hR->scale * hS->scale;
                 tc_plan(c.BN, L.p.kc, &L.p.stages, &L.p.a_slots, fp8, c.cg2, c.wide, !c.pruned);
                 L.p.upper = c.self ? 1 : 0;
                 L.p.rowpar = rowpar;
                 L.p.beta = c.ip ? S->beta_ip : S->beta;
-                L.p.cstat = fp8 ? S->cstat8 : (c.ip ? S->cstat_ip : S->cstat);
+                L.p.cstat = fp8 ? S->cstat8 : (c.ip ? S->cstat_ip : hS->cstat);
                 L.p.sc_r = fp8 ? R->sc8 : nullptr;
                 L.p.sc_s = fp8 ? S->scc8 : nullptr;
                 L.p.cand = band;                 // candidates share the band buffer and counter
@@ -309,7 +318,7 @@ static int run_pass(const PassCfg &c, PassOut *po)
             rc = launch_finalize_ip(band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2, jo, cnt + 3,
                                     cnt + 2, sms * 8, st, (int)nR, (int)nS);
             ++launches;
-        } else if (!rc && (c.prec == DL_PREC_BF16 || c.prec == DL_PREC_FP8E4M3)) {
+        } else if (!rc && tc_prec(c.prec)) {
             rc = launch_finalize(band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2, c.t_acc,
                                  c.t_rej, jo, cnt + 3, cnt + 2, sms * 8, st, (int)nR, (int)nS);
             ++launches;
@@ -343,7 +352,7 @@ static int run_pass(const PassCfg &c, PassOut *po)
     if (!rc) {
         po->out_cnt = hc[0];
         po->band_cnt = hc[1];                                  // list fill (band or candidate list)
-        po->band_only = (c.prec == DL_PREC_BF16 || c.prec == DL_PREC_FP8E4M3) ? hc[2] : hc[1];
+        po->band_only = tc_prec(c.prec) ? hc[2] : hc[1];
         po->fp64_cnt = hc[3];
         po->err = (int)hc[4];
         if (c.timing) {
@@ -365,6 +374,11 @@ static int run_pass(const PassCfg &c, PassOut *po)
 // join of a new store sizes its buffers from them.
 static std::mutex g_rate_mu;
 static double g_rate_out = 0.0, g_rate_band = 0.0;
+
+// AUTO above d = 512 takes FP16 from this many pairs on. FP16 is the faster one below it as well (300 x
+// 700, d = 640: 63 us, FP8 86; 2,000 x 2,000: 64 and 199), but small joins keep the FP8 path that AUTO
+// has always documented and reported for these widths; here it costs 20 us, further up milliseconds.
+constexpr double kWideF16Pairs = 262144.0;   // 2^18
 
 static int check_device(const dl_store *s)
 {
@@ -462,17 +476,30 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
     if (!rc) rc = check_device(Sx);
     if (rc) return rc;
     int prec = o.precision;
-    // AUTO: BF16 while its R tile fits in shared memory (d <= 512), else the FP8 tensor-core
-    // path (d <= 1024, always within the domain); both give the exact set. The histogram
-    // distances are not contractions: they run on the CUDA cores (FP32 + bound + FP64).
+    // AUTO, all of them exact: FP16 where both stores hold it, else BF16, while the R tile fits in
+    // shared memory (d <= 512). Above that FP8, unless the join is large (kWideF16Pairs): FP8's tensor
+    // time is half FP16's, but its 3-bit fraction leaves many more pairs to the FP32 recheck, 8 d bytes
+    // of rows each (65,536 x 50,001, d = 1024, unit-norm mixture: 16.8 M pairs, 2.6 + 9.3 ms; in FP16
+    // 0.56 M pairs, 4.0 + 0.4 ms). The histogram distances are not contractions: they run on the CUDA cores (FP32 +
+    // bound + FP64).
     const bool ip = metric == DL_METRIC_IP;
-    if (prec == DL_PREC_AUTO)
-        prec = hmetric ? DL_PREC_FP32 : (ip || R->dp <= 512) ? DL_PREC_BF16 : DL_PREC_FP8E4M3;
+    const bool f16 = R->h.fmt == kHalfF16 && Sx->h.fmt == kHalfF16;
+    if (prec == DL_PREC_AUTO) {
+        if (hmetric)
+            prec = DL_PREC_FP32;
+        else if (ip)
+            prec = DL_PREC_BF16;
+        else if (R->dp <= 512)
+            prec = f16 ? DL_PREC_FP16 : DL_PREC_BF16;
+        else
+            prec = f16 && !o.prune && o.cta_pair != 2 && (double)R->n * (double)Sx->n >= kWideF16Pairs ? DL_PREC_FP16
+                                                                                                       : DL_PREC_FP8E4M3;
+    }
     if (ip && (prec != DL_PREC_BF16 || (self && o.self_mode == DL_SELF_FULL) || o.prune)) {
         set_error("dl_sim_join: the inner-product join runs in BF16, R x S or the upper self mode, without pruning");
         return DL_EUNSUPPORTED;
     }
-    if (hmetric && (prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3)) {
+    if (hmetric && tc_prec(prec)) {
         set_error("dl_sim_join: L1 and chi-square run on DL_PREC_FP32 (or FP32_PLAIN), not on tensor cores");
         return DL_EUNSUPPORTED;
     }
@@ -486,12 +513,16 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
             return DL_EINVAL;
         }
     }
-    if (prec != DL_PREC_BF16 && prec != DL_PREC_FP8E4M3 && prec != DL_PREC_FP32 && prec != DL_PREC_FP32_PLAIN) {
+    if (!tc_prec(prec) && prec != DL_PREC_FP32 && prec != DL_PREC_FP32_PLAIN) {
         set_error("dl_sim_join: bad precision %d", prec);
         return DL_EINVAL;
     }
     if (prec == DL_PREC_BF16 && R->dp > 512) {
         set_error("dl_sim_join: BF16 tensor-core path supports d <= 512 (d=%d)", R->d);
+        return DL_EUNSUPPORTED;
+    }
+    if (prec == DL_PREC_FP16 && (!f16 || (R->dp > 512 && (o.prune || o.cta_pair == 2)))) {
+        set_error("dl_sim_join: FP16 needs features within FP16's range in both stores, and d <= 512 with prune or cta_pair 2");
         return DL_EUNSUPPORTED;
     }
     if (o.tile_n != 0 && o.tile_n != 128 && o.tile_n != 256) {
@@ -508,9 +539,10 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
         return DL_EINVAL;
     }
     // tile configuration: given, or autotuned per shape class (tensor-core precisions, dense join)
-    const bool tc = prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3;
-    const int tune_kind = (prec == DL_PREC_FP8E4M3) ? (self ? kTuneEpsSelf8 : kTuneEpsRxS8)
-                                                    : (self ? kTuneEpsSelf : kTuneEpsRxS);
+    const bool tc = tc_prec(prec);
+    const int tune_kind = prec == DL_PREC_FP8E4M3 ? (self ? kTuneEpsSelf8 : kTuneEpsRxS8)
+                          : prec == DL_PREC_FP16  ? (self ? kTuneEpsSelf16 : kTuneEpsRxS16)
+                                                  : (self ? kTuneEpsSelf : kTuneEpsRxS);
     bool tune_trial = false;
     int code = (o.tile_n ? o.tile_n : 256) | (o.cta_pair == 2 ? kTunePair : 0) | (o.epilogue_warps == 16 ? kTuneWide : 0);
     if (tc && !o.prune && o.tile_n == 0 && o.cta_pair == 0 && o.epilogue_warps == 0)
@@ -575,14 +607,14 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
             hb = (int64_t)std::min(g_rate_band * n_pairs, (double)(1 << 26));
         }
         c.cap = fixed ? o.out_capacity : std::max<int64_t>(1 << 16, hp + hp / 4);
-        // the BF16 path's candidate list holds proven matches and band pairs
-        const int64_t want = ((prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3) ? hp : 0) + hb;
+        // the tensor-core paths' candidate list holds proven matches and band pairs
+        const int64_t want = (tc ? hp : 0) + hb;
         c.band_cap = std::max<int64_t>(1 << 16, want + want / 4);
     }
 
     PruneUnits pu;
     int64_t tiles_total = 0, tiles_kept = 0;
-    if (o.prune && (prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3) && hmetric == 0) {
+    if (o.prune && tc && hmetric == 0) {
         rc = prune_units(R, Sx, self, BN, e2, c.st, &pu);
         if (rc) return rc;
         c.units = pu.units;
@@ -666,9 +698,9 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
     s.fp64_pairs = (int64_t)po.fp64_cnt;
     s.reruns = reruns;
     s.precision = prec;
-    s.tile_n = (prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3) ? BN : 0;
-    s.cta_pair = (prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3) ? (cg2 ? 2 : 1) : 0;
-    s.epilogue_warps = (prec == DL_PREC_BF16 || prec == DL_PREC_FP8E4M3) ? (wide ? 16 : 8) : 0;
+    s.tile_n = tc ? BN : 0;
+    s.cta_pair = tc ? (cg2 ? 2 : 1) : 0;
+    s.epilogue_warps = tc ? (wide ? 16 : 8) : 0;
     s.ms_main = po.ms_main;
     s.ms_recheck = po.ms_recheck;
     s.ms_total = po.ms_total;
@@ -722,8 +754,8 @@ int dl_debug_scores(const dl_store *R, const dl_store *S, int32_t precision, flo
         set_error("dl_debug_scores: bad arguments");
         return DL_EINVAL;
     }
-    if (precision != DL_PREC_BF16 && precision != DL_PREC_FP8E4M3) {
-        set_error("dl_debug_scores: precision must be BF16 or FP8");
+    if (!tc_prec(precision)) {
+        set_error("dl_debug_scores: precision must be BF16, FP16 or FP8");
         return DL_EINVAL;
     }
     if (R->n * S->n > (int64_t(1) << 28) || R->n == 0 || S->n == 0) {
@@ -731,17 +763,22 @@ int dl_debug_scores(const dl_store *R, const dl_store *S, int32_t precision, flo
         return DL_EINVAL;
     }
     const bool fp8 = precision == DL_PREC_FP8E4M3;
-    if ((!fp8 && R->dp > 512) || (fp8 && R->d > 1024)) {
+    if ((precision == DL_PREC_BF16 && R->dp > 512) || (fp8 && R->d > 1024)) {
         set_error("dl_debug_scores: d too large for this precision");
         return DL_EUNSUPPORTED;
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
     int rc = DL_OK;
+    const int fmt = precision == DL_PREC_FP16 ? kHalfF16 : kHalfBF16;
+    Half *hR = nullptr, *hS = nullptr;
     if (fp8) {
         rc = ensure_fp8(const_cast<dl_store *>(R), st);
         if (!rc) rc = ensure_fp8(const_cast<dl_store *>(S), st);
-        if (rc) return rc;
+    } else {
+        rc = get_half(const_cast<dl_store *>(R), fmt, st, &hR);
+        if (!rc) rc = get_half(const_cast<dl_store *>(S), fmt, st, &hS);
     }
+    if (rc) return rc;
     const int64_t mt = (R->n + 127) / 128;
     void *ws = nullptr;
     rc = dev_alloc(&ws, 256 + mt * 128 * sizeof(float4) + 65536 * sizeof(uint2), st);
@@ -751,12 +788,12 @@ int dl_debug_scores(const dl_store *R, const dl_store *S, int32_t precision, flo
     uint2 *cand = (uint2 *)((char *)rowpar + mt * 128 * sizeof(float4));
     cudaMemsetAsync(cnt, 0, 256, st);
     // thresholds for eps = 0 (the dump does not depend on them; candidates are discarded)
-    rc = launch_rowpar(R->nq64, R->rowb, R->n, mt * 128, R->dp, 0.0, nullptr, gamma64(R->d), rowpar, st,
+    rc = launch_rowpar(R->nq64, fp8 ? nullptr : hR->rowb, R->n, mt * 128, R->dp, 0.0, nullptr, gamma64(R->d), rowpar, st,
                        fp8 ? R->rowb8 : nullptr);
     const CUtensorMap *tmA = nullptr, *tmB = nullptr;
     const int BN = 256;
-    if (!rc) rc = fp8 ? get_tmap8(const_cast<dl_store *>(R), 128, &tmA) : get_tmap(const_cast<dl_store *>(R), 128, &tmA);
-    if (!rc) rc = fp8 ? get_tmap8(const_cast<dl_store *>(S), BN, &tmB) : get_tmap(const_cast<dl_store *>(S), BN, &tmB);
+    if (!rc) rc = fp8 ? get_tmap8(const_cast<dl_store *>(R), 128, &tmA) : get_tmap(const_cast<dl_store *>(R), hR, 128, &tmA);
+    if (!rc) rc = fp8 ? get_tmap8(const_cast<dl_store *>(S), BN, &tmB) : get_tmap(const_cast<dl_store *>(S), hS, BN, &tmB);
     const int4 *units = nullptr;
     int n_units = 0;
     if (!rc) rc = get_units(R->n, S->n, false, BN, device_sm_count(), &units, &n_units);
@@ -772,10 +809,12 @@ int dl_debug_scores(const dl_store *R, const dl_store *S, int32_t precision, flo
         L.p.nR = (int)R->n;
         L.p.nS = (int)S->n;
         L.p.kc = fp8 ? R->dp8 / 128 : R->dp / 64;
-        tc_plan(BN, L.p.kc, &L.p.stages, &L.p.a_slots, fp8);
+        L.p.fmt = fmt == kHalfBF16;
+        L.p.scale = fp8 ? 1.0f : hR->scale * hS->scale;
+        tc_plan(BN, L.p.kc, &L.p.stages, &L.p.a_slots, fp8, false, false, precision == DL_PREC_FP16);
         L.p.rowpar = rowpar;
         L.p.beta = S->beta;
-        L.p.cstat = fp8 ? S->cstat8 : S->cstat;
+        L.p.cstat = fp8 ? S->cstat8 : hS->cstat;
         L.p.sc_r = fp8 ? R->sc8 : nullptr;
         L.p.sc_s = fp8 ? S->scc8 : nullptr;
         L.p.cand = cand;

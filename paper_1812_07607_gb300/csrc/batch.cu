@@ -372,6 +372,17 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
             set_error("dl_batch_join: epsilon requests need d <= 512 (d=%d)", d);
             return DL_EUNSUPPORTED;
         }
+        // both stores' 16-bit copies in one format: FP16 where both hold it, unless BF16 was asked for
+        const int fmt = Qe->h.fmt == kHalfF16 && S->h.fmt == kHalfF16 && o.precision != DL_PREC_BF16 ? kHalfF16 : kHalfBF16;
+        Half *hQ = nullptr, *hS = nullptr;
+        rc = get_half(Qe, fmt, st, &hQ);
+        if (!rc) rc = get_half(const_cast<dl_store *>(S), fmt, st, &hS);
+        if (rc) {
+            dev_free(tk_block, st);
+            cleanup();
+            return rc;
+        }
+        stats.precision = fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
         bool tune_trial = false;
         const int code = o.tile_n ? o.tile_n : tune_pick(Qe->dp, kTuneBatch, ne, S->n, &tune_trial);
         const int BN = tune_bn(code);
@@ -420,10 +431,10 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
                 dev_free(ws, st);
                 break;
             }
-            rc = launch_rowpar(Qe->nq64, Qe->rowb, ne, mt * 128, Qe->dp, 0.0, row_e2, gamma64(d), rowpar, st);
+            rc = launch_rowpar(Qe->nq64, hQ->rowb, ne, mt * 128, Qe->dp, 0.0, row_e2, gamma64(d), rowpar, st);
             const CUtensorMap *tmA = nullptr, *tmB = nullptr;
-            if (!rc) rc = get_tmap(Qe, 128, &tmA);
-            if (!rc) rc = get_tmap(const_cast<dl_store *>(S), BN, &tmB);
+            if (!rc) rc = get_tmap(Qe, hQ, 128, &tmA);
+            if (!rc) rc = get_tmap(const_cast<dl_store *>(S), hS, BN, &tmB);
             if (!rc) {
                 TcLaunch L;
                 std::memset(&L.p, 0, sizeof L.p);
@@ -436,12 +447,14 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
                 L.p.nR = (int)ne;
                 L.p.nS = (int)S->n;
                 L.p.kc = Qe->dp / 64;
+                L.p.fmt = fmt == kHalfBF16;
+                L.p.scale = hQ->scale * hS->scale;
                 tc_plan(BN, Qe->dp / 64, &L.p.stages, &L.p.a_slots, false, false, wide, true);
                 L.wide = wide;
                 L.p.upper = 0;
                 L.p.rowpar = rowpar;
                 L.p.beta = S->beta;
-                L.p.cstat = S->cstat;
+                L.p.cstat = hS->cstat;
                 L.p.cand = cand;
                 L.p.cand_cnt = cnt + 0;
                 L.p.cand_cap = (unsigned long long)cap;

@@ -58,7 +58,7 @@ inline double gamma64(int d) { return (d + 4) * kU64; }
 // tree): (d + 8) 2^-24.
 inline double gamma32(int d) { return (d + 8) * kU32; }
 
-// Assumed relative bound of the tensor-core FP32 accumulation of d BF16 x BF16
+// Assumed relative bound of the tensor-core FP32 accumulation of d 16-bit x 16-bit
 // products (the products are exact in FP32; summation order and rounding of the
 // hardware adder are not documented): d * 2^-20, sixteen times the textbook
 // d * 2^-24. Checked empirically by the bound-validity test.
@@ -74,21 +74,31 @@ struct TmapCache {
     CUtensorMap map;
 };
 
+// A 16-bit copy of a store's rows for the tensor cores, with the statistics of its rounding.
+enum HalfFormat { kHalfF16 = 0, kHalfBF16 = 1 };
+struct Half {
+    int fmt = kHalfBF16;
+    float scale = 1.0f;      // x~ = scale * code: a power of two for FP16, 1 for BF16
+    uint16_t *x = nullptr;   // [n][dp] codes, zero padded
+    float4 *rowb = nullptr;  // [n] {||x - x~|| up, ||x~|| up, ||x|| up, |beta - ||x||^2/2| up}
+    float4 *cstat = nullptr; // [n_pad / 32] per 32-row chunk {P1, P2, P3, min beta} of the bound
+    TmapCache tmaps[3];      // cached per box height
+};
+
 struct Store {
     int64_t n = 0;
     int32_t d = 0;
-    int32_t dp = 0;          // d rounded up to a multiple of 64 (BF16 copy row length)
+    int32_t dp = 0;          // d rounded up to a multiple of 64 (16-bit copies' row length)
     int64_t n_pad = 0;       // n rounded up to a multiple of 256 (column-side padding)
     int device = 0;
     int64_t *ids = nullptr;  // [n] ids, in store order
     int32_t *orig = nullptr; // [n] caller's row index of each store row (rows are kept in norm order)
     float *x32 = nullptr;    // [n][d] FP32 master copy, in store order
-    __nv_bfloat16 *xb = nullptr;  // [n][dp] BF16 copy, zero padded
     double *nq64 = nullptr;  // [n] sum of squares in FP64
     float *beta = nullptr;   // [n_pad] RN32(nq64 / 2); +inf in padding
-    float4 *rowb = nullptr;  // [n] {||x - x~|| up, ||x~|| up, ||x|| up, |beta - ||x||^2/2| up}
-    float4 *cstat = nullptr; // [n_pad / 32] per 32-row chunk {P1, P2, P3, min beta} of the BF16 bound
-    TmapCache tmaps[3];      // BF16 boxes, cached per box height
+    Half h;                  // the 16-bit copy every store holds: FP16, or BF16 for wide-range features
+    Half alt;                // BF16 copy of a store that holds FP16 (built on first use)
+    void *alt_block = nullptr;
     // FP8 e4m3 copy (built on the first FP8 join): row i is s_i * e4m3 codes, s_i a power of two
     int32_t dp8 = 0;         // d rounded up to a multiple of 128 (one 128-byte swizzle row per K chunk)
     void *fp8_block = nullptr;
@@ -147,9 +157,12 @@ struct PruneUnits {
 };
 int prune_units(const dl_store *R, const dl_store *S, bool upper, int BN, double e2, cudaStream_t st, PruneUnits *pu);
 
-// Build (or fetch from the store's cache) a 2-D BF16 tensor map over the store's
-// BF16 copy with a box of 64 columns x box_rows rows and the 128-byte swizzle.
-int get_tmap(Store *s, int box_rows, const CUtensorMap **out);
+// The store's 16-bit copy in the given format: FP16 only where the store holds it (DL_EUNSUPPORTED
+// otherwise), BF16 always (built on first use where the store holds FP16).
+int get_half(Store *s, int fmt, cudaStream_t st, Half **out);
+// Build (or fetch from the copy's cache) a 2-D tensor map over a 16-bit copy with a box of 64
+// columns x box_rows rows and the 128-byte swizzle.
+int get_tmap(Store *s, Half *h, int box_rows, const CUtensorMap **out);
 
 // FP8 copy of a store (built once, on first use) and its tensor maps (128-byte rows).
 int ensure_fp8(Store *s, cudaStream_t st);
@@ -173,7 +186,8 @@ int device_sm_count();
 // kTuneWide for the 16-warp epilogue.
 constexpr int kTunePair = 1 << 12;
 constexpr int kTuneWide = 1 << 13;
-enum TuneKind { kTuneEpsRxS = 0, kTuneEpsSelf = 1, kTuneTopk = 2, kTuneEpsRxS8 = 3, kTuneEpsSelf8 = 4, kTuneBatch = 5 };
+enum TuneKind { kTuneEpsRxS = 0, kTuneEpsSelf = 1, kTuneTopk = 2, kTuneEpsRxS8 = 3, kTuneEpsSelf8 = 4, kTuneBatch = 5,
+                kTuneEpsRxS16 = 6, kTuneEpsSelf16 = 7 };
 inline int tune_bn(int code) { return code & 0xfff; }
 inline bool tune_pair(int code) { return (code & kTunePair) != 0; }
 inline bool tune_wide(int code) { return (code & kTuneWide) != 0; }

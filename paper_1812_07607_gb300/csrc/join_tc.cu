@@ -3,15 +3,16 @@
 // The nested-loop join of Sec. 5 evaluates every pair (q, x). With
 //   D(q, x) = ||q||^2 + ||x||^2 - 2 q.x
 // the only pair-wise term is the dot product, a dense contraction. This kernel
-// computes A = Q~ X~^T on the tcgen05 tensor cores (BF16 or FP8 e4m3 in, FP32
+// computes A = Q~ X~^T on the tcgen05 tensor cores (FP16, BF16 or FP8 e4m3 in, FP32
 // accumulate in TMEM) and classifies every pair in a fused epilogue against per-row
 // thresholds that carry a proven error bound, so that each pair is either a proven
 // match, a proven non-match, or an undecided "band" pair that the recheck settles
 // exactly. With h = q.x - ||x||^2/2 the epilogue works on h~ = fl(A s - beta)
-// (s = 1 for BF16; for FP8 the exact power of two s_q s_chunk).
+// (s = 1 for BF16, the power of two s_R s_S of the two stores for FP16, and for FP8 the power of two
+// s_q s_chunk of the row and the 32-column chunk).
 //
 // Per CTA (persistent, one per SM, 320 threads, warp-specialised):
-//   warp 0      TMA producer: the 128-row R tile (all K chunks of 128 bytes: 64 BF16
+//   warp 0      TMA producer: the 128-row R tile (all K chunks of 128 bytes: 64 16-bit
 //               or 128 FP8 columns) is loaded once per unit into one of one or two A
 //               slots; S tiles stream through a ring of stages, one K chunk of BN
 //               rows per stage (128-byte swizzle).
@@ -130,7 +131,7 @@ __device__ __forceinline__ void flush_stage(const TcParams &p, uint2 *stg, uint3
 }
 
 // Pair-by-pair path for one 32-column chunk, for pairs (r, c0 + j) with h = fl(A s - beta_j)
-// (s = 1 for BF16; for FP8 the exact power of two s_q s_chunk, so one rounding). A pair with
+// (s an exact power of two, so one rounding). A pair with
 // h >= tau_rej of its row -- a proven match
 // (h >= tau_acc) or a band pair -- becomes a candidate. Warp-collective; `hit` marks the
 // lanes (rows) whose chunk bound failed, the others have no candidate in this chunk.
@@ -317,7 +318,7 @@ __device__ __forceinline__ void slow_topk(const TcParams &p, const uint32_t (&v)
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
             const int c = col0 + hh * 32 + j;
-            const float h = __uint_as_float(v[hh * 32 + j]) - bt[hh * 32 + j];
+            const float h = __fmaf_rn(__uint_as_float(v[hh * 32 + j]), p.scale, -bt[hh * 32 + j]);
             const float U = __fadd_ru(h, eh);
             if (c < p.nS && U >= fmaxf(theta, theta_row)) {
                 const float2 st = topk_insert(p, sidx, r, c, U, __fsub_rd(h, eh), theta, cnt, theta_row);
@@ -469,7 +470,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
                         break;
                     }
                     mbar_arrive_expect_tx(a_full + slot, a_bytes);
-                    for (int c = 0; c < kc; ++c)   // a K chunk is 128 bytes: 64 BF16 or 128 FP8 columns
+                    for (int c = 0; c < kc; ++c)   // a K chunk is 128 bytes: 64 16-bit or 128 FP8 columns
                         tma_load_2d(sA + slot * a_bytes + c * 16384, &tmA, a_full + slot, c * kChunkCols,
                                     (un.x * kRowTiles + (int)crank) * 128);
                     a_pend[slot] = true;
@@ -542,8 +543,8 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc =
-                FP8 ? idesc_e4m3_f32(CG2 ? 256 : 128, BN) : idesc_bf16_f32(CG2 ? 256 : 128, BN);
+            const uint32_t idesc = FP8 ? idesc_e4m3_f32(CG2 ? 256 : 128, BN)
+                                       : idesc_f16_f32(CG2 ? 256 : 128, BN) | (p.fmt ? kIdescBF16 : 0u);
             uint32_t stage = 0, phase = 0, t = 0;
             bool ok = true, any_mma = false;
             int i = 0;
@@ -724,7 +725,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             // 64 columns [piece*64, piece*64+64) of this warp's half, values in v
             auto process64 = [&](uint32_t (&v)[64], int piece) {
                 // FP8: h = fl(A s_q s_chunk - beta), one rounding (the scale product is an exact power of two)
-                const float sc0 = FP8 ? sq * sxs[2 * piece] : 1.0f, sc1 = FP8 ? sq * sxs[2 * piece + 1] : 1.0f;
+                const float sc0 = FP8 ? sq * sxs[2 * piece] : p.scale, sc1 = FP8 ? sq * sxs[2 * piece + 1] : p.scale;
                 const float4 cs0 = cst[2 * piece], cs1 = cst[2 * piece + 1];
                 const float eh0 = __fmaf_ru(rp.z, cs0.x, __fmaf_ru(rp.w, cs0.y, cs0.z));
                 const float eh1 = __fmaf_ru(rp.z, cs1.x, __fmaf_ru(rp.w, cs1.y, cs1.z));
@@ -772,7 +773,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
 
             // One 32-column chunk ci of this warp's HC columns, values v[o .. o+31] (epsilon-join).
             auto eps_chunk = [&](auto &v, int o, int ci) {
-                const float sc = FP8 ? sq * sxs[ci] : 1.0f;
+                const float sc = FP8 ? sq * sxs[ci] : p.scale;
                 const float4 cs = cst[ci];
                 const float eh = __fmaf_ru(rp.z, cs.x, __fmaf_ru(rp.w, cs.y, cs.z));
                 if (p.dump_h) {   // diagnostics: every pair's h and bound, at caller row order
@@ -808,17 +809,17 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
                     }
                 }
             };
-            // Top-k, one 32-column chunk ci (BF16 only: scale 1): the columns whose upper bound
+            // Top-k, one 32-column chunk ci (16-bit operands): the columns whose upper bound
             // reaches the best threshold go to the slot's list, their lower bounds to its heap.
             auto topk_chunk = [&](auto &v, int o, int ci) {
                 const float4 cs = cst[ci];
                 const float ehs = __fadd_ru(__fmaf_ru(rp.z, cs.x, __fmaf_ru(rp.w, cs.y, cs.z)), rp.x);
                 const float mx = max_tree32(v, o);
-                if (__fsub_ru(mx, cs.w) >= __fsub_rd(fmaxf(theta, theta_row), ehs) && r < p.nR) {
+                if (__fmaf_ru(mx, p.scale, -cs.w) >= __fsub_rd(fmaxf(theta, theta_row), ehs) && r < p.nR) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
                         const int c = colw + ci * 32 + j;
-                        const float h = __uint_as_float(v[o + j]) - beta[ci * 32 + j];
+                        const float h = __fmaf_rn(__uint_as_float(v[o + j]), p.scale, -beta[ci * 32 + j]);
                         const float U = __fadd_ru(h, ehs);
                         if (c < p.nS && U >= fmaxf(theta, theta_row)) {
                             const float2 stt = topk_insert(p, sidx, r, c, U, __fsub_rd(h, ehs), theta, tcnt, theta_row);
@@ -988,7 +989,7 @@ static int launch_one(const TcLaunch &L, size_t smem, cudaStream_t st, int *grid
 int launch_tc_join(const TcLaunch &L, cudaStream_t st, bool topk, bool fp8, int *grid_out)
 {
     if (topk && fp8) {
-        set_error("top-k runs on the BF16 path only");
+        set_error("top-k runs on the 16-bit path only");
         return DL_EUNSUPPORTED;
     }
     if ((L.cg2 && (topk || L.BN != 256 || L.wide)) || (L.wide && L.BN != 256)) {

@@ -16,7 +16,9 @@ struct TcParams {
     const uint32_t *tile_mask;   // when not NULL: [R tiles][mask_ntw] bits; a unit's S tiles with a
     int mask_ntw;                // clear bit are skipped (the pruned join; one-SM tiles only)
     int nR, nS;
-    int kc;                  // K chunks of 64 (dp / 64)
+    int kc;                  // K chunks of 128 bytes: 64 16-bit or 128 FP8 columns
+    uint32_t fmt;            // 16-bit operands: 0 when both are FP16, 1 when both are BF16
+    float scale;             // 16-bit operands: product of the two copies' scales (a power of two)
     int stages;              // S ring depth
     int a_slots;             // R-tile slots (2: the next unit's R tile loads during this one)
     int upper;               // 1: self-join, only columns c > r are pairs

@@ -201,7 +201,7 @@ __device__ __forceinline__ void tc_fence_after()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 (BF16 inputs here), FP32 accumulate.
+// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 (both inputs FP16 or both BF16), FP32 accumulate.
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t accumulate)
 {
@@ -287,15 +287,15 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr)
     return d;
 }
 
-// Instruction descriptor for kind::f16 with BF16 A/B, FP32 D, both K-major.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
+// Instruction descriptor for kind::f16, FP32 D, A and B both K-major and both FP16; with
+// kIdescBF16 added, both BF16.
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N)
 {
     return (1u << 4)                                   // D format: F32
-           | (1u << 7)                                 // A format: BF16
-           | (1u << 10)                                // B format: BF16
            | (static_cast<uint32_t>(N >> 3) << 17)     // N / 8
            | (static_cast<uint32_t>(M >> 4) << 24);    // M / 16
 }
+constexpr uint32_t kIdescBF16 = (1u << 7) | (1u << 10);   // A and B formats: BF16
 
 // Instruction descriptor for kind::f8f6f4 with E4M3 A/B (format code 0), FP32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_e4m3_f32(int M, int N)

@@ -143,8 +143,7 @@ __global__ void __launch_bounds__(256)
     const double nq_dn = __dmul_rd(nq, 1.0 - rel);
     const double a_acc = __dsub_ru(nq_up, __dmul_rd(e2, 1.0 - g64)) * 0.5;
     const double a_rej = __dsub_rd(nq_dn, __dmul_ru(e2, 1.0 + 2.0 * g64)) * 0.5;
-    const float4 rb = rowb[i];
-    const float2 r8 = rowb8 ? rowb8[i] : make_float2(rb.x, rb.y);
+    const float2 r8 = rowb8 ? rowb8[i] : make_float2(rowb[i].x, rowb[i].y);
     rowpar[i] = make_float4(__double2float_ru(a_acc), __double2float_rd(a_rej), r8.x, r8.y);
 }
 

@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstring>
 
+#include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
 #include "internal.h"
@@ -90,123 +91,219 @@ int device_sm_count()
 }
 
 // ------------------------------------------------------------------ K1
-// One warp per row. Computes, from the FP32 row x:
-//   nq64  = sum x_k^2 in FP64 (products exact, rounding only in the sum),
-//   the BF16 copy x~ = RN_bf16(x) (zero padded to dp),
-//   upper bounds of ||x - x~|| and ||x~|| (FP32 sums of squares rounded up at every
-//   step, square roots rounded up), and of ||x|| (from the FP64 sum, inflated by the
-//   sum and sqrt rounding),
-//   beta = RN32(nq64 / 2) and an upper bound of |beta - ||x||^2 / 2|,
-// and flags rows with a non-finite value or |x_k| > 2^40.
-__global__ void __launch_bounds__(256) k1_norm_quant(const float *__restrict__ x32, int64_t n, int d, int dp,
-                                                     __nv_bfloat16 *__restrict__ xb, double *__restrict__ nq64,
-                                                     float *__restrict__ beta, float4 *__restrict__ rowb,
-                                                     int *__restrict__ err)
+// Format of a store's 16-bit copy, from the largest feature magnitude of the store and the smallest
+// of its non-zero rows' largest: FP16 with one power-of-two scale s (x = s x16, the largest magnitude
+// just below 2^15 s) when every row is within 2^18 of the largest, so that a row's rounding stays at
+// FP16's 2^-12 of its large features and below 2^-21 of its largest for the small ones; BF16
+// otherwise. FP16 rounds eight times finer than BF16 at the same tensor-core rate, which leaves
+// about a fifth of the undecided pairs at d = 128 (the accumulation term of the bound stays).
+__host__ __device__ inline int half_format(unsigned max_bits, unsigned min_bits, float *scale)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row0 = ((int64_t)blockIdx.x * 8 + warp) * 32;   // this warp's 32 rows
-    if (row0 >= n) return;
-    const int rows = (int)(n - row0 < 32 ? n - row0 : 32);
-    // the sums of row r end in lane r, so the per-row tail (FP64, a square root) runs once per
-    // 32 rows with every lane busy: a warp-wide FP64 instruction costs the same at one lane
-    double m1 = 0.0;
-    float m2 = 0.f, m3 = 0.f;
-    bool mbad = false;
-    for (int r = 0; r < rows; ++r) {
-        const int64_t row = row0 + r;
-        const float *xr = x32 + row * d;
-        __nv_bfloat16 *br = xb + row * dp;
-        double s1 = 0.0;
-        float s2 = 0.f, s3 = 0.f;   // rounded up at every step: upper bounds of the exact sums
-        bool bad = false;
-        for (int k = lane; k < dp; k += 32) {
-            const float v = (k < d) ? __ldg(xr + k) : 0.0f;
-            if (!(fabsf(v) <= 1099511627776.0f)) bad = true;  // also catches NaN
-            const __nv_bfloat16 b = __float2bfloat16_rn(v);
-            br[k] = b;
-            const float fb = __bfloat162float(b);
-            const float e = v - fb;   // exact: x~ shares x's leading bits
-            const double dv = (double)v;
-            s1 = __dadd_rn(s1, __dmul_rn(dv, dv));
-            s2 = __fmaf_ru(e, e, s2);
-            s3 = __fmaf_ru(fb, fb, s3);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s1 = __dadd_rn(s1, __shfl_xor_sync(0xffffffffu, s1, o));
-            s2 = __fadd_ru(s2, __shfl_xor_sync(0xffffffffu, s2, o));
-            s3 = __fadd_ru(s3, __shfl_xor_sync(0xffffffffu, s3, o));
-        }
-        bad = __any_sync(0xffffffffu, bad);
-        if (lane == r) {
-            m1 = s1;
-            m2 = s2;
-            m3 = s3;
-            mbad = bad;
-        }
-    }
-    if (lane < rows) {
-        const int64_t row = row0 + lane;
-        const double s1 = m1;
-        const float s2 = m2, s3 = m3;
-        if (mbad) atomicOr(err, 1);
-        // Any-order FP64 sum of dp non-negative exact terms: relative error <= (dp-1) 2^-53.
-        const double fac = 1.0 + (double)(dp + 4) * 2.220446049250313e-16;
-        const double grow = 1.0 + 8.881784197001252e-16;   // 1 + 2^-50 covers the sqrt / product roundings
-        nq64[row] = s1;
-        const float rq = __fsqrt_ru(s2);
-        const float nqt = __fsqrt_ru(s3);
-        const float nx = __double2float_ru(sqrt(s1 * fac) * grow);
-        const double h = 0.5 * s1;
-        const float bt = __double2float_rn(h);
-        const float berr = __double2float_ru((fabs((double)bt - h) + h * (double)(dp + 2) * 2.220446049250313e-16) * grow);
-        beta[row] = bt;
-        rowb[row] = make_float4(rq, nqt, nx, berr);
-    }
+    *scale = 1.0f;
+    if (max_bits == 0u) return kHalfF16;                        // every feature is 0
+    const int e = (int)(max_bits >> 23) - 126, el = (int)(min_bits >> 23) - 126;   // max = m 2^e, m in [1/2, 1)
+    if (e < -47 || e > 41 || e - el > 18) return kHalfBF16;   // below 2^-47 two scales' product leaves the normal range
+    const unsigned sb = (unsigned)(e - 15 + 127) << 23;         // 2^(e - 15)
+    memcpy(scale, &sb, 4);
+    return kHalfF16;
 }
 
-// One warp per 32-row chunk: column-side maxima of the BF16 error-bound terms,
-//   P1 = max ||x||,   P2 = max ||x - x~|| + (gamma_tc + 1.01 u) max ||x~||,
-//   P3 = max |beta err| + u max beta + absolute slack,
-//   and the chunk's smallest beta (for the epilogue's whole-chunk reject test),
-// so that for a query row q and any column x in the chunk the error of the
-// epilogue value h = fl(A~ - beta) is at most  rq * P1 + ||q~|| * P2 + P3.
-// Also fills beta's padding with +inf (padded columns can never match).
-__global__ void __launch_bounds__(256) k1_chunk_stats(const float *__restrict__ beta_in, const float4 *__restrict__ rowb,
-                                                      int64_t n, int64_t n_pad, float g2, float p3_abs,
-                                                      float *__restrict__ beta, float4 *__restrict__ cstat)
+// Significant bits an FP16 copy keeps (FP16 has 11, BF16 8): 9 for 256 < d <= 512. Those joins are
+// bound by the tensor cores under the power cap, where fewer toggling bits mean higher clocks:
+// 131,072^2 unit-norm rows, d = 512, back to back, 11 bits 11.87 ms, 10 bits 11.71, 9 bits 11.52, BF16
+// 11.53, with 0.51, 0.75, 1.24 and 2.29 M undecided pairs. Narrower joins are bound by their epilogue
+// (d = 128: 3.33 ms at any width), wider ones by the recheck's longer rows.
+static int f16_bits(int dp) { return dp > 256 && dp <= 512 ? 9 : 11; }
+
+struct BuildParams {
+    const float *src;          // features at the source's row order
+    const int64_t *src_ids;
+    const int32_t *perm;       // store row i <- source row perm[i] (NULL: row i)
+    int64_t n, n_pad;
+    int d, dp;
+    const unsigned *mm;        // the store's magnitudes (k_sort_keys)
+    float *x32;                // outputs below; x32, ids, orig, nq64 and beta may be NULL together
+    int64_t *ids;
+    int32_t *orig;
+    double *nq64;
+    float *beta;
+    uint16_t *xh;
+    float4 *rowb, *cstat;
+    float g2, p3_abs;
+    int force_bf16;
+    int bits;                  // significant bits of the FP16 codes
+    int vec;                   // features start on 8 bytes and d is even: load pairs
+    int *err;
+};
+
+// Chunk statistics of the error bound (see k1_build) from a chunk's rows, one a lane; a padding row
+// has zero bounds and beta = +inf.
+__device__ __forceinline__ void chunk_stat(float rq, float nqt, float nx, float berr, float bt, float g2, float p3_abs,
+                                           float4 *out)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t chunk = (int64_t)blockIdx.x * 8 + warp;
-    if (chunk * 32 >= n_pad) return;
-    const int64_t row = chunk * 32 + lane;
-    float rq = 0.f, nqt = 0.f, nx = 0.f, berr = 0.f, bt = 0.f;
-    float bmin = __int_as_float(0x7f800000);   // +inf: padding rows do not lower the chunk minimum
-    if (row < n) {
-        const float4 rb = rowb[row];
-        rq = rb.x;
-        nqt = rb.y;
-        nx = rb.z;
-        berr = rb.w;
-        bt = fabsf(beta_in[row]);
-        bmin = beta_in[row];
-    } else {
-        beta[row] = __int_as_float(0x7f800000);   // +inf
-    }
+    float bmin = bt, bmax = bt < __int_as_float(0x7f800000) ? fabsf(bt) : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         rq = fmaxf(rq, __shfl_xor_sync(0xffffffffu, rq, o));
         nqt = fmaxf(nqt, __shfl_xor_sync(0xffffffffu, nqt, o));
         nx = fmaxf(nx, __shfl_xor_sync(0xffffffffu, nx, o));
         berr = fmaxf(berr, __shfl_xor_sync(0xffffffffu, berr, o));
-        bt = fmaxf(bt, __shfl_xor_sync(0xffffffffu, bt, o));
+        bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
         bmin = fminf(bmin, __shfl_xor_sync(0xffffffffu, bmin, o));
     }
-    if (lane == 0) {
+    if ((threadIdx.x & 31) == 0) {
         const float p2 = __fmaf_ru(g2, nqt, rq);
-        const float p3 = __fadd_ru(__fmaf_ru(5.9604644775390625e-08f, bt, berr), p3_abs);
-        cstat[chunk] = make_float4(nx, p2, p3, bmin);
+        const float p3 = __fadd_ru(__fmaf_ru(5.9604644775390625e-08f, bmax, berr), p3_abs);
+        *out = make_float4(nx, p2, p3, bmin);
     }
+}
+
+// One CTA per chunk of 32 store rows, four rows a warp, everything a store derives in one pass over
+// the source: the gathered FP32 row x, its id and caller row, and
+//   nq64  = sum x_k^2 in FP64 (products exact, rounding only in the sum),
+//   the 16-bit copy x~ (FP16 times the store's scale, or BF16; zero padded to dp),
+//   upper bounds of ||x - x~|| and ||x~|| (FP32 sums of squares rounded up at every step,
+//   square roots rounded up), and of ||x|| (from the FP64 sum, inflated by the sum and sqrt
+//   rounding),
+//   beta = RN32(nq64 / 2) and an upper bound of |beta - ||x||^2 / 2|,
+// rows with a non-finite value or |x_k| > 2^40 flagged; then the chunk's column-side maxima of the
+// error-bound terms,
+//   P1 = max ||x||,   P2 = max ||x - x~|| + (gamma_tc + 1.01 u) max ||x~||,
+//   P3 = max |beta err| + u max beta + absolute slack,
+//   and the chunk's smallest beta (for the epilogue's whole-chunk reject test),
+// so that for a query row q and any column x in the chunk the error of the epilogue value
+// h = fl(A~ s - beta) is at most  rq * P1 + ||q~|| * P2 + P3. Padding rows get beta = +inf (they
+// never match).
+//
+// What bounds it: HBM (4 d in, 4 d + 2 dp out a row); a warp keeps four rows' loads in flight. The
+// FP64 tail runs on one warp, a row a lane (a warp-wide FP64 instruction costs the same at one
+// lane). 100,003 x 128 rows: 47 us; the gather, a 32-rows-a-warp norm pass and the chunk pass took
+// 27 + 129 + 4 us, and 54 us where a batch's 9,500 query rows left most of the chip idle.
+__global__ void __launch_bounds__(256) k1_build(const BuildParams p)
+{
+    __shared__ double sm_s1[32];
+    __shared__ float sm_s2[32], sm_s3[32];
+    __shared__ int sm_bad[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t row0 = (int64_t)blockIdx.x * 32 + warp * 4;
+    float scale = 1.0f;
+    const bool f16 = !p.force_bf16 && half_format(p.mm[2], ~p.mm[3], &scale) == kHalfF16;
+    const float inv = 1.0f / scale;   // exact: a power of two
+    const float *xr[4];
+    double s1[4] = {0.0, 0.0, 0.0, 0.0};
+    float s2[4] = {0.f, 0.f, 0.f, 0.f}, s3[4] = {0.f, 0.f, 0.f, 0.f};   // rounded up at every step
+    bool bad[4] = {false, false, false, false};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t row = row0 + r;
+        const int64_t j = row < p.n ? (p.perm ? (int64_t)p.perm[row] : row) : 0;
+        xr[r] = p.src + j * p.d;
+        if (p.ids && row < p.n && lane == 0) {
+            p.ids[row] = p.src_ids[j];
+            p.orig[row] = (int32_t)j;
+        }
+    }
+    for (int k = 2 * lane; k < p.dp; k += 64) {   // two neighbouring features a lane
+        float v[4][2];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) v[r][h] = 0.0f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (row0 + r >= p.n) continue;
+            if (p.vec) {
+                if (k < p.d) *reinterpret_cast<float2 *>(v[r]) = __ldg(reinterpret_cast<const float2 *>(xr[r] + k));
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (k + h < p.d) v[r][h] = __ldg(xr[r] + k + h);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int64_t row = row0 + r;
+            if (row >= p.n) continue;
+            uint16_t c[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float x = v[r][h];
+                if (!(fabsf(x) <= 1099511627776.0f)) bad[r] = true;   // also catches NaN
+                float fx;
+                if (f16) {
+                    // x / s is exact; its magnitude is rounded to p.bits bits (half up), then to FP16's grid
+                    const int sh = 24 - p.bits;
+                    const unsigned u = ((__float_as_uint(x * inv) + (1u << (sh - 1))) >> sh) << sh;
+                    const __half q = __float2half_rn(__uint_as_float(u));
+                    c[h] = __half_as_ushort(q);
+                    fx = __half2float(q) * scale;
+                } else {
+                    const __nv_bfloat16 q = __float2bfloat16_rn(x);
+                    c[h] = __bfloat16_as_ushort(q);
+                    fx = __bfloat162float(q);
+                }
+                const float e = x - fx;   // exact: x~ shares x's leading bits, or is 0
+                s1[r] = __fma_rn((double)x, (double)x, s1[r]);
+                s2[r] = __fmaf_ru(e, e, s2[r]);
+                s3[r] = __fmaf_ru(fx, fx, s3[r]);
+                if (p.x32 && (p.d & 1) && k + h < p.d) p.x32[row * p.d + k + h] = x;
+            }
+            if (p.x32 && !(p.d & 1) && k < p.d)   // store rows of an even length start on 8 bytes
+                *reinterpret_cast<float2 *>(p.x32 + row * p.d + k) = make_float2(v[r][0], v[r][1]);
+            *reinterpret_cast<uint32_t *>(p.xh + row * p.dp + k) = (uint32_t)c[0] | ((uint32_t)c[1] << 16);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s1[r] = __dadd_rn(s1[r], __shfl_xor_sync(0xffffffffu, s1[r], o));
+            s2[r] = __fadd_ru(s2[r], __shfl_xor_sync(0xffffffffu, s2[r], o));
+            s3[r] = __fadd_ru(s3[r], __shfl_xor_sync(0xffffffffu, s3[r], o));
+        }
+        const bool any = __any_sync(0xffffffffu, bad[r]);
+        if (lane == 0) {
+            sm_s1[warp * 4 + r] = s1[r];
+            sm_s2[warp * 4 + r] = s2[r];
+            sm_s3[warp * 4 + r] = s3[r];
+            sm_bad[warp * 4 + r] = any;
+        }
+    }
+    __syncthreads();
+    if (warp) return;
+    const int64_t row = (int64_t)blockIdx.x * 32 + lane;
+    float rq = 0.f, nqt = 0.f, nx = 0.f, berr = 0.f, bt = __int_as_float(0x7f800000);   // a padding row
+    if (row < p.n) {
+        const double q1 = sm_s1[lane];
+        if (sm_bad[lane]) atomicOr(p.err, 1);
+        // Any-order FP64 sum of dp non-negative exact terms: relative error <= (dp-1) 2^-53.
+        const double fac = 1.0 + (double)(p.dp + 4) * 2.220446049250313e-16;
+        const double grow = 1.0 + 8.881784197001252e-16;   // 1 + 2^-50 covers the sqrt / product roundings
+        rq = __fsqrt_ru(sm_s2[lane]);
+        nqt = __fsqrt_ru(sm_s3[lane]);
+        nx = __double2float_ru(sqrt(q1 * fac) * grow);
+        const double h = 0.5 * q1;
+        bt = __double2float_rn(h);
+        berr = __double2float_ru((fabs((double)bt - h) + h * (double)(p.dp + 2) * 2.220446049250313e-16) * grow);
+        if (p.nq64) p.nq64[row] = q1;
+        p.rowb[row] = make_float4(rq, nqt, nx, berr);
+    }
+    if (p.beta) p.beta[row] = bt;
+    chunk_stat(rq, nqt, nx, berr, bt, p.g2, p.p3_abs, p.cstat + blockIdx.x);
+}
+
+// The inner-product join's column term (0, +inf on padding rows) and its chunk statistics, one warp
+// per chunk.
+__global__ void __launch_bounds__(256) k1_ip_stats(const float4 *__restrict__ rowb, int64_t n, int64_t n_pad, float g2,
+                                                   float p3_abs, float *__restrict__ beta_ip, float4 *__restrict__ cstat)
+{
+    const int64_t chunk = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (chunk * 32 >= n_pad) return;
+    const int64_t row = chunk * 32 + (threadIdx.x & 31);
+    const float4 rb = row < n ? rowb[row] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float bt = row < n ? 0.f : __int_as_float(0x7f800000);
+    beta_ip[row] = bt;
+    chunk_stat(rb.x, rb.y, rb.z, rb.w, bt, g2, p3_abs, cstat + chunk);
 }
 
 // ------------------------------------------------------------------ norm ordering
@@ -218,46 +315,62 @@ __global__ void __launch_bounds__(256) k1_chunk_stats(const float *__restrict__ 
 constexpr int kSortBuckets = 65536;
 static size_t align256(size_t x);
 
-__global__ void __launch_bounds__(256) k_sort_keys(const float *__restrict__ x, int64_t n, int d,
-                                                   float *__restrict__ keys, unsigned *__restrict__ minmax)
+// Squared norms of the rows (row i: source row gather[i] when given) and the store's magnitudes, kept
+// by atomicMax on zeroed words: mm[0] = ~(smallest squared norm's bits), mm[1] = the largest's,
+// mm[2] = the largest |x_k|'s bits, mm[3] = ~(the smallest non-zero row's largest |x_k|'s).
+__global__ void __launch_bounds__(256) k_sort_keys(const float *__restrict__ x, const int32_t *__restrict__ gather,
+                                                   int64_t n, int d, float *__restrict__ keys, unsigned *__restrict__ mm)
 {
-    __shared__ unsigned s_min[8], s_max[8];
+    __shared__ unsigned sm[8][4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * 8 + warp;
-    unsigned kmin = 0xffffffffu, kmax = 0u;
-    if (row < n) {
-        const float *xr = x + row * d;
-        float s = 0.f;
-        for (int k = lane; k < d; k += 32) {
-            const float v = __ldg(xr + k);
-            s = fmaf(v, v, s);
-        }
+    const int64_t row0 = ((int64_t)blockIdx.x * 8 + warp) * 4;   // four rows a warp
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, m[4] = {0.f, 0.f, 0.f, 0.f};
+    const float *xr[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (!(s <= 3.0e38f)) s = 3.0e38f;   // non-finite rows are rejected later; keep the key ordered
-        if (lane == 0) keys[row] = s;
-        kmin = kmax = __float_as_uint(s);   // non-negative floats order like their bits
+    for (int r = 0; r < 4; ++r) {
+        const int64_t row = row0 + r;
+        xr[r] = x + (row < n ? (gather ? (int64_t)gather[row] : row) : 0) * d;
     }
-    if (lane == 0) {
-        s_min[warp] = kmin;
-        s_max[warp] = kmax;
+    for (int k = lane; k < d; k += 32) {
+        float v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = row0 + r < n ? __ldg(xr[r] + k) : 0.f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            s[r] = fmaf(v[r], v[r], s[r]);
+            m[r] = fmaxf(m[r], fabsf(v[r]));
+        }
     }
+    unsigned w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+            m[r] = fmaxf(m[r], __shfl_xor_sync(0xffffffffu, m[r], o));
+        }
+        if (!(s[r] <= 3.0e38f)) s[r] = 3.0e38f;   // non-finite rows are rejected later; keep the key ordered
+        if (row0 + r < n) {
+            if (lane == 0) keys[row0 + r] = s[r];
+            const unsigned sb = __float_as_uint(s[r]), mb = __float_as_uint(m[r]);   // non-negative floats order like their bits
+            w[0] = max(w[0], ~sb);
+            w[1] = max(w[1], sb);
+            w[2] = max(w[2], mb);
+            if (mb) w[3] = max(w[3], ~mb);
+        }
+    }
+    if (lane < 4) sm[warp][lane] = lane == 0 ? w[0] : lane == 1 ? w[1] : lane == 2 ? w[2] : w[3];
     __syncthreads();
-    if (threadIdx.x == 0) {   // one atomic pair per block of eight rows
-        for (int w = 1; w < 8; ++w) {
-            kmin = min(kmin, s_min[w]);
-            kmax = max(kmax, s_max[w]);
-        }
-        if (kmin != 0xffffffffu) {
-            atomicMin(minmax + 0, kmin);
-            atomicMax(minmax + 1, kmax);
-        }
+    if (threadIdx.x < 4) {   // one atomic of each kind per block of 32 rows
+        unsigned v = 0u;
+        for (int i = 0; i < 8; ++i) v = max(v, sm[i][threadIdx.x]);
+        if (v) atomicMax(mm + threadIdx.x, v);
     }
 }
 
-__device__ __forceinline__ int sort_bucket(float k, const unsigned *minmax)
+__device__ __forceinline__ int sort_bucket(float k, const unsigned *mm)
 {
-    const float lo = __uint_as_float(minmax[0]), hi = __uint_as_float(minmax[1]);
+    const float lo = __uint_as_float(~mm[0]), hi = __uint_as_float(mm[1]);
     if (!(hi > lo)) return 0;
     const float f = (k - lo) / (hi - lo) * (float)kSortBuckets;
     int b = (int)f;
@@ -271,27 +384,37 @@ __global__ void __launch_bounds__(256) k_sort_hist(const float *__restrict__ key
     if (i < n) atomicAdd(hist + sort_bucket(keys[i], minmax), 1u);
 }
 
-// Exclusive prefix sum of the 65,536 bucket counts, one block of 1024 threads.
+// Exclusive prefix sum of the 65,536 bucket counts, one block of 1024 threads, 64 counts each, read
+// 16 bytes at a time with every load of a pass in flight (70 us when a loop of single loads did it).
 __global__ void __launch_bounds__(1024) k_sort_scan(unsigned *__restrict__ hist)
 {
-    __shared__ unsigned part[1024];
-    constexpr int kPer = kSortBuckets / 1024;
-    const int t = threadIdx.x;
+    __shared__ unsigned part[32];
+    constexpr int kQuads = kSortBuckets / 1024 / 4;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    uint4 *h4 = reinterpret_cast<uint4 *>(hist) + t * kQuads;
     unsigned loc = 0;
-    for (int i = 0; i < kPer; ++i) loc += hist[t * kPer + i];
-    part[t] = loc;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const unsigned v = (t >= off) ? part[t - off] : 0u;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kQuads; ++i) {
+        const uint4 v = h4[i];
+        loc += v.x + v.y + v.z + v.w;
     }
-    unsigned run = part[t] - loc;
-    for (int i = 0; i < kPer; ++i) {
-        const unsigned c = hist[t * kPer + i];
-        hist[t * kPer + i] = run;
-        run += c;
+    unsigned run = loc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o) run += y;
+    }
+    if (lane == 31) part[w] = run;
+    __syncthreads();
+    unsigned before = lane < w ? part[lane] : 0u;
+    before = __reduce_add_sync(0xffffffffu, before);
+    run += before - loc;
+#pragma unroll
+    for (int i = 0; i < kQuads; ++i) {
+        const uint4 c = h4[i];
+        const uint4 o = make_uint4(run, run + c.x, run + c.x + c.y, run + c.x + c.y + c.z);
+        run = o.w + c.w;
+        h4[i] = o;
     }
 }
 
@@ -301,25 +424,6 @@ __global__ void __launch_bounds__(256) k_sort_scatter(const float *__restrict__ 
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) perm[atomicAdd(offs + sort_bucket(keys[i], minmax), 1u)] = (int32_t)i;
-}
-
-// Store row i <- caller row perm[i] (features and id), one warp per row.
-__global__ void __launch_bounds__(256) k_gather_rows(const float *__restrict__ src, const int64_t *__restrict__ src_ids,
-                                                     const int32_t *__restrict__ perm, int64_t n, int d,
-                                                     float *__restrict__ dst, int64_t *__restrict__ dst_ids,
-                                                     int32_t *__restrict__ orig)
-{
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * 8 + warp;
-    if (row >= n) return;
-    const int32_t j = perm[row];
-    const float *sr = src + (int64_t)j * d;
-    float *dr = dst + row * d;
-    for (int k = lane; k < d; k += 32) dr[k] = __ldg(sr + k);
-    if (lane == 0) {
-        dst_ids[row] = src_ids[j];
-        orig[row] = j;
-    }
 }
 
 // ------------------------------------------------------------------ FP8 copy
@@ -455,7 +559,7 @@ int ensure_fp8(Store *s, cudaStream_t st)
         count_launch();
     }
     const float g2 = f32_ru(gamma_tc8(dp8) + 1.01 * kU32);
-    k1_fp8_stats<<<chunk_blocks, 256, 0, st>>>(rowb8, s->cstat, s->n, s->n_pad, g2, cstat8);
+    k1_fp8_stats<<<chunk_blocks, 256, 0, st>>>(rowb8, s->h.cstat, s->n, s->n_pad, g2, cstat8);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -473,29 +577,86 @@ int ensure_fp8(Store *s, cudaStream_t st)
     return DL_OK;
 }
 
-// The inner-product join's column term is 0: h = q.x. Its chunk stats come from the same
-// kernel as the squared-L2 ones, run on a zero column term, so P1 and P2 (the encoding and
-// accumulation terms of the BF16 bound) are the store's own and P3 keeps the L2 beta error
-// (a conservative extra); padding rows get +inf, so they never match.
+// BF16 copy of a store whose 16-bit copy is FP16 (for joins that ask for BF16, and with stores that
+// hold BF16), built once, on first use.
+static int ensure_bf16(Store *s, cudaStream_t st)
+{
+    std::lock_guard<std::mutex> lk(s->mu);
+    if (s->h.fmt == kHalfBF16 || s->alt_block) return DL_OK;
+    const size_t b_x = align256(sizeof(uint16_t) * s->n * s->dp), b_rb = align256(sizeof(float4) * s->n),
+                 b_cs = align256(sizeof(float4) * (s->n_pad / 32));
+    void *blk = nullptr;
+    int rc = dev_alloc(&blk, b_x + b_rb + b_cs + 256, st);
+    if (rc) return rc;
+    char *q = (char *)blk;
+    BuildParams p{};
+    p.src = s->x32;
+    p.n = s->n;
+    p.n_pad = s->n_pad;
+    p.d = s->d;
+    p.dp = s->dp;
+    p.xh = (uint16_t *)q;
+    p.rowb = (float4 *)(q + b_x);
+    p.cstat = (float4 *)(q + b_x + b_rb);
+    p.err = (int *)(q + b_x + b_rb + b_cs);   // the features were checked when the store was made
+    p.g2 = f32_ru(gamma_tc(s->dp) + 1.01 * kU32);
+    p.p3_abs = f32_ru(abs_slack_tc(s->dp));
+    p.force_bf16 = 1;
+    p.bits = f16_bits(s->dp);
+    p.vec = (s->d & 1) == 0;
+    k1_build<<<(unsigned)(s->n_pad / 32), 256, 0, st>>>(p);
+    count_launch();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        dev_free(blk, st);
+        return cuda_fail(e, "BF16 store copy");
+    }
+    s->alt.fmt = kHalfBF16;
+    s->alt.x = p.xh;
+    s->alt.rowb = p.rowb;
+    s->alt.cstat = p.cstat;
+    s->alt_block = blk;
+    return DL_OK;
+}
+
+int get_half(Store *s, int fmt, cudaStream_t st, Half **out)
+{
+    *out = nullptr;
+    if (s->h.fmt == fmt) {
+        *out = &s->h;
+        return DL_OK;
+    }
+    if (fmt != kHalfBF16) {
+        set_error("the store's features span too wide a range for an FP16 copy");
+        return DL_EUNSUPPORTED;
+    }
+    const int rc = ensure_bf16(s, st);
+    if (!rc) *out = &s->alt;
+    return rc;
+}
+
+// The inner-product join's column term is 0: h = q.x. Its chunk stats are those of the BF16 copy, so
+// P1 and P2 (the encoding and accumulation terms of the bound) are the store's own and P3 keeps the
+// L2 beta error (a conservative extra); padding rows get +inf, so they never match.
 int ensure_ip(Store *s, cudaStream_t st)
 {
+    Half *h = nullptr;
+    int rc = get_half(s, kHalfBF16, st, &h);
+    if (rc) return rc;
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->ip_block) return DL_OK;
     const size_t b_b = align256(sizeof(float) * s->n_pad), b_cs = align256(sizeof(float4) * (s->n_pad / 32));
     void *blk = nullptr;
-    int rc = dev_alloc(&blk, b_b + b_cs, st);
+    rc = dev_alloc(&blk, b_b + b_cs, st);
     if (rc) return rc;
     float *beta_ip = (float *)blk;
     float4 *cstat_ip = (float4 *)((char *)blk + b_b);
-    cudaError_t e = cudaMemsetAsync(beta_ip, 0, sizeof(float) * s->n_pad, st);
-    if (e == cudaSuccess) {
-        const float g2 = f32_ru(gamma_tc(s->dp) + 1.01 * kU32);
-        const float p3a = f32_ru(abs_slack_tc(s->dp));
-        k1_chunk_stats<<<(unsigned)((s->n_pad / 32 + 7) / 8), 256, 0, st>>>(beta_ip, s->rowb, s->n, s->n_pad, g2, p3a,
-                                                                            beta_ip, cstat_ip);
-        count_launch();
-        e = cudaGetLastError();
-    }
+    k1_ip_stats<<<(unsigned)((s->n_pad / 32 + 7) / 8), 256, 0, st>>>(h->rowb, s->n, s->n_pad,
+                                                                     f32_ru(gamma_tc(s->dp) + 1.01 * kU32),
+                                                                     f32_ru(abs_slack_tc(s->dp)), beta_ip, cstat_ip);
+    count_launch();
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         dev_free(blk, st);
@@ -523,31 +684,31 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-int get_tmap(Store *s, int box_rows, const CUtensorMap **out)
+int get_tmap(Store *s, Half *h, int box_rows, const CUtensorMap **out)
 {
     std::lock_guard<std::mutex> lk(s->mu);
-    for (auto &t : s->tmaps)
+    for (auto &t : h->tmaps)
         if (t.valid && t.box_rows == box_rows) {
             *out = &t.map;
             return DL_OK;
         }
     TmapCache *slot = nullptr;
-    for (auto &t : s->tmaps)
+    for (auto &t : h->tmaps)
         if (!t.valid) {
             slot = &t;
             break;
         }
-    if (!slot) slot = &s->tmaps[0];
+    if (!slot) slot = &h->tmaps[0];
     auto fn = encode_fn();
     if (!fn) {
         set_error("cuTensorMapEncodeTiled is not available from the driver");
         return DL_ECUDA;
     }
     cuuint64_t gdim[2] = {(cuuint64_t)s->dp, (cuuint64_t)(s->n > 0 ? s->n : 1)};
-    cuuint64_t gstride[1] = {(cuuint64_t)s->dp * sizeof(__nv_bfloat16)};
+    cuuint64_t gstride[1] = {(cuuint64_t)s->dp * sizeof(uint16_t)};
     cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t estride[2] = {1, 1};
-    CUresult r = fn(&slot->map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)s->xb, gdim, gstride, box, estride,
+    CUresult r = fn(&slot->map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, (void *)h->x, gdim, gstride, box, estride,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
@@ -641,11 +802,11 @@ int store_create_impl(dl_store **out, const int64_t *ids, const float *feats, in
     DL_CUDA_TRY(cudaGetDevice(&s->device));
 
     const size_t b_ids = align256(sizeof(int64_t) * n), b_orig = align256(sizeof(int32_t) * n),
-                 b_x32 = align256(sizeof(float) * n * d), b_xb = align256(sizeof(__nv_bfloat16) * n * s->dp),
+                 b_x32 = align256(sizeof(float) * n * d), b_xh = align256(sizeof(uint16_t) * n * s->dp),
                  b_nq = align256(sizeof(double) * n), b_beta = align256(sizeof(float) * s->n_pad),
                  b_rowb = align256(sizeof(float4) * n), b_cst = align256(sizeof(float4) * (s->n_pad / 32)),
                  b_err = 256;
-    const size_t total = b_ids + b_orig + b_x32 + b_xb + b_nq + b_beta + b_rowb + b_cst + b_err;
+    const size_t total = b_ids + b_orig + b_x32 + b_xh + b_nq + b_beta + b_rowb + b_cst + b_err;
     void *base = nullptr;
     int rc = dev_alloc(&base, total, st);
     if (rc != DL_OK) {
@@ -659,15 +820,15 @@ int store_create_impl(dl_store **out, const int64_t *ids, const float *feats, in
     p += b_orig;
     s->x32 = (float *)p;
     p += b_x32;
-    s->xb = (__nv_bfloat16 *)p;
-    p += b_xb;
+    s->h.x = (uint16_t *)p;
+    p += b_xh;
     s->nq64 = (double *)p;
     p += b_nq;
     s->beta = (float *)p;
     p += b_beta;
-    s->rowb = (float4 *)p;
+    s->h.rowb = (float4 *)p;
     p += b_rowb;
-    s->cstat = (float4 *)p;
+    s->h.cstat = (float4 *)p;
     p += b_cst;
     int *d_err = (int *)p;
 
@@ -675,10 +836,10 @@ int store_create_impl(dl_store **out, const int64_t *ids, const float *feats, in
     const bool host = (where == DL_MEM_HOST);
     const size_t t_x = host ? align256(sizeof(float) * n * d) : 0, t_ids = host ? align256(sizeof(int64_t) * n) : 0,
                  t_keys = align256(sizeof(float) * n), t_perm = align256(sizeof(int32_t) * n),
-                 t_hist = sizeof(unsigned) * kSortBuckets, t_mm = 256;
+                 t_hist = sizeof(unsigned) * kSortBuckets;
     void *tmp = nullptr;
     if (n > 0) {
-        rc = dev_alloc(&tmp, t_x + t_ids + t_keys + t_perm + t_hist + t_mm, st);
+        rc = dev_alloc(&tmp, t_x + t_ids + t_keys + t_perm + t_hist, st);
         if (rc != DL_OK) {
             dev_free(base, st);
             delete s;
@@ -692,69 +853,73 @@ int store_create_impl(dl_store **out, const int64_t *ids, const float *feats, in
         delete s;
         return code;
     };
-    cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
+    cudaError_t e = cudaMemsetAsync(d_err, 0, b_err, st);
     if (e != cudaSuccess) return fail(cuda_fail(e, "dl_store_create memset"));
+    unsigned *mm = (unsigned *)d_err + 4;   // the store's magnitudes, beside the error word
+    BuildParams bp{};
+    bp.src = feats;
+    bp.src_ids = ids;
+    bp.perm = gather;
     if (n > 0) {
         char *q = (char *)tmp;
-        const float *src_x = feats;
-        const int64_t *src_ids = ids;
         if (host) {
             float *hx = (float *)q;
             int64_t *hid = (int64_t *)(q + t_x);
             e = cudaMemcpyAsync(hx, feats, sizeof(float) * n * d, cudaMemcpyHostToDevice, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(hid, ids, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st);
             if (e != cudaSuccess) return fail(cuda_fail(e, "dl_store_create upload"));
-            src_x = hx;
-            src_ids = hid;
+            bp.src = hx;
+            bp.src_ids = hid;
         }
         q += t_x + t_ids;
         float *keys = (float *)q;
         int32_t *perm = (int32_t *)(q + t_keys);
         unsigned *hist = (unsigned *)(q + t_keys + t_perm);
-        unsigned *mm = (unsigned *)(q + t_keys + t_perm + t_hist);
-        e = cudaMemsetAsync(hist, 0, t_hist, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(mm, 0xff, 4, st);      // min <- 0xffffffff
-        if (e == cudaSuccess) e = cudaMemsetAsync(mm + 1, 0, 4, st);     // max <- 0
-        if (e != cudaSuccess) return fail(cuda_fail(e, "dl_store_create memset"));
-        const unsigned gw = (unsigned)((n + 7) / 8), gt = (unsigned)((n + 255) / 256);
-        k_sort_keys<<<gw, 256, 0, st>>>(src_x, n, d, keys, mm);
+        const unsigned gt = (unsigned)((n + 255) / 256);
+        k_sort_keys<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(bp.src, gather, n, d, keys, mm);
+        count_launch();
         if (!gather) {
+            e = cudaMemsetAsync(hist, 0, t_hist, st);
+            if (e != cudaSuccess) return fail(cuda_fail(e, "dl_store_create memset"));
             k_sort_hist<<<gt, 256, 0, st>>>(keys, n, mm, hist);
             k_sort_scan<<<1, 1024, 0, st>>>(hist);
             k_sort_scatter<<<gt, 256, 0, st>>>(keys, n, mm, hist, perm);
             count_launch(3);
+            bp.perm = perm;
         }
-        k_gather_rows<<<gw, 256, 0, st>>>(src_x, src_ids, gather ? gather : perm, n, d, s->x32, s->ids, s->orig);
-        k1_norm_quant<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s->x32, n, d, s->dp, s->xb, s->nq64, s->beta,
-                                                                  s->rowb, d_err);   // 32 rows per warp
-        count_launch(3);
     }
-    const float g2 = f32_ru(gamma_tc(s->dp) + 1.01 * kU32);
-    const float p3a = f32_ru(abs_slack_tc(s->dp));
-    k1_chunk_stats<<<(unsigned)((s->n_pad / 32 + 7) / 8), 256, 0, st>>>(s->beta, s->rowb, n, s->n_pad, g2, p3a, s->beta,
-                                                                        s->cstat);
+    bp.n = n;
+    bp.n_pad = s->n_pad;
+    bp.d = d;
+    bp.dp = s->dp;
+    bp.mm = mm;
+    bp.x32 = s->x32;
+    bp.ids = s->ids;
+    bp.orig = s->orig;
+    bp.nq64 = s->nq64;
+    bp.beta = s->beta;
+    bp.xh = s->h.x;
+    bp.rowb = s->h.rowb;
+    bp.cstat = s->h.cstat;
+    bp.g2 = f32_ru(gamma_tc(s->dp) + 1.01 * kU32);
+    bp.p3_abs = f32_ru(abs_slack_tc(s->dp));
+    bp.vec = (d & 1) == 0 && (reinterpret_cast<uintptr_t>(bp.src) & 7) == 0;
+    bp.bits = f16_bits(s->dp);
+    bp.err = d_err;
+    k1_build<<<(unsigned)(s->n_pad / 32), 256, 0, st>>>(bp);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(cuda_fail(e, "store kernels launch"));
-    int h_err = 0;
-    unsigned h_mm[2] = {0u, 0u};
-    if (n > 0) {
-        const unsigned *mm = (const unsigned *)((char *)tmp + t_x + t_ids + t_keys + t_perm + t_hist);
-        e = cudaMemcpyAsync(h_mm, mm, sizeof h_mm, cudaMemcpyDeviceToHost, st);
-        if (e != cudaSuccess) return fail(cuda_fail(e, "dl_store_create readback"));
-    }
-    e = cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    unsigned h_back[8] = {0u};   // the error word, then (from word 4) the magnitudes
+    e = cudaMemcpyAsync(h_back, d_err, sizeof h_back, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(cuda_fail(e, "dl_store_create sync"));
-    if (h_err) {
+    if (h_back[0]) {
         set_error("dl_store_create: a feature is non-finite or exceeds 2^40 in magnitude");
         return fail(DL_EINVAL);
     }
-    {
-        float mx;
-        std::memcpy(&mx, &h_mm[1], sizeof mx);
-        s->nq_max = mx;
-    }
+    std::memcpy(&s->nq_max, &h_back[5], sizeof s->nq_max);
+    s->h.fmt = half_format(h_back[6], ~h_back[7], &s->h.scale);
     dev_free(tmp, st);
     *out = s;
     return DL_OK;
@@ -915,6 +1080,7 @@ int dl_store_destroy(dl_store *s)
     if (prev != s->device) cudaSetDevice(s->device);
     dev_free(s->ids, 0);   // ids is the base of the store's single allocation
     if (s->fp8_block) dev_free(s->fp8_block, 0);
+    if (s->alt_block) dev_free(s->alt_block, 0);
     if (s->ip_block) dev_free(s->ip_block, 0);
     if (s->clabel) dev_free(s->clabel, 0);
     for (auto &b : s->balls)

@@ -477,6 +477,13 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         return DL_EINVAL;
     }
     const bool use_tc = (o.precision != DL_PREC_FP32) && Q->dp <= 512;
+    // the 16-bit copies' format: FP16 where both stores hold it, unless BF16 was asked for
+    const bool f16 = Q->h.fmt == kHalfF16 && S->h.fmt == kHalfF16;
+    if (o.precision == DL_PREC_FP16 && !(f16 && use_tc)) {
+        set_error("top-k: FP16 needs features within FP16's range in both stores and d <= 512");
+        return DL_EUNSUPPORTED;
+    }
+    const int fmt = f16 && o.precision != DL_PREC_BF16 ? kHalfF16 : kHalfBF16;
     bool tune_trial = false;
     if ((o.epilogue_warps != 0 && o.epilogue_warps != 8 && o.epilogue_warps != 16) ||
         (o.epilogue_warps == 16 && o.tile_n == 128)) {
@@ -569,13 +576,18 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     f.n_fp64 = misc + 1;
     if (nQ > 0 && nS > 0) {
         if (use_tc) {
-            k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, Q->rowb, nQ, rows, g64,
-                                                                          (double)S->nq_max * 1.0001, rowpar, row_theta);
-            count_launch();
-            ++launches;
+            Half *hQ = nullptr, *hS = nullptr;
+            rc = get_half(const_cast<dl_store *>(Q), fmt, st, &hQ);
+            if (!rc) rc = get_half(const_cast<dl_store *>(S), fmt, st, &hS);
+            if (!rc) {
+                k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, hQ->rowb, nQ, rows, g64,
+                                                                              (double)S->nq_max * 1.0001, rowpar, row_theta);
+                count_launch();
+                ++launches;
+            }
             const CUtensorMap *tmA = nullptr, *tmB = nullptr;
-            rc = get_tmap(const_cast<dl_store *>(Q), 128, &tmA);
-            if (!rc) rc = get_tmap(const_cast<dl_store *>(S), BN, &tmB);
+            if (!rc) rc = get_tmap(const_cast<dl_store *>(Q), hQ, 128, &tmA);
+            if (!rc) rc = get_tmap(const_cast<dl_store *>(S), hS, BN, &tmB);
             const int4 *units = nullptr;
             int n_units = 0;
             if (!rc) rc = topk_units(nQ, nS, BN, splits, &units, &n_units);
@@ -591,12 +603,14 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                 L.p.nR = (int)nQ;
                 L.p.nS = (int)nS;
                 L.p.kc = Q->dp / 64;
+                L.p.fmt = fmt == kHalfBF16;
+                L.p.scale = hQ->scale * hS->scale;
                 tc_plan(BN, Q->dp / 64, &L.p.stages, &L.p.a_slots, false, false, wide);
                 L.wide = wide;
                 L.p.upper = 0;
                 L.p.rowpar = rowpar;
                 L.p.beta = S->beta;
-                L.p.cstat = S->cstat;
+                L.p.cstat = hS->cstat;
                 L.p.err = (int *)(misc + 3);
                 L.p.tk_k = k;
                 L.p.tk_cap = cap;
@@ -639,7 +653,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
             if (e != cudaSuccess) rc = cuda_fail(e, "top-k memset");
         }
     } else if (nQ > 0) {   // empty store: every slot is unused
-        k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, Q->rowb, nQ, rows, g64, 0.0, rowpar,
+        k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, Q->h.rowb, nQ, rows, g64, 0.0, rowpar,
                                                                       row_theta);
         k_topk_finalize<<<1, 128, 0, st>>>(f);   // no candidates for any row -> fills -1
         count_launch();
@@ -722,7 +736,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         s.pairs_out = 0;
         s.band_pairs = flagged;   // rows re-solved by the exact scan
         s.fp64_pairs = (int64_t)h2[1];
-        s.precision = use_tc ? DL_PREC_BF16 : DL_PREC_FP32;
+        s.precision = !use_tc ? DL_PREC_FP32 : fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
         s.tile_n = use_tc ? BN : 0;
         s.epilogue_warps = use_tc ? (wide ? 16 : 8) : 0;
         s.kernels_launched = launches;
@@ -787,12 +801,13 @@ extern "C" int dl_topk_join(const dl_store *Q, const dl_store *S, int32_t metric
         o = *opts;
     else
         dl_join_opts_default(&o);
-    if (o.precision != DL_PREC_AUTO && o.precision != DL_PREC_BF16 && o.precision != DL_PREC_FP32) {
+    if (o.precision != DL_PREC_AUTO && o.precision != DL_PREC_BF16 && o.precision != DL_PREC_FP16 &&
+        o.precision != DL_PREC_FP32) {
         set_error("dl_topk_join: precision %d not available for top-k", o.precision);
         return DL_EUNSUPPORTED;
     }
     cudaStream_t st = (cudaStream_t)o.cuda_stream;
-    if (hist && o.precision == DL_PREC_BF16) {
+    if (hist && (o.precision == DL_PREC_BF16 || o.precision == DL_PREC_FP16)) {
         set_error("dl_topk_join: the L1 and chi-square distances run in DL_PREC_FP32 (not on tensor cores)");
         return DL_EUNSUPPORTED;
     }

@@ -47,6 +47,9 @@ std::vector<int> candidates(int kind)
     case kTuneEpsRxS8:
     case kTuneEpsSelf8:
         return {256, 256 | kTuneWide, 256 | kTunePair};
+    case kTuneEpsRxS16:   // FP16: an SM pair has lost to one SM on every shape measured
+    case kTuneEpsSelf16:
+        return {256, 256 | kTuneWide, 128};
     case kTuneBatch:
         return {256, 256 | kTuneWide};
     default:   // top-k: single-SM tiles

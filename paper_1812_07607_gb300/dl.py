@@ -27,7 +27,8 @@ METRICS = {"l2": DL_METRIC_L2, "cosine": DL_METRIC_COSINE, "l1": DL_METRIC_L1, "
 DL_DEDUP_ALL, DL_DEDUP_FILTER_MATCH, DL_DEDUP_MATCH_FILTER = 0, 1, 2
 DEDUP_PLANS = {"all": DL_DEDUP_ALL, "filter_match": DL_DEDUP_FILTER_MATCH, "match_filter": DL_DEDUP_MATCH_FILTER}
 DL_PREC_AUTO, DL_PREC_BF16, DL_PREC_FP8E4M3, DL_PREC_FP32, DL_PREC_FP32_PLAIN = range(5)
-PRECISIONS = {"auto": 0, "bf16": 1, "fp8": 2, "fp32": 3, "fp32_plain": 4}
+DL_PREC_FP16 = 5
+PRECISIONS = {"auto": 0, "bf16": 1, "fp8": 2, "fp32": 3, "fp32_plain": 4, "fp16": 5}
 DL_MEM_HOST, DL_MEM_DEVICE = 0, 1
 DL_SELF_UPPER, DL_SELF_FULL = 0, 1
 
