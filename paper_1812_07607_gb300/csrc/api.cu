@@ -24,7 +24,7 @@ namespace dl {
 // ------------------------------------------------------------------ pinned host memory
 static thread_local unsigned long long *t_counters = nullptr;
 
-static int pinned_counters(unsigned long long **p)
+int pinned_counters(unsigned long long **p)
 {
     if (!t_counters) {
         cudaError_t e = cudaHostAlloc((void **)&t_counters, 64, cudaHostAllocDefault);

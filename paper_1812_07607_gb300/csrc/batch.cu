@@ -142,19 +142,6 @@ __global__ void __launch_bounds__(256)
 
 static size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Units of the epsilon pass: every row tile against every S tile (no self pairs), in
-// S-range-major order so that the CTAs running together share S tiles through L2.
-static int batch_units(int64_t nR, int64_t nS, int BN, int sms, std::vector<int4> *v)
-{
-    const int mt = (int)((nR + 127) / 128), nt = (int)((nS + BN - 1) / BN);
-    int L = 64;
-    while (L > 1 && (int64_t)mt * ((nt + L - 1) / L) < 4LL * sms) L >>= 1;
-    v->clear();
-    for (int nb = 0; nb < nt; nb += L)
-        for (int m = 0; m < mt; ++m) v->push_back(make_int4(m, nb, std::min(nb + L, nt), 0));
-    return DL_OK;
-}
-
 }  // namespace dl
 
 using namespace dl;
@@ -394,8 +381,6 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
         cudaEvent_t tev[2] = {nullptr, nullptr};
         if (tune_trial)
             for (auto &ev : tev) cudaEventCreate(&ev);
-        std::vector<int4> units;
-        batch_units(ne, S->n, BN, sms, &units);
         int64_t cap;
         {
             std::lock_guard<std::mutex> lk(const_cast<dl_store *>(S)->mu);
@@ -405,15 +390,13 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
         }
         for (int attempt = 0;; ++attempt) {
             void *ws = nullptr;
-            const size_t b_units = al(units.size() * sizeof(int4)), b_rowpar = al(mt * 128 * sizeof(float4)),
+            const size_t b_rowpar = al(mt * 128 * sizeof(float4)),
                          b_cand = al(cap * sizeof(uint2)), b_rc = al((size_t)n_req * 8) * 3;
-            rc = dev_alloc(&ws, 256 + b_units + b_rowpar + b_cand + b_rc, st);
+            rc = dev_alloc(&ws, 256 + b_rowpar + b_cand + b_rc, st);
             if (rc) break;
             char *pw = (char *)ws;
             unsigned long long *cnt = (unsigned long long *)pw;   // [0] cand [1] fp64 [2] band [3] err
             pw += 256;
-            int4 *d_units = (int4 *)pw;
-            pw += b_units;
             float4 *rowpar = (float4 *)pw;
             pw += b_rowpar;
             uint2 *cand = (uint2 *)pw;
@@ -424,8 +407,6 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
             cudaError_t e = cudaMemsetAsync(ws, 0, 256, st);
             if (e == cudaSuccess) e = cudaMemsetAsync(req_cnt, 0, (size_t)n_req * 8, st);
             if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, (size_t)n_req * 8, st);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(d_units, units.data(), units.size() * sizeof(int4), cudaMemcpyHostToDevice, st);
             if (e != cudaSuccess) {
                 rc = cuda_fail(e, "dl_batch_join eps setup");
                 dev_free(ws, st);
@@ -441,9 +422,7 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
                 L.tmA = tmA;
                 L.tmB = tmB;
                 L.BN = BN;
-                L.grid = std::min((int)units.size(), sms);
-                L.p.units = d_units;
-                L.p.n_units = (int)units.size();
+                tc_grid_units(&L, mt, (S->n + BN - 1) / BN, sms);
                 L.p.nR = (int)ne;
                 L.p.nS = (int)S->n;
                 L.p.kc = Qe->dp / 64;

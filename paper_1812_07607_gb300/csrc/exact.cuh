@@ -7,6 +7,14 @@
 
 namespace dl {
 
+// Bit number of the (n+1)-th set bit of v, n in [0, 3]; 32 or more when there are fewer. (A dozen
+// instructions; __fns walks the word.)
+__device__ __forceinline__ unsigned nth_set(unsigned v, int n)
+{
+    const unsigned v1 = v & (v - 1u), v2 = v1 & (v1 - 1u), v3 = v2 & (v2 - 1u);
+    return (unsigned)__ffs((int)(n < 2 ? (n ? v1 : v) : (n == 2 ? v2 : v3))) - 1u;
+}
+
 // FP32 thresholds for a squared threshold e2 at dimension d: accept if the FP32
 // distance sum D32 <= t_acc, reject if D32 > t_rej, else evaluate the canonical
 // FP64 sum. Sound for |D32 - D| <= (d+8) 2^-24 D + (d+8) 2^-148 and for the
@@ -69,6 +77,17 @@ __device__ __forceinline__ void ff_merge(FFSum &a, float bs, float bc, float bm)
     a.s = s;
     a.c = __fadd_rn(__fadd_rn(a.c, bc), e);
     a.m = __fadd_rn(a.m, bm);
+}
+
+// (double)f without the FP64 pipe, which conversions take as well (a warp's instruction occupies it
+// for 16 cycles or more of an SM): the exponent and fraction fields moved over, subnormals scaled up
+// first and their exponent corrected.
+__device__ __forceinline__ double widen(float f)
+{
+    const bool sub = (__float_as_uint(f) & 0x7f800000u) == 0u;   // subnormal or zero
+    const unsigned u = __float_as_uint(sub ? f * 16777216.0f : f), m = u & 0x7fffffffu;
+    const unsigned hi = m ? (m >> 3) + (sub ? 0x38000000u - (24u << 20) : 0x38000000u) : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
 // Float-float value S of sum_k (q_k - x_k)^2 by the whole warp (lane l takes k = l, l+32, ...;
@@ -175,6 +194,69 @@ __device__ __forceinline__ bool warp_exact_decide(const float *__restrict__ q, c
     return sum <= e2;
 }
 
+// FP32 squared distances of the pairs (q, x) of the lanes in bm, each returned in its own lane. Four
+// pairs are summed at a time, one per 8-lane group, over 16-byte slices with four of each row in
+// flight per lane (single features when d is no multiple of 4), then a shuffle tree within the group.
+__device__ __forceinline__ float warp_pairs_sq32(unsigned bm, const float *q, const float *x, int d)
+{
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const int grp = (int)(lane >> 3), gl = (int)(lane & 7);
+    float mine = 0.f;
+    unsigned rem = bm;
+    while (rem) {
+        const unsigned pos = nth_set(rem, grp);   // this group's entry: the (grp+1)-th pending lane
+        const bool have = pos < 32u;
+        const int k = have ? (int)pos : 0;
+        const float *qk = reinterpret_cast<const float *>(
+            __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(q), k));
+        const float *xk = reinterpret_cast<const float *>(
+            __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(x), k));
+        float s = 0.f;
+        if (have) {
+            if ((d & 3) == 0) {
+                const float4 *q4 = reinterpret_cast<const float4 *>(qk);
+                const float4 *x4 = reinterpret_cast<const float4 *>(xk);
+                const int n4 = d >> 2;
+                for (int i0 = gl; i0 < n4; i0 += 32) {
+                    float4 a[4], b[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = i0 + 8 * u;
+                        a[u] = i < n4 ? __ldg(q4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        b[u] = i < n4 ? __ldg(x4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        float t = a[u].x - b[u].x;
+                        s = fmaf(t, t, s);
+                        t = a[u].y - b[u].y;
+                        s = fmaf(t, t, s);
+                        t = a[u].z - b[u].z;
+                        s = fmaf(t, t, s);
+                        t = a[u].w - b[u].w;
+                        s = fmaf(t, t, s);
+                    }
+                }
+            } else {
+                for (int i = gl; i < d; i += 8) {
+                    const float t = __ldg(qk + i) - __ldg(xk + i);
+                    s = fmaf(t, t, s);
+                }
+            }
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        const int r = __popc(rem & below);   // this lane's rank among the pending ones
+        const float got = __shfl_sync(0xffffffffu, s, (r & 3) * 8);
+        if (((rem >> lane) & 1u) && r < 4) mine = got;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) rem &= rem - 1u;   // the four settled entries leave the set
+    }
+    return mine;
+}
+
 // Exact decisions for the band entries among a warp's 32 candidate entries. Each lane in
 // bm holds a band pair (q, x) with its own squared threshold e2 and FP32 thresholds. Four
 // pairs are settled at a time, one per 8-lane group: the group sums the pair's FP32
@@ -193,7 +275,7 @@ __device__ __forceinline__ bool warp_band_decide(unsigned bm, const float *q, co
     bool mine = false, und = false;
     unsigned rem = bm;
     while (rem) {
-        const unsigned pos = __fns(rem, 0, grp + 1);   // this group's entry: the (grp+1)-th pending lane
+        const unsigned pos = nth_set(rem, grp);   // this group's entry: the (grp+1)-th pending lane
         const bool have = pos < 32u;
         const int k = have ? (int)pos : 0;
         const float *qk = reinterpret_cast<const float *>(
@@ -310,7 +392,7 @@ __device__ __forceinline__ bool warp_band_decide_ip(unsigned bm, const float *q,
     bool mine = false, und = false;
     unsigned rem = bm;
     while (rem) {
-        const unsigned pos = __fns(rem, 0, grp + 1);
+        const unsigned pos = nth_set(rem, grp);
         const bool have = pos < 32u;
         const int k = have ? (int)pos : 0;
         const float *qk = reinterpret_cast<const float *>(

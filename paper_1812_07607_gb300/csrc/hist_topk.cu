@@ -20,6 +20,8 @@
 //                      written.
 #include <algorithm>
 
+#include "cta.cuh"
+#include "exact.cuh"
 #include "kernels.h"
 #include "simt_tile.cuh"
 
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(256) k_hist_dist_few(const HistTk f)
 template <int M>
 __device__ __forceinline__ double canon_term(float q, float x)
 {
-    const double a = (double)q, b = (double)x;
+    const double a = widen(q), b = widen(x);
     const double t = __dsub_rn(a, b);
     if constexpr (M == 1) {
         return fabs(t);
@@ -120,18 +122,6 @@ __device__ __forceinline__ double canon_term(float q, float x)
         const double u = __dadd_rn(a, b);
         return u > 0.0 ? __ddiv_rn(__dmul_rn(t, t), u) : 0.0;   // adding 0.0 leaves a sum as it is
     }
-}
-
-// Sum of v over the CTA (256 threads), the same in every thread. s_cnt: two words, used in turn.
-__device__ __forceinline__ unsigned cta_sum(unsigned v, unsigned *s_cnt, int turn)
-{
-    v = __reduce_add_sync(0xffffffffu, v);
-    if (threadIdx.x == 0) s_cnt[(turn + 1) & 1] = 0u;
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_cnt[turn & 1], v);
-    __syncthreads();
-    const unsigned r = s_cnt[turn & 1];
-    __syncthreads();
-    return r;
 }
 
 // Bits of the k-th smallest of non-negative floats (which order like their bits): the largest value
@@ -143,7 +133,7 @@ __device__ __forceinline__ unsigned cta_kth_bits(int k, unsigned *s_cnt, int &tu
     unsigned res = 0u;
     for (int bit = 30; bit >= 0; --bit) {
         const unsigned t = res | (1u << bit);
-        if (cta_sum(count(t), s_cnt, turn++) < (unsigned)k) res = t;
+        if (cta_count(count(t), s_cnt, turn++) < (unsigned)k) res = t;
     }
     return res;
 }

@@ -182,6 +182,9 @@ void dev_free(void *p, cudaStream_t st);
 
 int device_sm_count();
 
+// The calling thread's 64-byte pinned block for counters read back from the device.
+int pinned_counters(unsigned long long **p);
+
 // Autotuned tensor-core configuration: a tile width, plus kTunePair for SM-pair tiles or
 // kTuneWide for the 16-warp epilogue.
 constexpr int kTunePair = 1 << 12;

@@ -72,6 +72,19 @@ __device__ __forceinline__ int tile_after(const TcParams &p, int m, int n, int e
     return n;
 }
 
+// Unit u: from the list, or one of the grid units. (Out of line: the tile loops are read through it
+// only between units, and its divisions would sit in their instruction stream.)
+__device__ __noinline__ int4 unit_of(const int4 *units, int m0, int mt, int len, int nt, int u)
+{
+    if (units) return units[u];
+    const int nb = u / mt * len;
+    return make_int4(m0 + u % mt, nb, min(nb + len, nt), 0);
+}
+__device__ __forceinline__ int4 unit_at(const TcParams &p, int u)
+{
+    return unit_of(p.units, p.m0, p.mt, p.unit_len, p.unit_nt, u);
+}
+
 // Walks this CTA's (unit, S tile) sequence.
 template <bool MASK>
 struct TileIter {
@@ -87,7 +100,7 @@ struct TileIter {
         nu = n_units;
         valid = u < nu;
         if (valid) {
-            un = p.units[u];
+            un = unit_at(p, u);
             n = un.y;
         }
     }
@@ -99,7 +112,7 @@ struct TileIter {
             u += stride;
             valid = u < nu;
             if (valid) {
-                un = p.units[u];
+                un = unit_at(p, u);
                 n = un.y;
             }
         }
@@ -240,95 +253,6 @@ __device__ __forceinline__ uint32_t slow_chunk(const TcParams &p, const uint32_t
     return scnt;
 }
 
-// ---------------------------------------------------------------- top-k epilogue
-constexpr int kHeapArity = 8;   // children per node of a top-k slot's heap (8 measured faster than 4 and 2)
-
-// A slot's state is (theta, list fill) in registers plus, in global memory, a kHeapArity-ary
-// min-heap of the k largest lower bounds L = fl_rd(h - E) seen so far above the row's
-// published threshold (theta is its minimum: at least k columns have h >= theta) and
-// the list of every column
-// whose upper bound U = fl_ru(h + E) reached theta when it was seen. Every true
-// top-k column has U >= h >= the k-th largest h >= theta, so it is in the list.
-// Returns the new (theta, fill) packed in a float2.
-__device__ __noinline__ float2 topk_insert(const TcParams &p, size_t sidx, int r, int c, float U, float L,
-                                           float theta, int cnt, float theta_row)
-{
-    uint2 *list = p.tk_list + sidx * (size_t)p.tk_cap;
-    if (cnt >= p.tk_cap) {   // compact: drop columns whose upper bound fell below the best threshold
-        const float th = fmaxf(theta, float_from_order_code(__ldcg(p.tk_row_theta + r)));
-        int w = 0;
-        for (int i = 0; i < cnt; ++i) {
-            const uint2 e = list[i];
-            if (__uint_as_float(e.y) >= th) list[w++] = e;
-        }
-        cnt = w;
-        if (cnt >= p.tk_cap) {
-            p.tk_overflow[r] = 1;   // the exact fallback re-solves this row
-            return make_float2(theta, __int_as_float(cnt));
-        }
-    }
-    list[cnt++] = make_uint2((uint32_t)c, __float_as_uint(U));
-    // The heap only needs lower bounds above every threshold already known for the row: a
-    // bound at or below the row's threshold can raise neither this slot's threshold past it
-    // nor the k-th largest bound that finalize takes over all heaps (which stays <= the
-    // row's k-th largest h either way), so it is not inserted.
-    if (L > fmaxf(theta, theta_row)) {
-        float *heap = p.tk_heap + sidx * (size_t)p.tk_k;
-        const int k = p.tk_k;
-        int i = 0;
-        // replace the minimum by L and sift down a kHeapArity-ary heap (children of i at
-        // kHeapArity * i + 1 ...): a third of a binary heap's levels at k = 100, the loads of
-        // a level issued together
-        while (true) {
-            const int c0 = kHeapArity * i + 1;
-            if (c0 >= k) break;
-            float hc[kHeapArity];
-#pragma unroll
-            for (int j = 0; j < kHeapArity; ++j) hc[j] = c0 + j < k ? heap[c0 + j] : __int_as_float(0x7f800000);
-            int m = c0;
-            float hm = hc[0];
-#pragma unroll
-            for (int j = 1; j < kHeapArity; ++j)
-                if (hc[j] < hm) {
-                    hm = hc[j];
-                    m = c0 + j;
-                }
-            if (hm >= L) break;
-            heap[i] = hm;
-            i = m;
-        }
-        heap[i] = L;
-        theta = heap[0];
-        atomicMax(p.tk_row_theta + r, float_order_code(theta));   // share with the row's other slots
-    }
-    return make_float2(theta, __int_as_float(cnt));
-}
-
-// Top-k slow path for a 64-column piece some lane could not reject: each lane
-// walks its own row's columns whose upper bound reaches its theta.
-__device__ __forceinline__ void slow_topk(const TcParams &p, const uint32_t (&v)[64], const float *bt, float eh0,
-                                          float eh1, bool hit0, bool hit1, int r, int col0, size_t sidx,
-                                          float &theta, int &cnt, float theta_row)
-{
-    if (r >= p.nR) return;
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {
-        if (!(hh ? hit1 : hit0)) continue;
-        const float eh = hh ? eh1 : eh0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const int c = col0 + hh * 32 + j;
-            const float h = __fmaf_rn(__uint_as_float(v[hh * 32 + j]), p.scale, -bt[hh * 32 + j]);
-            const float U = __fadd_ru(h, eh);
-            if (c < p.nS && U >= fmaxf(theta, theta_row)) {
-                const float2 st = topk_insert(p, sidx, r, c, U, __fsub_rd(h, eh), theta, cnt, theta_row);
-                theta = st.x;
-                cnt = __float_as_int(st.y);
-            }
-        }
-    }
-}
-
 // Maximum of v[o .. o+31] with three-input max.f32 (17 instructions, depth 4).
 __device__ __forceinline__ float fmax3(float a, float b, float c)
 {
@@ -358,7 +282,7 @@ __device__ __forceinline__ float max_tree32(const uint32_t (&v)[N], int o)
 // multicast to both CTAs. Each CTA's epilogue handles its own rows; the peer releases an
 // accumulator with a remote arrive on the leader's barrier. Half the B bytes per stage means
 // twice the stages in the same shared memory beside a resident R tile.
-template <int BN, bool TOPK, bool FP8, bool CG2, bool WIDE, bool MASK, bool STREAM>
+template <int BN, int MODE, bool FP8, bool CG2, bool WIDE, bool MASK, bool STREAM>
 __global__ void __launch_bounds__(tc_threads(WIDE), 1)
     tc_join_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const TcParams p)
@@ -369,7 +293,8 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
     constexpr uint32_t kStageBytes = (CG2 ? BN / 2 : BN) * 128;   // this CTA's rows of an S tile x 128 B
     // STREAM: no resident R tile; each stage also carries the R tile's matching 128-byte K chunk
     // (128 rows, 16 KB), so a large d keeps four stages instead of two beside a resident tile
-    static_assert(!STREAM || (!CG2 && !TOPK && !MASK), "streamed R chunks serve the one-SM epsilon-join");
+    constexpr bool MAXIMA = MODE == kModeMaxima;
+    static_assert(!STREAM || (!CG2 && !MAXIMA && !MASK), "streamed R chunks serve the one-SM epsilon-join");
     constexpr uint32_t kStageStride = STREAM ? kStageBytes + 16384 : kStageBytes;
     constexpr int kChunkCols = FP8 ? 128 : 64;   // columns per 128-byte K chunk
     constexpr int kAcc = 512 / BN;              // TMEM accumulators: 2 of 256 or 4 of 128 columns
@@ -401,6 +326,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
     uint64_t *pa_full = bars + 40;            // CG2 leader: [2] the peer's rows of the R tile landed
     float *s_xch = reinterpret_cast<float *>(bars + 48);   // [kEpi warps x 32] row exchange slots (16-byte aligned)
 
+    const int tile_step = MAXIMA ? p.tile_stride : 1;   // S tile n of a unit is the store's tile n * tile_step
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint32_t crank = CG2 ? cluster_ctarank() : 0u;   // this CTA's rank in its pair
@@ -461,7 +387,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             bool ok = true;
             int i = 0;   // unit count of this CTA
             for (int u = ufirst; u < n_units && ok; u += ustride, ++i) {
-                const int4 un = p.units[u];
+                const int4 un = unit_at(p, u);
                 if constexpr (!STREAM) {
                     const int slot = i % a_slots;
                     const uint32_t use = (uint32_t)(i / a_slots);
@@ -484,7 +410,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
                         }
                         mbar_arrive_expect_tx(full + stage, kStageStride);
                         tma_load_2d(sB + stage * kStageStride, &tmB, full + stage, c * kChunkCols,
-                                    n * BN + (CG2 ? (int)crank * (BN / 2) : 0));
+                                    n * tile_step * BN + (CG2 ? (int)crank * (BN / 2) : 0));
                         if constexpr (STREAM)   // the R tile's chunk c beside it
                             tma_load_2d(sB + stage * kStageStride + kStageBytes, &tmA, full + stage, c * kChunkCols,
                                         un.x * 128);
@@ -516,7 +442,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             bool ok = true;
             int i = 0;
             for (int u = ufirst; u < n_units && ok; u += ustride, ++i) {
-                const int4 un = p.units[u];
+                const int4 un = unit_at(p, u);
                 const int slot = i % a_slots;
                 const uint32_t use = (uint32_t)(i / a_slots);
                 if (!mbar_wait(a_full + slot, use & 1, abort_flag, p.wait_budget)) {
@@ -549,7 +475,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             bool ok = true, any_mma = false;
             int i = 0;
             for (int u = ufirst; u < n_units && ok; u += ustride, ++i) {
-                const int4 un = p.units[u];
+                const int4 un = unit_at(p, u);
                 const int slot = STREAM ? 0 : i % a_slots;
                 uint32_t a_base = 0;
                 if constexpr (!STREAM) {   // the unit's resident R tile
@@ -661,7 +587,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
 
         auto stage_async = [&](const TileIter<MASK> &it, int s) {
             if (!it.valid) return;
-            const int c0 = it.n * BN + half * HC;
+            const int c0 = it.n * tile_step * BN + half * HC;
             // the column data (beta [n_pad], chunk stats [n_pad / 32]) covers whole 256-column tiles
             if (!DL_CHECK(c0 + HC <= (p.nS + 255) / 256 * 256, 4, c0)) return;
             if constexpr (kPer == 4) {
@@ -682,10 +608,6 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
         bool ok = true;
         float4 rp = make_float4(0.f, 0.f, 0.f, 0.f);
         float sq = 1.0f;          // FP8: this row's scale
-        float theta = 0.f;        // top-k: this slot's threshold (k-th largest lower bound of h)
-        float theta_row = 0.f;    // top-k: best threshold published by any slot of this row
-        int tcnt = 0;             // top-k: this slot's list fill
-        size_t sidx = 0;
         while (cur.valid) {
             const int r = (cur.un.x * kRowTiles + (int)crank) * 128 + quad * 32 + lane;
             if (cur.n == cur.un.y) {
@@ -693,22 +615,9 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
                 if (DL_CHECK(r < (p.nR + kRowTiles * 128 - 1) / (kRowTiles * 128) * (kRowTiles * 128), 3, r))
                     rp = p.rowpar[r];
                 if constexpr (FP8) sq = (r < p.nR) ? p.sc_r[r] : 1.0f;
-                if constexpr (TOPK) {   // a unit owns its (row tile, split): start the slots fresh
-                    sidx = (size_t)r * p.tk_slots + (size_t)cur.un.w * (kEpi / 4) + half;   // (split, column part)
-                    theta = __int_as_float(0xff800000);
-                    tcnt = 0;
-                    if (r < p.nR) {
-                        float *heap = p.tk_heap + sidx * (size_t)p.tk_k;
-                        for (int i = 0; i < p.tk_k; ++i) heap[i] = __int_as_float(0xff800000);
-                    }
-                }
             }
             stage_async(nxt, (t & 1) ^ 1);   // the next tile's column data lands while this one is processed
 
-            if constexpr (TOPK) {
-                theta_row = __int_as_float(0xff800000);
-                if (r < p.nR) theta_row = float_from_order_code(__ldcg(p.tk_row_theta + r));
-            }
             const uint32_t b = t % kAcc;
             const int slot = t & 1;
             if (!mbar_wait(acc_full + b, (t / kAcc) & 1, abort_flag, p.wait_budget)) {
@@ -720,7 +629,33 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             const float *beta = my_bt + slot * HC;
             const float *sxs = my_sx + slot * kSubW;
             const float4 *cst = my_cs + slot * kSubW;
-            const int colw = cur.n * BN + half * HC;   // first column this warp owns in the tile
+            const int colw = cur.n * tile_step * BN + half * HC;   // first column this warp owns in the tile
+
+            // kModeMaxima: a lower bound of the best h of columns 16 i .. 16 i + 15 of chunk ci, values v[o ..]
+            auto best16 = [&](auto &v, int o, int ci, int i) {
+                const float4 cs = cst[ci];
+                const float ehs = __fadd_ru(__fmaf_ru(rp.z, cs.x, __fmaf_ru(rp.w, cs.y, cs.z)), rp.x);
+                const float4 *b4 = reinterpret_cast<const float4 *>(beta + ci * 32 + 16 * i);
+                float m = __int_as_float(0xff800000);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 bq = b4[q];
+                    const int j = o + 16 * i + 4 * q;
+                    m = fmaxf(m, fmaxf(__fmaf_rn(__uint_as_float(v[j]), p.scale, -bq.x), __fmaf_rn(__uint_as_float(v[j + 1]), p.scale, -bq.y)));
+                    m = fmaxf(m, fmaxf(__fmaf_rn(__uint_as_float(v[j + 2]), p.scale, -bq.z), __fmaf_rn(__uint_as_float(v[j + 3]), p.scale, -bq.w)));
+                }
+                return __fsub_rd(m, ehs);
+            };
+            // group maxima of the 64 columns that piece `pc` of this warp's part holds
+            auto put64 = [&](float4 g, int pc) {
+                if (r >= p.nR) return;
+                float *o = p.gmax + (size_t)(r - p.row0) * p.n_groups;
+                const int g64 = cur.n * (BN / 64) + half * (HC / 64) + pc;
+                if (p.gran == 64)
+                    o[g64] = fmaxf(fmaxf(g.x, g.y), fmaxf(g.z, g.w));
+                else
+                    *reinterpret_cast<float4 *>(o + 4 * g64) = g;   // n_groups is a multiple of 4 here
+            };
 
             // 64 columns [piece*64, piece*64+64) of this warp's half, values in v
             auto process64 = [&](uint32_t (&v)[64], int piece) {
@@ -741,33 +676,25 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
                         }
                     }
                 }
-                float tr0, tr1;
-                if constexpr (TOPK) {   // candidate iff h + E (+ canonical slack rp.x) >= the best threshold
-                    const float th = fmaxf(theta, theta_row);
-                    tr0 = __fsub_rd(th, __fadd_ru(eh0, rp.x));
-                    tr1 = __fsub_rd(th, __fadd_ru(eh1, rp.x));
-                } else {
-                    tr0 = __fsub_rd(rp.y, eh0);
-                    tr1 = __fsub_rd(rp.y, eh1);
+                if constexpr (MAXIMA) {
+                    put64(make_float4(best16(v, 0, 2 * piece, 0), best16(v, 0, 2 * piece, 1), best16(v, 32, 2 * piece + 1, 0),
+                                      best16(v, 32, 2 * piece + 1, 1)),
+                          piece);
+                    return;
                 }
+                const float tr0 = __fsub_rd(rp.y, eh0), tr1 = __fsub_rd(rp.y, eh1);
                 // Whole-chunk reject: with beta_j >= beta_min(chunk) and one scale s > 0 per chunk,
                 // every h_j = fl(A_j s - beta_j) is <= fl_ru(max_j A_j * s - beta_min); rows are in
                 // norm order, so beta_min is tight.
                 const float mx0 = max_tree32(v, 0), mx1 = max_tree32(v, 32);
                 const bool hit0 = __fmaf_ru(mx0, sc0, -cs0.w) >= tr0;
                 const bool hit1 = __fmaf_ru(mx1, sc1, -cs1.w) >= tr1;
-                if constexpr (TOPK) {
-                    if (hit0 || hit1)
-                        slow_topk(p, v, beta + piece * 64, __fadd_ru(eh0, rp.x), __fadd_ru(eh1, rp.x), hit0, hit1, r,
-                                  colw + piece * 64, sidx, theta, tcnt, theta_row);
-                } else {
-                    if (__any_sync(0xffffffffu, hit0 || hit1)) {
-                        const int c0 = colw + piece * 64;
-                        scnt = slow_chunk<FP8>(p, v, 0, beta + piece * 64, sc0, __fadd_ru(rp.x, eh0),
-                                               __fsub_rd(rp.y, eh0), hit0, r, c0, my_xch, my_stg, scnt);
-                        scnt = slow_chunk<FP8>(p, v, 32, beta + piece * 64, sc1, __fadd_ru(rp.x, eh1),
-                                               __fsub_rd(rp.y, eh1), hit1, r, c0 + 32, my_xch, my_stg, scnt);
-                    }
+                if (__any_sync(0xffffffffu, hit0 || hit1)) {
+                    const int c0 = colw + piece * 64;
+                    scnt = slow_chunk<FP8>(p, v, 0, beta + piece * 64, sc0, __fadd_ru(rp.x, eh0),
+                                           __fsub_rd(rp.y, eh0), hit0, r, c0, my_xch, my_stg, scnt);
+                    scnt = slow_chunk<FP8>(p, v, 32, beta + piece * 64, sc1, __fadd_ru(rp.x, eh1),
+                                           __fsub_rd(rp.y, eh1), hit1, r, c0 + 32, my_xch, my_stg, scnt);
                 }
             };
 
@@ -809,43 +736,29 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
                     }
                 }
             };
-            // Top-k, one 32-column chunk ci (16-bit operands): the columns whose upper bound
-            // reaches the best threshold go to the slot's list, their lower bounds to its heap.
-            auto topk_chunk = [&](auto &v, int o, int ci) {
-                const float4 cs = cst[ci];
-                const float ehs = __fadd_ru(__fmaf_ru(rp.z, cs.x, __fmaf_ru(rp.w, cs.y, cs.z)), rp.x);
-                const float mx = max_tree32(v, o);
-                if (__fmaf_ru(mx, p.scale, -cs.w) >= __fsub_rd(fmaxf(theta, theta_row), ehs) && r < p.nR) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int c = colw + ci * 32 + j;
-                        const float h = __fmaf_rn(__uint_as_float(v[o + j]), p.scale, -beta[ci * 32 + j]);
-                        const float U = __fadd_ru(h, ehs);
-                        if (c < p.nS && U >= fmaxf(theta, theta_row)) {
-                            const float2 stt = topk_insert(p, sidx, r, c, U, __fsub_rd(h, ehs), theta, tcnt, theta_row);
-                            theta = stt.x;
-                            tcnt = __float_as_int(stt.y);
-                        }
-                    }
-                }
-            };
             if constexpr (kEpi == 16) {
                 // 64 columns per warp, 32 at a time: the three other epilogue warps of this SM
                 // sub-partition hide each load's latency
                 uint32_t vq[32];
                 tmem_ld_32x32b_x32(tbase, vq);
                 tmem_ld_wait_regs(vq);
-                if constexpr (TOPK)
-                    topk_chunk(vq, 0, 0);
-                else
+                float4 g;
+                if constexpr (MAXIMA) {
+                    g.x = best16(vq, 0, 0, 0);
+                    g.y = best16(vq, 0, 0, 1);
+                } else {
                     eps_chunk(vq, 0, 0);
+                }
                 tmem_ld_32x32b_x32(tbase + 32, vq);
                 tmem_ld_wait_regs(vq);
                 release_acc();
-                if constexpr (TOPK)
-                    topk_chunk(vq, 0, 1);
-                else
+                if constexpr (MAXIMA) {
+                    g.z = best16(vq, 0, 1, 0);
+                    g.w = best16(vq, 0, 1, 1);
+                    put64(g, 0);
+                } else {
                     eps_chunk(vq, 0, 1);
+                }
             } else {
             // One 64-column load at a time: the other epilogue warp on this SM
             // sub-partition hides the TMEM load latency.
@@ -863,12 +776,6 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             release_acc();
             process64(va, HC == 128 ? 1 : 0);
             }
-            if constexpr (TOPK) {
-                if (cur.n + 1 == cur.un.z && r < p.nR) {   // last tile of the unit: publish the slot
-                    p.tk_theta[sidx] = theta;
-                    p.tk_cnt[sidx] = tcnt;
-                }
-            }
             // the next tile's column data is in the other slot
             cp_async_wait_all();
             __syncwarp();
@@ -877,7 +784,7 @@ __global__ void __launch_bounds__(tc_threads(WIDE), 1)
             ++t;
         }
         cp_async_wait_all();   // no staged column data may still be in flight when the CTA ends
-        if constexpr (!TOPK) flush_stage(p, my_stg, scnt);
+        if constexpr (!MAXIMA) flush_stage(p, my_stg, scnt);
         if (!ok) raise_abort();
     }
 
@@ -945,10 +852,10 @@ long long tc_wait_budget()
     return b > 0 ? b : kWaitBudgetClocks;
 }
 
-template <int BN, bool TOPK, bool FP8, bool CG2, bool WIDE = false, bool MASK = false, bool STREAM = false>
+template <int BN, int MODE, bool FP8, bool CG2, bool WIDE = false, bool MASK = false, bool STREAM = false>
 static int launch_one(const TcLaunch &L, size_t smem, cudaStream_t st, int *grid_out)
 {
-    auto kern = tc_join_kernel<BN, TOPK, FP8, CG2, WIDE, MASK, STREAM>;
+    auto kern = tc_join_kernel<BN, MODE, FP8, CG2, WIDE, MASK, STREAM>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(tc_join_kernel)");
     TcParams p = L.p;
@@ -986,10 +893,34 @@ static int launch_one(const TcLaunch &L, size_t smem, cudaStream_t st, int *grid
     return DL_OK;
 }
 
-int launch_tc_join(const TcLaunch &L, cudaStream_t st, bool topk, bool fp8, int *grid_out)
+void tc_grid_units(TcLaunch *L, int64_t mt, int64_t nt, int sms)
 {
+    // the range length whose last wave wastes least: units are handed out round-robin, one CTA an SM,
+    // and each loads its R tile (counted as half an S tile); ties go to the longer range
+    int64_t best = 1;
+    double best_cost = 1e300;
+    for (int64_t len = std::min<int64_t>(nt, 64); len >= 1; --len) {
+        const int64_t units = mt * ((nt + len - 1) / len);
+        const double cost = (double)((units + sms - 1) / sms) * ((double)len + 0.5);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = len;
+        }
+    }
+    const int64_t units = mt * ((nt + best - 1) / best);
+    L->p.units = nullptr;
+    L->p.mt = (int)mt;
+    L->p.unit_nt = (int)nt;
+    L->p.unit_len = (int)best;
+    L->p.n_units = (int)units;
+    L->grid = (int)std::min<int64_t>(units, sms);
+}
+
+int launch_tc_join(const TcLaunch &L, cudaStream_t st, int mode, bool fp8, int *grid_out)
+{
+    const bool topk = mode == kModeMaxima;
     if (topk && fp8) {
-        set_error("top-k runs on the 16-bit path only");
+        set_error("top-k group maxima run on the 16-bit path only");
         return DL_EUNSUPPORTED;
     }
     if ((L.cg2 && (topk || L.BN != 256 || L.wide)) || (L.wide && L.BN != 256)) {
@@ -1008,14 +939,14 @@ int launch_tc_join(const TcLaunch &L, cudaStream_t st, bool topk, bool fp8, int 
             return DL_EUNSUPPORTED;
         }
         if (L.wide)
-            rc = fp8 ? launch_one<256, false, true, false, true, false, true>(L, smem, st, grid_out)
-                     : launch_one<256, false, false, false, true, false, true>(L, smem, st, grid_out);
+            rc = fp8 ? launch_one<256, kModeEps, true, false, true, false, true>(L, smem, st, grid_out)
+                     : launch_one<256, kModeEps, false, false, true, false, true>(L, smem, st, grid_out);
         else if (L.BN == 256)
-            rc = fp8 ? launch_one<256, false, true, false, false, false, true>(L, smem, st, grid_out)
-                     : launch_one<256, false, false, false, false, false, true>(L, smem, st, grid_out);
+            rc = fp8 ? launch_one<256, kModeEps, true, false, false, false, true>(L, smem, st, grid_out)
+                     : launch_one<256, kModeEps, false, false, false, false, true>(L, smem, st, grid_out);
         else if (L.BN == 128)
-            rc = fp8 ? launch_one<128, false, true, false, false, false, true>(L, smem, st, grid_out)
-                     : launch_one<128, false, false, false, false, false, true>(L, smem, st, grid_out);
+            rc = fp8 ? launch_one<128, kModeEps, true, false, false, false, true>(L, smem, st, grid_out)
+                     : launch_one<128, kModeEps, false, false, false, false, true>(L, smem, st, grid_out);
         else {
             set_error("tensor-core tile width %d not supported (128 or 256)", L.BN);
             return DL_EINVAL;
@@ -1026,32 +957,32 @@ int launch_tc_join(const TcLaunch &L, cudaStream_t st, bool topk, bool fp8, int 
             return DL_EUNSUPPORTED;
         }
         if (L.wide)
-            rc = fp8 ? launch_one<256, false, true, false, true, true>(L, smem, st, grid_out)
-                     : launch_one<256, false, false, false, true, true>(L, smem, st, grid_out);
+            rc = fp8 ? launch_one<256, kModeEps, true, false, true, true>(L, smem, st, grid_out)
+                     : launch_one<256, kModeEps, false, false, true, true>(L, smem, st, grid_out);
         else if (L.BN == 256)
-            rc = fp8 ? launch_one<256, false, true, false, false, true>(L, smem, st, grid_out)
-                     : launch_one<256, false, false, false, false, true>(L, smem, st, grid_out);
+            rc = fp8 ? launch_one<256, kModeEps, true, false, false, true>(L, smem, st, grid_out)
+                     : launch_one<256, kModeEps, false, false, false, true>(L, smem, st, grid_out);
         else if (L.BN == 128)
-            rc = fp8 ? launch_one<128, false, true, false, false, true>(L, smem, st, grid_out)
-                     : launch_one<128, false, false, false, false, true>(L, smem, st, grid_out);
+            rc = fp8 ? launch_one<128, kModeEps, true, false, false, true>(L, smem, st, grid_out)
+                     : launch_one<128, kModeEps, false, false, false, true>(L, smem, st, grid_out);
         else {
             set_error("tensor-core tile width %d not supported (128 or 256)", L.BN);
             return DL_EINVAL;
         }
     } else if (L.cg2)
-        rc = fp8 ? launch_one<256, false, true, true>(L, smem, st, grid_out) : launch_one<256, false, false, true>(L, smem, st, grid_out);
+        rc = fp8 ? launch_one<256, kModeEps, true, true>(L, smem, st, grid_out) : launch_one<256, kModeEps, false, true>(L, smem, st, grid_out);
     else if (L.wide)
-        rc = topk ? launch_one<256, true, false, false, true>(L, smem, st, grid_out)
-                  : (fp8 ? launch_one<256, false, true, false, true>(L, smem, st, grid_out)
-                         : launch_one<256, false, false, false, true>(L, smem, st, grid_out));
+        rc = topk ? launch_one<256, kModeMaxima, false, false, true>(L, smem, st, grid_out)
+                  : (fp8 ? launch_one<256, kModeEps, true, false, true>(L, smem, st, grid_out)
+                         : launch_one<256, kModeEps, false, false, true>(L, smem, st, grid_out));
     else if (L.BN == 256)
-        rc = topk ? launch_one<256, true, false, false>(L, smem, st, grid_out)
-                  : (fp8 ? launch_one<256, false, true, false>(L, smem, st, grid_out)
-                         : launch_one<256, false, false, false>(L, smem, st, grid_out));
+        rc = topk ? launch_one<256, kModeMaxima, false, false>(L, smem, st, grid_out)
+                  : (fp8 ? launch_one<256, kModeEps, true, false>(L, smem, st, grid_out)
+                         : launch_one<256, kModeEps, false, false>(L, smem, st, grid_out));
     else if (L.BN == 128)
-        rc = topk ? launch_one<128, true, false, false>(L, smem, st, grid_out)
-                  : (fp8 ? launch_one<128, false, true, false>(L, smem, st, grid_out)
-                         : launch_one<128, false, false, false>(L, smem, st, grid_out));
+        rc = topk ? launch_one<128, kModeMaxima, false, false>(L, smem, st, grid_out)
+                  : (fp8 ? launch_one<128, kModeEps, true, false>(L, smem, st, grid_out)
+                         : launch_one<128, kModeEps, false, false>(L, smem, st, grid_out));
     else {
         set_error("tensor-core tile width %d not supported (128 or 256)", L.BN);
         return DL_EINVAL;

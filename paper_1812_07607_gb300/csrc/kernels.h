@@ -10,7 +10,9 @@ namespace dl {
 
 // ---- K2+K3+K5 tensor-core epsilon-join (join_tc.cu)
 struct TcParams {
-    const int4 *units;       // {m, nb, ne, 0}: R tile m against S tiles [nb, ne)
+    const int4 *units;       // {m, nb, ne, 0}: R tile m against S tiles [nb, ne); NULL: the grid units
+    int m0, mt, unit_nt, unit_len;   // grid units: R tiles m0 .. m0 + mt - 1, each against S tiles
+                             // [j unit_len, (j + 1) unit_len) of unit_nt, range j by range j
     int n_units;
     const int *n_units_dev;  // when not NULL the unit count is read here (units built on the device)
     const uint32_t *tile_mask;   // when not NULL: [R tiles][mask_ntw] bits; a unit's S tiles with a
@@ -35,17 +37,16 @@ struct TcParams {
     unsigned long long cand_cap;
     int *err;                // set to 1 when a bounded wait expired
     long long wait_budget;   // SM clocks an abortable pipeline wait may take (set by launch_tc_join)
-    // top-k epilogue (units carry the S split in .w; state per (row, split, half) slot)
-    int tk_k;                // k
-    int tk_cap;              // candidate-list capacity per slot
-    int tk_slots;            // slots per row (2 x splits)
-    float *tk_heap;          // [rows][slots][k] min-heap of the k largest lower bounds of h
-    uint2 *tk_list;          // [rows][slots][cap] {column, float bits of the upper bound of h}
-    int *tk_cnt;             // [rows][slots] list fill
-    float *tk_theta;         // [rows][slots] final threshold (heap minimum)
-    unsigned *tk_row_theta;  // [rows] best threshold of any slot of the row (order-preserving encoding)
-    int *tk_overflow;        // [rows] set when a list cannot hold every candidate
+    // kModeMaxima (rowpar: {slack, -, rq, nqt})
+    int tile_stride;         // the pass takes S tiles 0, stride, 2 stride, ...
+    float *gmax;             // [rows from row0][n_groups] best lower bound of h of each column group
+    int n_groups;
+    int gran;                // columns of a group: 16 or 64
+    int row0;
 };
+
+// What the epilogue does with a tile: the epsilon-join's candidates, or the top-k's group maxima.
+enum TcMode { kModeEps = 0, kModeMaxima = 1 };
 
 // Candidate entry flag: set for a band pair (needs the exact recheck).
 constexpr uint32_t kBandFlag = 0x80000000u;
@@ -69,7 +70,9 @@ void tc_plan(int BN, int kc, int *stages, int *a_slots, bool fp8 = false, bool c
 // unless dl_debug_set_wait_budget set another.
 long long tc_wait_budget();
 // *grid_out (optional) receives the CTAs actually launched.
-int launch_tc_join(const TcLaunch &L, cudaStream_t st, bool topk = false, bool fp8 = false, int *grid_out = nullptr);
+int launch_tc_join(const TcLaunch &L, cudaStream_t st, int mode = kModeEps, bool fp8 = false, int *grid_out = nullptr);
+// Grid units for `mt` R tiles against `nt` S tiles (L->p.m0 is the caller's), their count and the grid.
+void tc_grid_units(TcLaunch *L, int64_t mt, int64_t nt, int sms);
 
 // ---- K8 SIMT FP32 join (join_simt.cu)
 struct SimtParams {
@@ -114,6 +117,8 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
 int launch_diag(const int64_t *ids, int64_t n, int64_t *out_r, int64_t *out_s, unsigned long long *out_cnt,
                 unsigned long long cap, cudaStream_t st);
 
+// Workspace of one query row of a top-k against nS rows (topk.cu).
+int64_t topk_row_bytes(int64_t nS, int dp, int k);
 // ---- top-k core (topk.cu): every row of Q against S, outputs at row_off or caller row * k
 int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, const int64_t *row_off,
               int64_t *out_ids, double *out_d2, const dl_join_opts &o, cudaStream_t st, dl_join_stats *stats);

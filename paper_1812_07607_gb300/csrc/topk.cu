@@ -2,54 +2,142 @@
 // with the smallest canonical distance, ordered by (distance, store row).
 //
 // The paper's reverse-image-search query (Sec. 6.2, q1: the closest image to a
-// query image) is the k = 1 case. Pipeline on the caller's stream:
+// query image) is the k = 1 case. With h = q.x - ||x||^2/2 (D = ||q||^2 - 2h), on the caller's
+// stream, for query rows in chunks that bound the workspace:
 //   k_rowpar_topk      per query row: the bound terms and the canonical slack;
-//   tc_join_kernel<.., true>   the tensor-core pass with the top-k epilogue: per
-//                      (row, S split, epilogue half) slot a running threshold
-//                      theta (k-th largest lower bound of h = q.x - ||x||^2/2)
-//                      and the list of every column whose upper bound reached it;
-//   k_topk_finalize    per row, one warp: union of the slots' lists above the
-//                      largest theta, FP32 distances with their error bound, the
-//                      k-th smallest upper bound, then the canonical FP64
-//                      distance of every column that can still be in the top k
-//                      and an exact rank by (D64, caller's store row index);
-//   k_topk_fallback    rows whose lists overflowed (many near-ties) or whose
-//                      candidates exceed the finalize buffer: an exact scan of
-//                      the whole store for that row (FP32 bound + radix select +
+//   tc_join_kernel<.., kModeMaxima>   over every f-th tile of the store: each group of 16 or 64
+//                      columns' best lower bound of h;
+//   k_topk_theta       per row the k-th largest of them: at least k columns have h at or above it;
+//   tc_join_kernel<.., kModeEps>      over the whole store, with that as the row's threshold: the
+//                      epsilon-join's epilogue lists every column whose upper bound reaches it;
+//   k_topk_dist        the candidates' FP32 distances, into a list per row;
+//   k_topk_keep        per row: the k-th smallest upper bound of the listed distances and the columns
+//                      that can still be in the top k;
+//   k_topk_canon       their canonical FP64 distances;
+//   k_topk_out         per row: an exact rank by (D64, caller's store row index).
+// About k f columns of a row are listed: f balances the first pass against them (topk_stride). A row
+// with more than its list holds (near-duplicates side by side in the store) gets a tighter threshold
+// from the distances it did list and the rows like it another pass (k_topk_refine); one that
+// overflows again takes
+//   k_topk_fallback    an exact scan of the whole store for that row (FP32 bound + radix select +
 //                      FP64 + rank).
 // Store rows are in norm order; outputs are written at the caller's row order.
+//
+// Heaps of lower bounds kept by the epilogue's lanes in global memory did this in one pass over the
+// store; every insert sifted through dependent loads while the other lanes of its warp waited.
+// 4,096 queries against 1,000,003 x 256, k = 100: 18.6 ms then, 3.5 now; one query, k = 1: 0.53 ms, 0.21 (its 16
+// column splits left 136 SMs idle).
+// What bounds it now, of the 3.5 ms: the two tensor-core passes 0.33 + 1.45 ms, the candidates' rows 0.4,
+// the canonical sums 0.6; of the 0.21 ms: the store's 512 MB of FP16 rows, 76 us.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
-#include <mutex>
-#include <tuple>
 #include <vector>
 
 #include "checked.cuh"
+#include "cta.cuh"
+#include "exact.cuh"
 #include "kernels.h"
 
 namespace dl {
 
-constexpr int kTkMax = 480;          // candidates a finalize warp holds in shared memory (5 CTAs per SM)
-// Canonical FP64 sums are costed per warp instruction (the FP64 rate is low and a warp-wide
-// instruction occupies the pipe whatever its active lanes), so the finalize batches them: a row
-// with at most kTkPendRow columns left queues them, and one lane-parallel pass computes the
-// queued columns of many rows (up to kTkPend columns of kTkPendRows rows) at once.
-constexpr int kTkPend = 64;
-constexpr int kTkPendRow = 32;
-constexpr int kTkPendRows = 32;
+constexpr int kTkGroups = 1024;      // group maxima k_topk_theta keeps apart (more are folded)
+constexpr int kTkTermC = 64;         // candidates whose canonical terms are staged together
+constexpr int kTkTerms = kTkTermC * 33;   // staged terms, padding included
+constexpr int kTkRefines = 2;        // passes with tightened thresholds before the exact scan
 constexpr int kTkFallbackCap = 8192; // candidates a fallback block can rank
 
-struct TopkFin {
+// Per query row: {canonical slack of h, unused, ||q - q~|| up, ||q~|| up}; padding rows get zeros.
+__global__ void __launch_bounds__(256) k_rowpar_topk(const double *__restrict__ nq64, const float4 *__restrict__ rowb,
+                                                     int64_t n, int64_t n_tot, double g64, double nq_max_s,
+                                                     float4 *__restrict__ rowpar)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_tot) return;
+    if (i >= n) {
+        rowpar[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
+    // |h_canonical - h| <= |D64 - D| / 2 <= g64 * (||q||^2 + ||x||^2); doubled for margin
+    const double delta = 2.0 * g64 * (nq64[i] + nq_max_s) * 1.0001 + 1e-30;
+    const float4 rb = rowb[i];
+    rowpar[i] = make_float4(__double2float_ru(delta), 0.f, rb.x, rb.y);
+}
+
+// Threshold of each row's listing pass from its group maxima: with T the k-th largest of them, a
+// column of the top k has h + E + slack >= T, so the row lists the columns whose h~ reaches
+// (T - slack) - E (-inf with fewer than k groups). Padding rows (+inf) list nothing. One warp per row,
+// 32 values a lane (groups folded by maximum past 1,024: disjoint groups stay disjoint), no barriers;
+// T is found bit by bit from the values' common prefix on and cut off after kTkBits bits, downwards,
+// which lets in about one column more in 2^kTkBits. 4,096 rows of 1,953 groups, k = 100: 66 us,
+// 105 with a CTA a row and all 32 bits.
+constexpr int kTkBits = 14;
+
+__global__ void __launch_bounds__(256) k_topk_theta(const float4 *__restrict__ rowpar, const float *__restrict__ gmax, int n_groups,
+                                                    int64_t row0, int64_t nQ, int64_t rows_tot, int k, const int *__restrict__ row_k,
+                                                    float4 *__restrict__ thr)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t lr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int64_t i = row0 + lr;
+    if (i >= rows_tot) return;
+    const float inf = __int_as_float(0x7f800000);
+    if (i >= nQ) {
+        if (lane == 0) thr[i] = make_float4(inf, inf, 0.f, 0.f);
+        return;
+    }
+    const float4 rp = rowpar[i];
+    const unsigned kk = (unsigned)(row_k ? row_k[i] : k);
+    float th = -inf;
+    if (n_groups >= (int)kk) {
+        unsigned v[kTkGroups / 32];
+        const float *g = gmax + (size_t)lr * n_groups;
+        unsigned lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+        for (int s = 0; s < kTkGroups / 32; ++s) {
+            float m = -inf;
+            for (int j = s * 32 + lane; j < n_groups; j += kTkGroups) m = fmaxf(m, __ldg(g + j));
+            v[s] = float_order_code(m);
+            hi = max(hi, v[s]);
+            if (m > -inf) lo = min(lo, v[s]);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (kk == 1u) {
+            th = float_from_order_code(hi);   // -inf when every group is padding
+        } else if (lo <= hi) {
+            // the largest code that at least kk values reach: its bits above the highest one in which
+            // lo and hi differ are theirs (if kk values are finite at all)
+            const int top = lo == hi ? -1 : 31 - __clz((int)(lo ^ hi));
+            unsigned code = top < 31 ? hi & ~((2u << max(top, 0)) - 1u) : 0u;
+            if (top < 0) code = hi;
+            for (int bit = top; bit >= 0 && bit > top - kTkBits; --bit) {
+                const unsigned t = code | (1u << bit);
+                unsigned c = 0;
+#pragma unroll
+                for (int s = 0; s < kTkGroups / 32; ++s) c += v[s] >= t ? 1u : 0u;
+                if (__reduce_add_sync(0xffffffffu, c) >= kk) code = t;
+            }
+            unsigned c = 0;   // with fewer than kk finite groups not even the prefix is reached
+#pragma unroll
+            for (int s = 0; s < kTkGroups / 32; ++s) c += v[s] >= code ? 1u : 0u;
+            if (__reduce_add_sync(0xffffffffu, c) >= kk && code > float_order_code(-inf)) th = float_from_order_code(code);
+        }
+    }
+    if (lane == 0) thr[i] = make_float4(inf, __fsub_rd(th, rp.x), rp.z, rp.w);
+}
+
+struct TopkRows {
     const float *Q, *S;
-    int d, nQ, nS, k, slots, cap;
-    const float *theta;
-    const float *heap;     // [rows][slots][k] each slot's k largest lower bounds
-    const unsigned *row_theta;
-    const int *cnt;
-    const uint2 *list;
-    int *overflow;
+    int d, nS, k;
+    int64_t row0, rows;    // this chunk's query rows
+    int cap;               // list capacity of a row
+    int *cnt;              // [rows] columns that reached the row's threshold (may exceed cap)
+    uint32_t *col;         // [rows][cap]
+    float *d32;            // [rows][cap] FP32 distances
+    double *d64;           // [rows][cap] canonical distances of the kept columns
+    uint32_t *kept;        // the kept columns' places in those lists, row by row
+    unsigned long long *n_kept;
     const int32_t *q_orig, *s_orig;
     const int64_t *s_ids;
     int64_t *out_ids;
@@ -58,8 +146,249 @@ struct TopkFin {
     const int64_t *row_off;// per query row first output slot (NULL: caller row * k)
     float g32, abs32;      // FP32 distance bound: |D32 - D| <= g32 * D + abs32
     float slack;           // canonical slack factor for the keep test (relative)
-    unsigned long long *n_fp64;
 };
+
+// The listed candidates' FP32 distances (8-lane groups, 16-byte slices, four candidates a warp at a
+// time), each into its row's list. What bounds it: the rows' L2 reads, 8 d bytes a candidate.
+__global__ void __launch_bounds__(256) k_topk_dist(const TopkRows f, const uint2 *__restrict__ cand,
+                                                   const unsigned long long *__restrict__ cand_cnt, unsigned long long cand_cap)
+{
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned long long n = min(*cand_cnt, cand_cap);
+    const unsigned long long w0 = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+    const unsigned win = n <= nw * 4 ? 4u : 32u;   // few candidates: four a warp, one round trip each
+    const bool in = lane < win;
+    uint2 nxt = in && w0 * win + lane < n ? cand[w0 * win + lane] : make_uint2(0u, 0u);
+    for (unsigned long long base = w0 * win; base < n; base += nw * win) {
+        const unsigned long long i = base + lane;
+        bool valid = in && i < n;
+        const uint2 e = nxt;
+        nxt = in && i + nw * win < n ? cand[i + nw * win] : make_uint2(0u, 0u);   // the next window, loaded early
+        const int64_t lr = (int64_t)e.x - f.row0;
+        const uint32_t c = e.y & ~kBandFlag;
+        if (valid && !DL_CHECK(lr >= 0 && lr < f.rows && c < (unsigned)f.nS, 10, i)) valid = false;
+        const unsigned vm = __ballot_sync(0xffffffffu, valid);
+        const float s = warp_pairs_sq32(vm, f.Q + (valid ? (size_t)e.x * f.d : 0), f.S + (valid ? (size_t)c * f.d : 0), f.d);
+        if (valid) {   // a place in the row's list: one atomic per run of lanes with the same row
+            const unsigned peers = __match_any_sync(vm, e.x);
+            const int leader = __ffs(peers) - 1;
+            int at = 0;
+            if ((int)lane == leader) at = atomicAdd(f.cnt + lr, __popc(peers));
+            at = __shfl_sync(peers, at, leader) + __popc(peers & ((1u << lane) - 1u));
+            if (at < f.cap) {
+                f.col[(size_t)lr * f.cap + at] = c;
+                f.d32[(size_t)lr * f.cap + at] = s;
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ float upper32(const TopkRows &f, float s)
+{
+    return __fmul_ru(__fadd_ru(__fmul_ru(s, 1.0f + f.g32), f.abs32), 1.0f + f.slack);
+}
+__device__ __forceinline__ float lower32(const TopkRows &f, float s)
+{
+    return __fsub_rd(__fmul_rd(s, 1.0f - f.g32), f.abs32);
+}
+
+// Thresholds of another listing pass: an overflowed row's from the k-th smallest of the distances it
+// did list (at least k columns lie within its upper bound u, so a column with D > u (1 + slack) is not
+// in the top k: h < RD((||q||^2_dn - e2 (1 + 2 g64)) / 2) - E proves that, as in k_rowpar); every other
+// row lists nothing (its list stands). One CTA per row of the chunk.
+__global__ void __launch_bounds__(256) k_topk_refine(const TopkRows f, const double *__restrict__ nq64, int dp, double g64,
+                                                     int64_t rows_pad, const float4 *__restrict__ rowpar, float4 *__restrict__ thr)
+{
+    __shared__ unsigned s_cnt[2];
+    const int64_t lr = blockIdx.x;
+    const int64_t i = f.row0 + lr;
+    const float inf = __int_as_float(0x7f800000);
+    if (lr >= f.rows || f.cnt[lr] <= f.cap) {
+        if (threadIdx.x == 0 && lr < rows_pad) thr[i] = make_float4(inf, inf, 0.f, 0.f);
+        return;
+    }
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0u;
+    __syncthreads();
+    const int kk = f.row_k ? f.row_k[i] : f.k;   // at most k, and a list holds more than k
+    const float *v = f.d32 + (size_t)lr * f.cap;
+    unsigned kb = 0u;
+    int turn = 0;
+    for (int bit = 30; bit >= 0; --bit) {   // bits of the k-th smallest (non-negative floats order like them)
+        const unsigned t = kb | (1u << bit);
+        unsigned c = 0;
+        for (int a = threadIdx.x; a < f.cap; a += 256) c += __float_as_uint(v[a]) < t ? 1u : 0u;
+        if (cta_count(c, s_cnt, turn++) < (unsigned)kk) kb = t;
+    }
+    if (threadIdx.x == 0) {
+        const double e2 = (double)upper32(f, __uint_as_float(kb));
+        const double nq_dn = __dmul_rd(nq64[i], 1.0 - (double)(dp + 2) * 2.220446049250313e-16);
+        const double rej = __dsub_rd(nq_dn, __dmul_ru(e2, 1.0 + 2.0 * g64)) * 0.5;
+        const float4 rp = rowpar[i];
+        thr[i] = make_float4(inf, __fsub_rd(__double2float_rd(rej), rp.x), rp.z, rp.w);
+        f.cnt[lr] = 0;
+    }
+}
+
+// One warp per query row: the columns of its list that can still be in the top k, moved to the list's
+// front (their count becomes the row's) and named in the chunk's kept list. A row whose list
+// overflowed is named in over_rows instead.
+__global__ void __launch_bounds__(256) k_topk_keep(const TopkRows f, int *__restrict__ over_rows, unsigned long long *__restrict__ n_over)
+{
+    constexpr int kReg = 8;   // distances a lane keeps in registers
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = lanemask_lt();
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t lr = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; lr < f.rows; lr += nw) {
+        const int m0 = f.cnt[lr];
+        if (m0 > f.cap) {
+            if (lane == 0) over_rows[atomicAdd(n_over, 1ULL)] = (int)(f.row0 + lr);
+            continue;
+        }
+        const unsigned kk = (unsigned)(f.row_k ? f.row_k[f.row0 + lr] : f.k);
+        float *d32 = f.d32 + (size_t)lr * f.cap;
+        uint32_t *col = f.col + (size_t)lr * f.cap;
+        float lim = __int_as_float(0x7f800000);
+        if (m0 > (int)kk) {   // the k-th smallest distance's upper bound: at least k columns lie within it
+            unsigned v[kReg], lo = 0x7fffffffu, hi = 0u;
+#pragma unroll
+            for (int s = 0; s < kReg; ++s) {
+                v[s] = s * 32 + lane < m0 ? __float_as_uint(d32[s * 32 + lane]) : 0x7fffffffu;
+                lo = min(lo, v[s]);
+                if (v[s] != 0x7fffffffu) hi = max(hi, v[s]);
+            }
+            for (int a = kReg * 32 + lane; a < m0; a += 32) {
+                const unsigned w = __float_as_uint(d32[a]);
+                lo = min(lo, w);
+                hi = max(hi, w);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            unsigned kb = lo;   // the k-th smallest's bits: its prefix is lo's and hi's common one
+            if (kk > 1u && lo != hi) {
+                const int top = 31 - __clz((int)(lo ^ hi));
+                kb = hi & ~((2u << top) - 1u);
+                for (int bit = top; bit >= 0; --bit) {
+                    const unsigned t = kb | (1u << bit);
+                    unsigned c = 0;
+#pragma unroll
+                    for (int s = 0; s < kReg; ++s) c += v[s] < t ? 1u : 0u;
+                    for (int a = kReg * 32 + lane; a < m0; a += 32) c += __float_as_uint(d32[a]) < t ? 1u : 0u;
+                    if (__reduce_add_sync(0xffffffffu, c) < kk) kb = t;
+                }
+            }
+            lim = upper32(f, __uint_as_float(kb));
+        }
+        int m = 0;
+        for (int b = 0; b < m0; b += 32) {   // moved down in place: a window is read before it is written
+            const int a = b + lane;
+            const float w = a < m0 ? d32[a] : 0.f;
+            const uint32_t c = a < m0 ? col[a] : 0u;
+            const bool keep = a < m0 && lower32(f, w) <= lim;
+            const unsigned km = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                d32[m + __popc(km & lt)] = w;
+                col[m + __popc(km & lt)] = c;
+            }
+            __syncwarp();
+            m += __popc(km);
+        }
+        unsigned long long at = 0;
+        if (lane == 0) {
+            f.cnt[lr] = m;
+            if (m) at = atomicAdd(f.n_kept, (unsigned long long)m);
+        }
+        at = __shfl_sync(0xffffffffu, at, 0);
+        for (int a = lane; a < m; a += 32) f.kept[at + a] = (uint32_t)((size_t)lr * f.cap + a);
+    }
+}
+
+// The kept columns' canonical distances, up to 64 columns of any rows at a time: every thread forms
+// terms, a run of each column's, then a thread per column adds its own in ascending k. What bounds it:
+// the FP64 pipe, costed per warp instruction (16 cycles of an SM): three operations a term with every
+// lane busy, the conversions done by the integer units.
+__global__ void __launch_bounds__(128) k_topk_canon(const TopkRows f)
+{
+    __shared__ double sh_t[kTkTerms];
+    __shared__ const float *sh_q[kTkTermC], *sh_x[kTkTermC];
+    const int tid = threadIdx.x;
+    const unsigned long long n = *f.n_kept;
+    for (unsigned long long b0 = (unsigned long long)blockIdx.x * kTkTermC; b0 < n; b0 += (unsigned long long)gridDim.x * kTkTermC) {
+        const int na = (int)min((unsigned long long)kTkTermC, n - b0);
+        uint32_t slot = 0;
+        if (tid < na) {
+            slot = f.kept[b0 + tid];
+            const uint32_t c = f.col[slot];
+            sh_q[tid] = f.Q + (size_t)(f.row0 + slot / f.cap) * f.d;
+            sh_x[tid] = f.S + (size_t)(DL_CHECK(c < (unsigned)f.nS, 11, c) ? c : 0u) * f.d;
+        }
+        const int run = na > 32 ? 32 : na > 16 ? 64 : na > 8 ? 128 : 256;   // terms of a column staged at a time
+        const int sh = 31 - __clz(run), ld = run + 1;   // na * ld <= kTkTerms
+        double s = 0.0;
+        __syncthreads();
+        for (int k0 = 0; k0 < f.d; k0 += run) {
+            const int nk = min(run, f.d - k0);
+#pragma unroll 4
+            for (int e = tid; e < na << sh; e += 128) {
+                const int a = e >> sh, k = e & (run - 1);
+                if (k < nk) {
+                    const double t = __dsub_rn(widen(__ldg(sh_q[a] + k0 + k)), widen(__ldg(sh_x[a] + k0 + k)));
+                    sh_t[a * ld + k] = __dmul_rn(t, t);
+                }
+            }
+            __syncthreads();
+            if (tid < na)
+                for (int k = 0; k < nk; ++k) s = __dadd_rn(s, sh_t[tid * ld + k]);
+            __syncthreads();
+        }
+        if (tid < na) f.d64[slot] = s;
+    }
+}
+
+// One warp per query row: the exact rank of its kept columns by (canonical distance, caller's store
+// row) and its outputs.
+__global__ void __launch_bounds__(256) k_topk_out(const TopkRows f)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t lr = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; lr < f.rows; lr += nw) {
+        const int m = f.cnt[lr];
+        if (m > f.cap) continue;   // overflowed: solved elsewhere
+        const int64_t i = f.row0 + lr;
+        const int kk = f.row_k ? f.row_k[i] : f.k;
+        const double *d64 = f.d64 + (size_t)lr * f.cap;
+        const uint32_t *col = f.col + (size_t)lr * f.cap;
+        const int64_t base = f.row_off ? f.row_off[i] : (int64_t)f.q_orig[i] * f.k;
+        for (int a0 = 0; a0 < m; a0 += 32) {
+            const int a = a0 + lane;
+            const uint32_t ca = a < m ? col[a] : 0u;
+            const double da = a < m ? d64[a] : 0.0;
+            const int32_t oa = a < m ? f.s_orig[ca] : 0;
+            int rank = 0;
+            for (int b0 = 0; b0 < m; b0 += 32) {   // 32 others at a time, passed around the warp
+                const int bb = b0 + lane;
+                const uint32_t cb = bb < m ? col[bb] : 0u;
+                const double db = bb < m ? d64[bb] : 0.0;
+                const int32_t ob = bb < m ? f.s_orig[cb] : 0;
+                const int nb = min(32, m - b0);
+                for (int j = 0; j < nb; ++j) {
+                    const double dj = __shfl_sync(0xffffffffu, db, j);
+                    const int32_t oj = __shfl_sync(0xffffffffu, ob, j);
+                    // canonical distances are non-negative: they order like their bits
+                    rank += __double_as_longlong(dj) < __double_as_longlong(da) || (__double_as_longlong(dj) == __double_as_longlong(da) && oj < oa);
+                }
+            }
+            if (a < m && rank < kk) {
+                f.out_ids[base + rank] = f.s_ids[ca];
+                f.out_d2[base + rank] = da;
+            }
+        }
+        for (int t = m + lane; t < kk; t += 32) {
+            f.out_ids[base + t] = -1;
+            f.out_d2[base + t] = -1.0;
+        }
+    }
+}
 
 __device__ __forceinline__ double canon_d64(const float *__restrict__ q, const float *__restrict__ x, int d)
 {
@@ -69,213 +398,6 @@ __device__ __forceinline__ double canon_d64(const float *__restrict__ q, const f
         s = __dadd_rn(s, __dmul_rn(t, t));
     }
     return s;
-}
-
-__device__ __forceinline__ float seq_d32(const float *__restrict__ q, const float *__restrict__ x, int d)
-{
-    float s = 0.f;
-    for (int k = 0; k < d; ++k) {
-        const float t = __ldg(q + k) - __ldg(x + k);
-        s = fmaf(t, t, s);
-    }
-    return s;
-}
-
-// k-th largest of n floats (by order code), found by one warp with a 4-pass
-// radix select over 8-bit digits; -inf when n < k. hist: 256 words of shared memory.
-__device__ float warp_kth_largest(const float *__restrict__ vals, int n, int k, unsigned *hist)
-{
-    const unsigned lane = threadIdx.x & 31;
-    if (n < k) return __int_as_float(0xff800000);
-    unsigned prefix = 0u, mask = 0u;
-    unsigned rank = (unsigned)(k - 1);   // 0-based, counted from the largest
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int t = lane; t < 256; t += 32) hist[t] = 0u;
-        __syncwarp();
-        for (int i = lane; i < n; i += 32) {
-            const unsigned c = float_order_code(vals[i]);
-            if ((c & mask) == prefix) atomicAdd(&hist[(c >> shift) & 255u], 1u);
-        }
-        __syncwarp();
-        unsigned digit = 0u, r2 = 0u;
-        if (lane == 0) {
-            unsigned acc = 0u;
-            for (int dg = 255; dg >= 0; --dg) {
-                if (acc + hist[dg] > rank) {
-                    digit = (unsigned)dg;
-                    r2 = rank - acc;
-                    break;
-                }
-                acc += hist[dg];
-            }
-        }
-        digit = __shfl_sync(0xffffffffu, digit, 0);
-        rank = __shfl_sync(0xffffffffu, r2, 0);
-        prefix |= digit << shift;
-        mask |= 255u << shift;
-        __syncwarp();
-    }
-    return float_from_order_code(prefix);
-}
-
-__global__ void __launch_bounds__(128) k_topk_finalize(const TopkFin f)
-{
-    __shared__ unsigned s_hist[4][256];
-    __shared__ uint32_t s_col[4][kTkMax];
-    __shared__ float s_u[4][kTkMax];
-    __shared__ float s_l[4][kTkMax];
-    __shared__ double s_d[4][kTkMax];
-    __shared__ float s_kth[4];
-    __shared__ int s_prow[4][kTkPend];       // queued columns: query row,
-    __shared__ uint32_t s_pcol[4][kTkPend];  // store row
-    __shared__ int2 s_pseg[4][kTkPendRows];  // queued rows: {query row, first entry | count << 16}
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned lt = lanemask_lt();
-    uint32_t *col = s_col[w];
-    float *su = s_u[w], *sl = s_l[w];
-    double *sd = s_d[w];
-    int np = 0, ns = 0;   // queued columns and rows of this warp (warp-uniform)
-    // The queued columns' canonical distances (one per lane), then each queued row's exact rank
-    // by (D64, caller's store row) and its outputs. Uses sd as scratch.
-    auto flush = [&]() {
-        for (int e = lane; e < np; e += 32)
-            sd[e] = canon_d64(f.Q + (size_t)s_prow[w][e] * f.d, f.S + (size_t)s_pcol[w][e] * f.d, f.d);
-        __syncwarp();
-        for (int g = 0; g < ns; ++g) {
-            const int2 sg = s_pseg[w][g];
-            const int i = sg.x, e0 = sg.y & 0xffff, n = sg.y >> 16;
-            const int kk = f.row_k ? f.row_k[i] : f.k;
-            const int64_t base = f.row_off ? f.row_off[i] : (int64_t)f.q_orig[i] * f.k;
-            for (int a = lane; a < n; a += 32) {
-                const double da = sd[e0 + a];
-                const uint32_t ca = s_pcol[w][e0 + a];
-                const int32_t oa = f.s_orig[ca];
-                int rank = 0;
-                for (int b = 0; b < n; ++b) {
-                    const double db = sd[e0 + b];
-                    rank += (db < da) || (db == da && f.s_orig[s_pcol[w][e0 + b]] < oa);
-                }
-                if (rank < kk) {
-                    f.out_ids[base + rank] = f.s_ids[ca];
-                    f.out_d2[base + rank] = da;
-                }
-            }
-            for (int t = n + lane; t < kk; t += 32) {
-                f.out_ids[base + t] = -1;
-                f.out_d2[base + t] = -1.0;
-            }
-        }
-        __syncwarp();
-        np = 0;
-        ns = 0;
-    };
-    for (int i = blockIdx.x * 4 + w; i < f.nQ; i += gridDim.x * 4) {
-        if (f.overflow[i]) continue;
-        // the row's k-th largest lower bound over all slots' heaps (the heaps hold each
-        // slot's k largest): every top-k column has U >= it
-        const int kk0 = f.row_k ? f.row_k[i] : f.k;
-        float th = warp_kth_largest(f.heap + (size_t)i * f.slots * f.k, f.slots * f.k, kk0, s_hist[w]);
-        for (int s = lane; s < f.slots; s += 32) th = fmaxf(th, f.theta[(size_t)i * f.slots + s]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) th = fmaxf(th, __shfl_xor_sync(0xffffffffu, th, o));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) th = fmaxf(th, __shfl_xor_sync(0xffffffffu, th, o));
-        int m = 0;
-        for (int s = 0; s < f.slots; ++s) {
-            const size_t si = (size_t)i * f.slots + s;
-            const int cs = f.cnt[si];
-            const uint2 *L = f.list + si * (size_t)f.cap;
-            for (int b = 0; b < cs; b += 32) {
-                const int idx = b + lane;
-                uint2 e = make_uint2(0u, 0u);
-                if (idx < cs) e = L[idx];
-                const bool keep = idx < cs && __uint_as_float(e.y) >= th;
-                const unsigned bm = __ballot_sync(0xffffffffu, keep);
-                const int pos = m + __popc(bm & lt);
-                if (keep && pos < kTkMax) col[pos] = DL_CHECK(e.x < (unsigned)f.nS, 10, e.x) ? e.x : 0u;
-                m += __popc(bm);
-            }
-        }
-        if (m > kTkMax) {   // too many candidates for this buffer: exact fallback
-            if (lane == 0) f.overflow[i] = 1;
-            continue;
-        }
-        __syncwarp();
-        const float *q = f.Q + (size_t)i * f.d;
-        for (int a = lane; a < m; a += 32) {
-            const float d32 = seq_d32(q, f.S + (size_t)col[a] * f.d, f.d);
-            su[a] = __fadd_ru(__fmul_ru(d32, 1.0f + f.g32), f.abs32);
-            sl[a] = __fsub_rd(__fmul_rd(d32, 1.0f - f.g32), f.abs32);
-        }
-        __syncwarp();
-        // k-th smallest upper bound (ties broken by position) -> at least k columns have D <= kth
-        if (lane == 0) s_kth[w] = __int_as_float(0x7f800000);
-        __syncwarp();
-        const int kk = f.row_k ? f.row_k[i] : f.k;
-        if (m > kk) {
-            for (int a = lane; a < m; a += 32) {
-                int rank = 0;
-                const float ua = su[a];
-                for (int b = 0; b < m; ++b) rank += (su[b] < ua) || (su[b] == ua && b < a);
-                if (rank == kk - 1) s_kth[w] = ua;
-            }
-        }
-        __syncwarp();
-        const float kth = __fmul_ru(s_kth[w], 1.0f + f.slack);
-        // the columns that can still be in the top k: each needs its canonical distance
-        int kept = 0;
-        for (int a0 = 0; a0 < m; a0 += 32) kept += __popc(__ballot_sync(0xffffffffu, a0 + lane < m && sl[a0 + lane] <= kth));
-        if (lane == 0 && kept) atomicAdd(f.n_fp64, (unsigned long long)kept);
-        if (kept <= kTkPendRow) {   // queue them with other rows' columns
-            if (np + kept > kTkPend || ns == kTkPendRows) flush();
-            int pos = np;
-            for (int a0 = 0; a0 < m; a0 += 32) {
-                const int a = a0 + lane;
-                const bool keep = a < m && sl[a] <= kth;
-                const unsigned bm = __ballot_sync(0xffffffffu, keep);
-                if (keep) {
-                    s_prow[w][pos + __popc(bm & lt)] = i;
-                    s_pcol[w][pos + __popc(bm & lt)] = col[a];
-                }
-                pos += __popc(bm);
-            }
-            if (lane == 0) s_pseg[w][ns] = make_int2(i, np | (kept << 16));
-            np += kept;
-            ++ns;
-            __syncwarp();
-            continue;
-        }
-        flush();   // sd is this row's now
-        for (int a0 = 0; a0 < m; a0 += 32) {
-            const int a = a0 + lane;
-            const bool keep = a < m && sl[a] <= kth;
-            if (a < m) sd[a] = keep ? canon_d64(q, f.S + (size_t)col[a] * f.d, f.d) : __longlong_as_double(0x7ff0000000000000LL);
-        }
-        __syncwarp();
-        const int64_t base = f.row_off ? f.row_off[i] : (int64_t)f.q_orig[i] * f.k;
-        int64_t *oid = f.out_ids + base;
-        double *od = f.out_d2 + base;
-        for (int a = lane; a < m; a += 32) {
-            const double da = sd[a];
-            if (!(da < __longlong_as_double(0x7ff0000000000000LL))) continue;   // not kept
-            const int32_t oa = f.s_orig[col[a]];
-            int rank = 0;
-            for (int b = 0; b < m; ++b) {
-                const double db = sd[b];
-                rank += (db < da) || (db == da && f.s_orig[col[b]] < oa);
-            }
-            if (rank < kk) {
-                oid[rank] = f.s_ids[col[a]];
-                od[rank] = da;
-            }
-        }
-        for (int t = kept + lane; t < kk; t += 32) {
-            oid[t] = -1;
-            od[t] = -1.0;
-        }
-        __syncwarp();
-    }
-    flush();
 }
 
 struct TopkFb {
@@ -402,70 +524,47 @@ __global__ void __launch_bounds__(256) k_topk_fallback(const TopkFb f)
     }
 }
 
-// Per query row: {canonical slack of h, unused, ||q - q~|| up, ||q~|| up}; padding rows get zeros.
-__global__ void __launch_bounds__(256) k_rowpar_topk(const double *__restrict__ nq64, const float4 *__restrict__ rowb,
-                                                     int64_t n, int64_t n_tot, double g64, double nq_max_s,
-                                                     float4 *__restrict__ rowpar, unsigned *__restrict__ row_theta)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_tot) return;
-    row_theta[i] = float_order_code(__int_as_float(0xff800000));   // -inf
-    if (i >= n) {
-        rowpar[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
-    }
-    // |h_canonical - h| <= |D64 - D| / 2 <= g64 * (||q||^2 + ||x||^2); doubled for margin
-    const double delta = 2.0 * g64 * (nq64[i] + nq_max_s) * 1.0001 + 1e-30;
-    const float4 rb = rowb[i];
-    rowpar[i] = make_float4(__double2float_ru(delta), 0.f, rb.x, rb.y);
-}
-
-__global__ void k_collect_overflow(const int *__restrict__ overflow, int n, int *__restrict__ rows,
-                                   int *__restrict__ count)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && overflow[i]) rows[atomicAdd(count, 1)] = i;
-}
-
-// ------------------------------------------------------------------ units with S splits
-static std::mutex g_tku_mu;
-static std::map<std::tuple<int, int64_t, int64_t, int, int>, std::pair<int4 *, int>> g_tku;
-
-static int topk_units(int64_t nQ, int64_t nS, int BN, int splits, const int4 **d_units, int *n_units)
-{
-    int dev = 0;
-    cudaGetDevice(&dev);
-    auto key = std::make_tuple(dev, nQ, nS, BN, splits);
-    std::lock_guard<std::mutex> lk(g_tku_mu);
-    auto it = g_tku.find(key);
-    if (it == g_tku.end()) {
-        const int mt = (int)((nQ + 127) / 128), nt = (int)((nS + BN - 1) / BN);
-        std::vector<int4> v;
-        // split-major: the CTAs running together walk the same S range (shared through L2),
-        // and later splits of a row start from the threshold its earlier splits published
-        for (int s = 0; s < splits; ++s)
-            for (int m = 0; m < mt; ++m) {
-                const int nb = (int)((int64_t)nt * s / splits), ne = (int)((int64_t)nt * (s + 1) / splits);
-                if (ne > nb) v.push_back(make_int4(m, nb, ne, s));
-            }
-        int4 *d = nullptr;
-        if (!v.empty()) {
-            cudaError_t e = cudaMalloc(&d, v.size() * sizeof(int4));
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(topk units)");
-            e = cudaMemcpy(d, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(topk units)");
-        }
-        it = g_tku.emplace(key, std::make_pair(d, (int)v.size())).first;
-    }
-    *d_units = it->second.first;
-    *n_units = it->second.second;
-    return DL_OK;
-}
-
+// ------------------------------------------------------------------ host side
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Every how many-th tile the first pass takes. That pass costs 2 d nS / f operations a row, and about
+// k f columns of a row are listed at some 0.2 ns each (a slow-path visit and an 8 d byte recheck):
+// the sum is least at f = sqrt(d nS / (1.6e5 k)). At most 16 (a row's list grows with f), and at
+// least 8 k groups of 16 columns stay.
+static int topk_stride(int64_t nS, int dp, int k)
+{
+    const double f = std::sqrt((double)nS * dp / (1.6e5 * k));
+    return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)std::min(f, 16.0), nS / (128LL * k)));
+}
+
+struct TopkShape {
+    int stride;         // tiles of the first pass
+    int cap;            // list capacity of a row
+    int gran;           // columns of a group
+    int n_groups;       // groups of a row (0: every column fits the list, no first pass)
+    int64_t per_cand;   // candidates of a row provided for
+    int64_t bytes() const { return 4LL * n_groups + 20LL * cap + 4 + 8 * per_cand; }
+};
+
+static TopkShape topk_shape(int64_t nS, int dp, int k, int BN)
+{
+    TopkShape s;
+    s.stride = topk_stride(nS, dp, k);
+    // the k-th best of every f-th tile is about the k f-th of the store, with a spread of f sqrt(k)
+    // (at k = 1 geometric: a row in 10^11 has more than 24 f columns above it)
+    s.cap = (2 * k * s.stride + 16 * s.stride + 128 + 31) / 32 * 32;
+    const int64_t nt_sub = ((nS + BN - 1) / BN + s.stride - 1) / s.stride;
+    s.gran = nt_sub * BN / 64 >= 8LL * k ? 64 : 16;
+    const bool all = nS <= s.cap;
+    s.n_groups = all ? 0 : (int)(nt_sub * BN / s.gran);
+    s.per_cand = all ? nS : std::min<int64_t>(nS, (int64_t)k * s.stride * 3 / 2 + 16LL * s.stride + 64);
+    return s;
+}
+
+int64_t topk_row_bytes(int64_t nS, int dp, int k) { return topk_shape(nS, dp, k, 256).bytes(); }
+
 // Top-k of every row of Q against S into out_ids / out_d2. k is the largest k of
-// any row (the heap size); row_k (device, optional) gives each row's own k and
+// any row; row_k (device, optional) gives each row's own k and
 // row_off (device, optional) each row's first output slot (default: caller row * k).
 int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, const int64_t *row_off,
               int64_t *out_ids, double *out_d2, const dl_join_opts &o, cudaStream_t st, dl_join_stats *stats)
@@ -493,238 +592,277 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     int code = (o.tile_n ? o.tile_n : 256) | (o.epilogue_warps == 16 ? kTuneWide : 0);
     if (use_tc && o.tile_n == 0 && o.epilogue_warps == 0) code = tune_pick(Q->dp, kTuneTopk, nQ, nS, &tune_trial);
     const int BN = tune_bn(code);
-    const bool wide = use_tc && tune_wide(code);   // 16 epilogue warps: slots per (row, split, quarter)
+    const bool wide = use_tc && tune_wide(code);   // 16 epilogue warps
     const int sms = device_sm_count();
-    const int64_t mt = (nQ + 127) / 128, nt = (nS + BN - 1) / BN;
-    int splits = 1;
-    if (mt > 0) splits = (int)std::min<int64_t>(std::max<int64_t>(1, (2 * sms + mt - 1) / mt), std::min<int64_t>(nt, 16));
-    if (splits < 1) splits = 1;
-    const int slots = (wide ? 4 : 2) * splits;
-    const int cap = std::max(64, (4 * k + 31) / 32 * 32);
-    const int64_t rows = mt * 128;
+    const int64_t mt = (nQ + 127) / 128, rows = mt * 128;
+    const int64_t nt = (nS + BN - 1) / BN;
 
-    const size_t b_rowpar = al256(rows * sizeof(float4)), b_heap = al256((size_t)rows * slots * k * sizeof(float)),
-                 b_list = al256((size_t)rows * slots * cap * sizeof(uint2)),
-                 b_cnt = al256((size_t)rows * slots * sizeof(int)), b_theta = al256((size_t)rows * slots * sizeof(float)),
-                 b_rth = al256((size_t)std::max<int64_t>(rows, 1) * sizeof(unsigned)),
-                 b_ovf = al256((size_t)std::max<int64_t>(nQ, 1) * sizeof(int)),
-                 b_rows = al256((size_t)std::max<int64_t>(nQ, 1) * sizeof(int)), b_misc = 256;
+    // the two passes' shape, and query rows per chunk so that its workspace stays near 1 GB
+    const TopkShape sh = topk_shape(nS, Q->dp, k, BN);
+    const int f = sh.stride, cap = sh.cap, gran = sh.gran, n_groups = sh.n_groups;
+    const int64_t nt_sub = (nt + f - 1) / f, per_cand = sh.per_cand;
+    const bool all = n_groups == 0;   // every column fits a row's list: no first pass
+    const int64_t per_row = sh.bytes();
+    const int64_t chunk_rows =
+        use_tc ? std::min<int64_t>(rows, std::max<int64_t>(1, (1LL << 30) / (per_row * 128)) * 128) : rows;
+
+    const size_t b_rowpar = al256((size_t)rows * sizeof(float4)), b_frows = al256((size_t)std::max<int64_t>(nQ, 1) * sizeof(int));
     const bool timing = o.timing || tune_trial;
-    void *ws = nullptr;
-    int rc = dev_alloc(&ws, b_rowpar + b_heap + b_list + b_cnt + b_theta + b_rth + b_ovf + b_rows + b_misc, st);
+    void *ws = nullptr, *cws = nullptr;
+    int rc = dev_alloc(&ws, 2 * b_rowpar + b_frows + 256, st);
     if (rc) return rc;
-    char *pw = (char *)ws;
-    float4 *rowpar = (float4 *)pw;
-    pw += b_rowpar;
-    float *heap = (float *)pw;
-    pw += b_heap;
-    uint2 *list = (uint2 *)pw;
-    pw += b_list;
-    int *cnt = (int *)pw;
-    pw += b_cnt;
-    float *theta = (float *)pw;
-    pw += b_theta;
-    unsigned *row_theta = (unsigned *)pw;
-    pw += b_rth;
-    int *ovf = (int *)pw;
-    pw += b_ovf;
-    int *frows = (int *)pw;
-    pw += b_rows;
-    unsigned long long *misc = (unsigned long long *)pw;   // [0] flagged rows [1] fp64 evals [2] err [3] tc err
+    float4 *rowpar = (float4 *)ws, *thr = (float4 *)((char *)ws + b_rowpar);
+    int *frows = (int *)((char *)ws + 2 * b_rowpar);
+    // [0] rows named in frows [1] fp64 evals [2] more near-ties than the fallback ranks [3] wait expired
+    // [4] candidates of a pass [5] columns kept by it
+    unsigned long long *misc = (unsigned long long *)((char *)ws + 2 * b_rowpar + b_frows);
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     if (timing)
         for (auto &e : ev) cudaEventCreate(&e);
     auto done = [&](int code) {
         for (auto &e : ev)
             if (e) cudaEventDestroy(e);
+        dev_free(cws, st);
         dev_free(ws, st);
         if (code) cudaStreamSynchronize(st);
         return code;
     };
+    unsigned long long *h = nullptr;
+    rc = pinned_counters(&h);
+    if (rc) return done(rc);
+    std::memset(h, 0, 48);
     cudaError_t e = cudaMemsetAsync(misc, 0, 256, st);
-    if (e == cudaSuccess && nQ > 0) e = cudaMemsetAsync(ovf, 0, (size_t)nQ * sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, b_cnt, st);
     if (e != cudaSuccess) return done(cuda_fail(e, "top-k memset"));
     if (timing) cudaEventRecord(ev[0], st);
     int launches = 0;
+    auto launched = [&](const char *what) {
+        count_launch();
+        ++launches;
+        const cudaError_t le = cudaGetLastError();
+        return le == cudaSuccess ? DL_OK : cuda_fail(le, what);
+    };
+    auto reset = [&]() {   // a pass's counters
+        cudaError_t re = cudaMemsetAsync(misc, 0, 8, st);
+        if (re == cudaSuccess) re = cudaMemsetAsync(misc + 4, 0, 16, st);
+        return re == cudaSuccess ? DL_OK : cuda_fail(re, "top-k memset");
+    };
+    auto read_misc = [&]() {
+        cudaError_t re = cudaMemcpyAsync(h, misc, 48, cudaMemcpyDeviceToHost, st);
+        if (re == cudaSuccess) re = cudaStreamSynchronize(st);
+        return re == cudaSuccess ? DL_OK : cuda_fail(re, "top-k");
+    };
     const double g64 = gamma64(d), g32 = gamma32(d);
-    TopkFin f;
-    f.Q = Q->x32;
-    f.S = S->x32;
-    f.d = d;
-    f.nQ = (int)nQ;
-    f.nS = (int)nS;
-    f.k = k;
-    f.slots = slots;
-    f.cap = cap;
-    f.theta = theta;
-    f.heap = heap;
-    f.row_theta = row_theta;
-    f.cnt = cnt;
-    f.list = list;
-    f.overflow = ovf;
-    f.q_orig = Q->orig;
-    f.s_orig = S->orig;
-    f.s_ids = S->ids;
-    f.out_ids = out_ids;
-    f.out_d2 = out_d2;
-    f.row_k = row_k;
-    f.row_off = row_off;
-    f.g32 = f32_ru(g32 * 1.0000001);
-    f.abs32 = f32_ru((double)(d + 8) * 1.401298464324817e-45 * 4.0);
-    f.slack = f32_ru(4.0 * g64 + 1e-12);
-    f.n_fp64 = misc + 1;
-    if (nQ > 0 && nS > 0) {
-        if (use_tc) {
-            Half *hQ = nullptr, *hS = nullptr;
+    TopkRows t{};
+    t.Q = Q->x32;
+    t.S = S->x32;
+    t.d = d;
+    t.nS = (int)nS;
+    t.k = k;
+    t.cap = cap;
+    t.q_orig = Q->orig;
+    t.s_orig = S->orig;
+    t.s_ids = S->ids;
+    t.out_ids = out_ids;
+    t.out_d2 = out_d2;
+    t.row_k = row_k;
+    t.row_off = row_off;
+    t.g32 = f32_ru(g32 * 1.0000001);
+    t.abs32 = f32_ru((double)(d + 8) * 1.401298464324817e-45 * 4.0);
+    t.slack = f32_ru(4.0 * g64 + 1e-12);
+    t.n_kept = misc + 5;
+    int64_t flagged = 0;   // rows named in frows for the exact scan
+    int64_t fp64 = 0;      // canonical distances of the other rows
+    if (nQ > 0 && (nS == 0 || use_tc)) {
+        Half *hQ = nullptr, *hS = nullptr;
+        const CUtensorMap *tmA = nullptr, *tmB = nullptr;
+        if (nS > 0) {
             rc = get_half(const_cast<dl_store *>(Q), fmt, st, &hQ);
             if (!rc) rc = get_half(const_cast<dl_store *>(S), fmt, st, &hS);
-            if (!rc) {
-                k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, hQ->rowb, nQ, rows, g64,
-                                                                              (double)S->nq_max * 1.0001, rowpar, row_theta);
-                count_launch();
-                ++launches;
-            }
-            const CUtensorMap *tmA = nullptr, *tmB = nullptr;
             if (!rc) rc = get_tmap(const_cast<dl_store *>(Q), hQ, 128, &tmA);
             if (!rc) rc = get_tmap(const_cast<dl_store *>(S), hS, BN, &tmB);
-            const int4 *units = nullptr;
-            int n_units = 0;
-            if (!rc) rc = topk_units(nQ, nS, BN, splits, &units, &n_units);
-            if (!rc && n_units > 0) {
+            if (!rc) {
+                k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, hQ->rowb, nQ, rows, g64,
+                                                                              (double)S->nq_max * 1.0001, rowpar);
+                rc = launched("k_rowpar_topk launch");
+            }
+        }
+        int64_t cand_cap = std::min<int64_t>(chunk_rows, nQ) * per_cand + 65536;
+        const size_t b_g = al256((size_t)chunk_rows * n_groups * 4), b_l = al256((size_t)chunk_rows * cap * 4),
+                     b_n = al256((size_t)chunk_rows * 4), b_d = al256((size_t)chunk_rows * cap * 8);
+        for (int64_t row0 = 0; row0 < nQ && !rc; row0 += chunk_rows) {
+            const int64_t cr = std::min(chunk_rows, nQ - row0), cr_pad = (cr + 127) / 128 * 128;
+            for (int pass = 0, again = 0, grown = 0; !rc; ++pass) {   // listing passes over this chunk
+                if (!cws) {
+                    rc = dev_alloc(&cws, b_g + 3 * b_l + b_n + b_d + (size_t)cand_cap * 8, st);
+                    if (rc) break;
+                }
+                float *gmax = (float *)cws;
+                t.col = (uint32_t *)((char *)cws + b_g);
+                t.d32 = (float *)((char *)cws + b_g + b_l);
+                t.kept = (uint32_t *)((char *)cws + b_g + 2 * b_l);
+                t.cnt = (int *)((char *)cws + b_g + 3 * b_l);
+                t.d64 = (double *)((char *)cws + b_g + 3 * b_l + b_n);
+                uint2 *cand = (uint2 *)((char *)cws + b_g + 3 * b_l + b_n + b_d);
+                t.row0 = row0;
+                t.rows = cr;
                 TcLaunch L;
                 std::memset(&L.p, 0, sizeof L.p);
-                L.tmA = tmA;
-                L.tmB = tmB;
-                L.BN = BN;
-                L.grid = std::min(n_units, sms);
-                L.p.units = units;
-                L.p.n_units = n_units;
-                L.p.nR = (int)nQ;
-                L.p.nS = (int)nS;
-                L.p.kc = Q->dp / 64;
-                L.p.fmt = fmt == kHalfBF16;
-                L.p.scale = hQ->scale * hS->scale;
-                tc_plan(BN, Q->dp / 64, &L.p.stages, &L.p.a_slots, false, false, wide);
-                L.wide = wide;
-                L.p.upper = 0;
-                L.p.rowpar = rowpar;
-                L.p.beta = S->beta;
-                L.p.cstat = hS->cstat;
-                L.p.err = (int *)(misc + 3);
-                L.p.tk_k = k;
-                L.p.tk_cap = cap;
-                L.p.tk_slots = slots;
-                L.p.tk_heap = heap;
-                L.p.tk_list = list;
-                L.p.tk_cnt = cnt;
-                L.p.tk_theta = theta;
-                L.p.tk_row_theta = row_theta;
-                L.p.tk_overflow = ovf;
-                // Units are split-major, so the first mt units are every row tile's first split.
-                // Running those alone first publishes each row's threshold before the other
-                // splits start: their slots then admit only columns that can still reach the
-                // top k (fewer list entries and heap inserts, most visibly for large k).
-                // (only when the first splits alone still fill most of the GPU)
-                const int first = (splits > 1 && n_units > mt && 2 * mt >= sms) ? (int)mt : n_units;
-                L.p.n_units = first;
-                L.grid = std::min(first, sms);
-                rc = launch_tc_join(L, st, true);
-                ++launches;
-                if (!rc && first < n_units) {
-                    L.p.units = units + first;
-                    L.p.n_units = n_units - first;
-                    L.grid = std::min(n_units - first, sms);
-                    rc = launch_tc_join(L, st, true);
-                    ++launches;
+                if (nS > 0) {
+                    L.tmA = tmA;
+                    L.tmB = tmB;
+                    L.BN = BN;
+                    L.wide = wide;
+                    L.p.nR = (int)nQ;
+                    L.p.nS = (int)nS;
+                    L.p.kc = Q->dp / 64;
+                    L.p.fmt = fmt == kHalfBF16;
+                    L.p.scale = hQ->scale * hS->scale;
+                    tc_plan(BN, Q->dp / 64, &L.p.stages, &L.p.a_slots, false, false, wide);
+                    L.p.beta = S->beta;
+                    L.p.cstat = hS->cstat;
+                    L.p.err = (int *)(misc + 3);
+                    L.p.m0 = (int)(row0 / 128);
                 }
+                if (pass == 0) {   // thresholds from the first pass's group maxima
+                    if (nS > 0 && !all) {
+                        L.p.rowpar = rowpar;
+                        L.p.tile_stride = f;
+                        L.p.gmax = gmax;
+                        L.p.n_groups = n_groups;
+                        L.p.gran = gran;
+                        L.p.row0 = (int)row0;
+                        tc_grid_units(&L, cr_pad / 128, nt_sub, sms);
+                        rc = launch_tc_join(L, st, kModeMaxima);
+                        ++launches;
+                        L.p.tile_stride = 1;
+                    }
+                    if (!rc && nS > 0) {
+                        k_topk_theta<<<(unsigned)(cr_pad / 8), 256, 0, st>>>(rowpar, gmax, n_groups, row0, nQ, row0 + cr_pad, k, row_k, thr);
+                        rc = launched("k_topk_theta launch");
+                    }
+                    if (!rc) {
+                        e = cudaMemsetAsync(t.cnt, 0, b_n, st);
+                        if (e != cudaSuccess) rc = cuda_fail(e, "top-k memset");
+                    }
+                } else if (again) {   // tighter thresholds for the rows whose list overflowed
+                    k_topk_refine<<<(unsigned)cr_pad, 256, 0, st>>>(t, Q->nq64, Q->dp, g64, cr_pad, rowpar, thr);
+                    rc = launched("k_topk_refine launch");
+                    if (!rc) {
+                        rc = reset();
+                    }
+                }
+                if (!rc && nS > 0) {
+                    L.p.rowpar = thr;
+                    L.p.cand = cand;
+                    L.p.cand_cnt = misc + 4;
+                    L.p.cand_cap = (unsigned long long)cand_cap;
+                    tc_plan(BN, Q->dp / 64, &L.p.stages, &L.p.a_slots, false, false, wide, true);
+                    tc_grid_units(&L, cr_pad / 128, nt, sms);
+                    rc = launch_tc_join(L, st);
+                    ++launches;
+                    if (!rc) {
+                        const int64_t grid = std::min<int64_t>((cand_cap + 255) / 256, (int64_t)sms * 8);
+                        k_topk_dist<<<(unsigned)grid, 256, 0, st>>>(t, cand, misc + 4, (unsigned long long)cand_cap);
+                        rc = launched("k_topk_dist launch");
+                    }
+                }
+                if (!rc) {
+                    const unsigned gw = (unsigned)std::min<int64_t>((cr + 7) / 8, (int64_t)sms * 32);   // a warp a row
+                    k_topk_keep<<<gw, 256, 0, st>>>(t, frows + flagged, misc);
+                    rc = launched("k_topk_keep launch");
+                    if (!rc && nS > 0) {
+                        k_topk_canon<<<(unsigned)std::min<int64_t>((cr * cap + kTkTermC - 1) / kTkTermC, (int64_t)sms * 12), 128, 0, st>>>(t);
+                        rc = launched("k_topk_canon launch");
+                    }
+                    if (!rc) {
+                        k_topk_out<<<gw, 256, 0, st>>>(t);
+                        rc = launched("k_topk_out launch");
+                    }
+                }
+                if (timing && row0 + chunk_rows >= nQ && pass == 0) cudaEventRecord(ev[1], st);
+                if (!rc) rc = read_misc();
+                if (rc) break;
+                if (h[3]) {
+                    set_error("top-k: a bounded device wait expired");
+                    return done(DL_ETIMEOUT);
+                }
+                if (h[4] > (unsigned long long)cand_cap) {   // the candidate list was too short: its exact size, again
+                    cand_cap = (int64_t)h[4] + (int64_t)(h[4] / 8) + 1024;
+                    dev_free(cws, st);
+                    cws = nullptr;
+                    if (++grown > 4) {
+                        set_error("top-k: the candidate list keeps overflowing");
+                        return done(DL_ENOMEM);
+                    }
+                    pass = -1;
+                    again = 0;
+                    rc = reset();
+                    continue;
+                }
+                if (h[0] == 0 || again == kTkRefines) {
+                    flagged += (int64_t)h[0];
+                    fp64 += (int64_t)h[5];
+                    break;
+                }
+                ++again;
             }
-            if (!rc) {
-                const int grid = (int)std::min<int64_t>((nQ + 3) / 4, (int64_t)sms * 16);
-                k_topk_finalize<<<grid, 128, 0, st>>>(f);
+            if (!rc && row0 + chunk_rows < nQ) {   // this chunk's named rows stay; its counters start over
+                rc = reset();
+            }
+        }
+    } else if (nQ > 0) {   // no tensor-core pass for this shape: every row takes the exact scan
+        std::vector<int> every((size_t)nQ);
+        for (int64_t i = 0; i < nQ; ++i) every[(size_t)i] = (int)i;
+        e = cudaMemcpyAsync(frows, every.data(), (size_t)nQ * sizeof(int), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) rc = cuda_fail(e, "top-k rows");
+        flagged = nQ;
+        if (timing) cudaEventRecord(ev[1], st);
+    }
+    // exact scan of the named rows
+    if (!rc && flagged > 0) {
+        const int64_t per_row = (int64_t)nS * 8 + (int64_t)kTkFallbackCap * 12;
+        const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(flagged, (256LL << 20) / per_row));
+        void *fb = nullptr;
+        rc = dev_alloc(&fb, al256(batch * (size_t)nS * 8) + al256(batch * (size_t)kTkFallbackCap * 12), st);
+        if (!rc) {
+            TopkFb g;
+            g.Q = Q->x32;
+            g.S = S->x32;
+            g.d = d;
+            g.nS = (int)nS;
+            g.k = k;
+            g.scr_u = (float *)fb;
+            g.scr_l = g.scr_u + batch * nS;
+            g.scr_c = (uint32_t *)((char *)fb + al256(batch * (size_t)nS * 8));
+            g.scr_d = (double *)(g.scr_c + batch * kTkFallbackCap);
+            g.q_orig = Q->orig;
+            g.s_orig = S->orig;
+            g.s_ids = S->ids;
+            g.out_ids = out_ids;
+            g.out_d2 = out_d2;
+            g.row_k = row_k;
+            g.row_off = row_off;
+            g.g32 = t.g32;
+            g.abs32 = t.abs32;
+            g.slack = t.slack;
+            g.err = (int *)(misc + 2);
+            g.n_fp64 = misc + 1;
+            for (int64_t b0 = 0; b0 < flagged && !rc; b0 += batch) {
+                g.rows = frows + b0;
+                g.n_rows = (int)std::min<int64_t>(batch, flagged - b0);
+                k_topk_fallback<<<g.n_rows, 256, 0, st>>>(g);
                 count_launch();
                 ++launches;
                 e = cudaGetLastError();
-                if (e != cudaSuccess) rc = cuda_fail(e, "k_topk_finalize launch");
+                if (e != cudaSuccess) rc = cuda_fail(e, "k_topk_fallback launch");
             }
-        } else {
-            // no tensor-core pass for this shape: every row takes the exact scan
-            e = cudaMemsetAsync(ovf, 0xff, (size_t)nQ * sizeof(int), st);
-            if (e != cudaSuccess) rc = cuda_fail(e, "top-k memset");
-        }
-    } else if (nQ > 0) {   // empty store: every slot is unused
-        k_rowpar_topk<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Q->nq64, Q->h.rowb, nQ, rows, g64, 0.0, rowpar,
-                                                                      row_theta);
-        k_topk_finalize<<<1, 128, 0, st>>>(f);   // no candidates for any row -> fills -1
-        count_launch();
-        count_launch();
-        ++launches;
-    }
-    if (timing) cudaEventRecord(ev[1], st);
-    // exact fallback for flagged rows
-    int64_t flagged = 0;
-    if (!rc && nQ > 0 && nS > 0) {
-        k_collect_overflow<<<(unsigned)((nQ + 255) / 256), 256, 0, st>>>(ovf, (int)nQ, frows, (int *)misc);
-        count_launch();
-        ++launches;
-        unsigned long long h[4] = {0, 0, 0, 0};
-        e = cudaMemcpyAsync(h, misc, sizeof h, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = cuda_fail(e, "top-k");
-        if (!rc && h[3]) {
-            set_error("top-k: a bounded device wait expired");
-            return done(DL_ETIMEOUT);
-        }
-        flagged = (int64_t)(h[0] & 0xffffffffULL);
-        if (!rc && flagged > 0) {
-            const int64_t per_row = (int64_t)nS * 8 + (int64_t)kTkFallbackCap * 12;
-            const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(flagged, (256LL << 20) / per_row));
-            void *fb = nullptr;
-            rc = dev_alloc(&fb, al256(batch * (size_t)nS * 8) + al256(batch * (size_t)kTkFallbackCap * 12), st);
-            if (!rc) {
-                TopkFb g;
-                g.Q = Q->x32;
-                g.S = S->x32;
-                g.d = d;
-                g.nS = (int)nS;
-                g.k = k;
-                g.scr_u = (float *)fb;
-                g.scr_l = g.scr_u + batch * nS;
-                g.scr_c = (uint32_t *)((char *)fb + al256(batch * (size_t)nS * 8));
-                g.scr_d = (double *)(g.scr_c + batch * kTkFallbackCap);
-                g.q_orig = Q->orig;
-                g.s_orig = S->orig;
-                g.s_ids = S->ids;
-                g.out_ids = out_ids;
-                g.out_d2 = out_d2;
-                g.row_k = row_k;
-                g.row_off = row_off;
-                g.g32 = f.g32;
-                g.abs32 = f.abs32;
-                g.slack = f.slack;
-                g.err = (int *)(misc + 2);
-                g.n_fp64 = misc + 1;
-                for (int64_t b0 = 0; b0 < flagged && !rc; b0 += batch) {
-                    g.rows = frows + b0;
-                    g.n_rows = (int)std::min<int64_t>(batch, flagged - b0);
-                    k_topk_fallback<<<g.n_rows, 256, 0, st>>>(g);
-                    count_launch();
-                    ++launches;
-                    e = cudaGetLastError();
-                    if (e != cudaSuccess) rc = cuda_fail(e, "k_topk_fallback launch");
-                }
-                dev_free(fb, st);
-            }
+            dev_free(fb, st);
         }
     }
     if (timing) cudaEventRecord(ev[2], st);
-    unsigned long long h2[4] = {0, 0, 0, 0};
-    if (!rc) {
-        e = cudaMemcpyAsync(h2, misc, sizeof h2, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = cuda_fail(e, "top-k");
-    }
-    if (!rc && h2[2]) {
+    if (!rc && flagged > 0) rc = read_misc();   // otherwise the last listing pass read them
+    if (!rc && h[2]) {
         set_error("top-k: more than %d store rows tie within rounding at the k-th distance of a query",
                   kTkFallbackCap);
         rc = DL_EUNSUPPORTED;
@@ -735,7 +873,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         s.pairs_evaluated = nQ * nS;
         s.pairs_out = 0;
         s.band_pairs = flagged;   // rows re-solved by the exact scan
-        s.fp64_pairs = (int64_t)h2[1];
+        s.fp64_pairs = fp64 + (int64_t)h[1];
         s.precision = !use_tc ? DL_PREC_FP32 : fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
         s.tile_n = use_tc ? BN : 0;
         s.epilogue_warps = use_tc ? (wide ? 16 : 8) : 0;
