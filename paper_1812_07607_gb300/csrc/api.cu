@@ -292,7 +292,7 @@ static int run_pass(const PassCfg &c, PassOut *po)
                 L.p.cand_cnt = cnt + 1;
                 L.p.cand_cap = (unsigned long long)c.band_cap;
                 L.p.err = (int *)(cnt + 4);
-                rc = launch_tc_join(L, st, false, fp8, &po->grid);
+                rc = launch_tc_join(L, st, kModeEps, fp8, &po->grid);
                 ++launches;
             }
         } else {
@@ -825,7 +825,7 @@ int dl_debug_scores(const dl_store *R, const dl_store *S, int32_t precision, flo
         L.p.dump_e = e_out;
         L.p.orig_r = R->orig;
         L.p.orig_s = S->orig;
-        rc = launch_tc_join(L, st, false, fp8);
+        rc = launch_tc_join(L, st, kModeDump, fp8);
     }
     cudaError_t e = cudaStreamSynchronize(st);
     dev_free(ws, st);

@@ -27,9 +27,9 @@ struct TcParams {
     const float4 *rowpar;    // [m_tiles*128] {alpha_acc, alpha_rej, rq, nqt}
     const float *beta;       // S: RN32(||x||^2/2), +inf padding
     const float4 *cstat;     // S: per 32-column chunk {P1, P2, P3, min beta}
-    float *dump_h;           // diagnostics: h of every pair [nR][nS] in caller order (NULL: off)
-    float *dump_e;           // diagnostics: the bound E of every pair
-    const int32_t *orig_r, *orig_s;   // diagnostics: caller row of each store row
+    float *dump_h;           // kModeDump: h of every pair [nR][nS] in caller order
+    float *dump_e;           // kModeDump: the bound E of every pair
+    const int32_t *orig_r, *orig_s;   // kModeDump: caller row of each store row
     const float *sc_r;       // FP8: per-row power-of-two scales of R (NULL for BF16)
     const float *sc_s;       // FP8: per-32-row-chunk scales of S
     uint2 *cand;             // candidates: {r, c | 0x80000000 if a band pair, else a proven match}
@@ -45,8 +45,9 @@ struct TcParams {
     int row0;
 };
 
-// What the epilogue does with a tile: the epsilon-join's candidates, or the top-k's group maxima.
-enum TcMode { kModeEps = 0, kModeMaxima = 1 };
+// What the epilogue does with a tile: the epsilon-join's candidates, the top-k's group maxima, or the
+// diagnostics' dump of every pair's h and bound.
+enum TcMode { kModeEps = 0, kModeMaxima = 1, kModeDump = 2 };
 
 // Candidate entry flag: set for a band pair (needs the exact recheck).
 constexpr uint32_t kBandFlag = 0x80000000u;

@@ -35,76 +35,70 @@ __device__ __forceinline__ void fence_mbar_init()
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
+// Barriers are addressed by their shared-memory address (smem_u32), formed once by their users.
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
+// How long a try_wait may leave its thread suspended. Without a hint a waiting warp comes back to
+// poll every few clocks, and the polls of a dozen waiting warps take shared-memory cycles from the
+// tensor cores' operand reads: 262,144-row self-join, d = 128, 6.00 -> 5.67 ms (8 epilogue warps),
+// 5.94 -> 5.44 (16), the same from 0.5 us to 1 ms.
+constexpr uint32_t kSuspendNs = 1000;
+
+// CLUSTER: acquire at cluster scope, for barriers that threads of the peer CTA arrive on remotely.
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
+    if constexpr (CLUSTER)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity), "r"(kSuspendNs)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity), "r"(kSuspendNs)
+            : "memory");
     return ok != 0;
 }
 
-// A budget below this many clocks is a test setting: every abortable wait expires at once.
-// (mbarrier.try_wait may itself block until the phase completes, so a short budget alone
+// A budget below this many clocks is a test setting: the kernels' roles give up before their first
+// wait. (mbarrier.try_wait may itself block until the phase completes, so a short budget alone
 // does not make a wait on a small, fast join run out.)
 constexpr long long kExpireAtOnce = 64;
 
+template <bool CLUSTER>
+__device__ __noinline__ bool mbar_wait_long(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long budget)
+{
+    const long long t0 = clock64();
+    while (true) {
+        if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
+        if (*abort_flag) return false;
+        if (clock64() - t0 > budget) return false;
+    }
+}
+
 // Wait for the phase with the given parity to complete. Returns false when
-// `budget` SM clocks pass or another role raised the CTA's abort flag.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                          long long budget = kWaitBudgetClocks)
+// `budget` SM clocks pass or another role raised the CTA's abort flag. (The bounded loop is out of
+// line: the pipelines' waits are mostly ready, and their loops stay short.)
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long budget)
 {
-    if (budget < kExpireAtOnce) return false;
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > budget) return false;
-    }
-}
-
-// As mbar_try_wait, with acquire at cluster scope: for barriers that threads of the
-// peer CTA arrive on remotely.
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                                  long long budget = kWaitBudgetClocks)
-{
-    if (budget < kExpireAtOnce) return false;
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (true) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > budget) return false;
-    }
+    return mbar_try_wait<CLUSTER>(bar, parity) || mbar_wait_long<CLUSTER>(bar, parity, abort_flag, budget);
 }
 
 // ------------------------------------------------------------------ clusters (CTA pairs)
@@ -116,10 +110,10 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
 }
 
 // Shared::cluster address of the same shared-memory location in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t mapa_shared(const void *p, uint32_t rank)
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank)
 {
     uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
     return a;
 }
 
@@ -148,13 +142,22 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map)
 
 // 2-D tiled load of one box into shared memory; completion is signalled on `bar`
 // as transaction bytes. x (innermost, elements) must be 16-byte aligned.
-__device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int x, int y)
+__device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const CUtensorMap *map, uint32_t bar, int x, int y)
 {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::
-            "r"(smem_u32(smem_dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
+            "r"(smem_dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
         : "memory");
+}
+
+// Untiled bulk copy of `bytes` (a multiple of 16, both addresses on 16 bytes) into shared memory;
+// completion is signalled on `bar` as transaction bytes.
+__device__ __forceinline__ void bulk_load(uint32_t smem_dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
 }
 
 // ------------------------------------------------------------------ tcgen05
@@ -226,11 +229,9 @@ __device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t
 }
 
 // Arrive once on `bar` when every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void mma_commit(uint64_t *bar)
+__device__ __forceinline__ void mma_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // CTA-pair MMA (M = 256: rows 0-127 from this CTA's A, 128-255 from the peer's, N columns
@@ -259,33 +260,28 @@ __device__ __forceinline__ void mma_f8_cg2(uint32_t d_tmem, uint64_t adesc, uint
 
 // CTA-pair commit: arrive once on the barrier at `bar`'s offset in every CTA of `cta_mask`
 // when the pair's MMAs issued so far by this thread have completed.
-__device__ __forceinline__ void mma_commit_cg2_mc(uint64_t *bar, uint16_t cta_mask)
+__device__ __forceinline__ void mma_commit_cg2_mc(uint32_t bar, uint16_t cta_mask)
 {
     asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_u32(bar)),
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
         "h"(cta_mask)
         : "memory");
 }
 
-__device__ __forceinline__ void mma_commit_cg2(uint64_t *bar)
+__device__ __forceinline__ void mma_commit_cg2(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // Shared-memory matrix descriptor for a K-major operand stored with the 128-byte
-// swizzle: rows of 128 B, 8-row groups 1024 B apart (SBO), descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr)
-{
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);    // start address
-    d |= static_cast<uint64_t>(1) << 16;                     // leading byte offset (unused for SW128 K-major)
-    d |= static_cast<uint64_t>(1024 >> 4) << 32;             // stride byte offset: 8 rows x 128 B
-    d |= static_cast<uint64_t>(1) << 46;                     // descriptor version
-    d |= static_cast<uint64_t>(2) << 61;                     // layout: 128-byte swizzle
-    return d;
-}
+// swizzle: rows of 128 B, 8-row groups 1024 B apart (SBO), descriptor version 1. Its low word is the
+// start address / 16 (below 2^14, so offsets / 16 can be added to it) and the leading byte offset
+// (unused for SW128 K-major); the high word is the same for all of them.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+constexpr uint32_t kSmemDescHi = (1024u >> 4)   // stride byte offset: 8 rows x 128 B
+                                 | (1u << 14)   // descriptor version
+                                 | (2u << 29);  // layout: 128-byte swizzle
+__device__ __forceinline__ uint64_t smem_desc(uint32_t lo) { return ((uint64_t)kSmemDescHi << 32) | lo; }
 
 // Instruction descriptor for kind::f16, FP32 D, A and B both K-major and both FP16; with
 // kIdescBF16 added, both BF16.
@@ -307,26 +303,6 @@ __host__ __device__ constexpr uint32_t idesc_e4m3_f32(int M, int N)
            | (static_cast<uint32_t>(M >> 4) << 24);    // M / 16
 }
 
-// 32 lanes x 64 consecutive 32-bit columns: thread t gets lane (base lane + t).
-__device__ __forceinline__ void tmem_ld_32x32b_x64(uint32_t taddr, uint32_t (&v)[64])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31]), "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39]), "=r"(v[40]), "=r"(v[41]), "=r"(v[42]), "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]), "=r"(v[48]), "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]), "=r"(v[55]), "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]), "=r"(v[61]), "=r"(v[62]), "=r"(v[63])
-        : "r"(taddr)
-        : "memory");
-}
-
-// Wait for this thread's tcgen05.ld operations; the registers are tied to the
-// wait so that no use of the loaded values can be scheduled before it.
-__device__ __forceinline__ void tmem_ld_wait_regs(uint32_t (&v)[64])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31]), "+r"(v[32]), "+r"(v[33]), "+r"(v[34]), "+r"(v[35]), "+r"(v[36]), "+r"(v[37]), "+r"(v[38]), "+r"(v[39]), "+r"(v[40]), "+r"(v[41]), "+r"(v[42]), "+r"(v[43]), "+r"(v[44]), "+r"(v[45]), "+r"(v[46]), "+r"(v[47]), "+r"(v[48]), "+r"(v[49]), "+r"(v[50]), "+r"(v[51]), "+r"(v[52]), "+r"(v[53]), "+r"(v[54]), "+r"(v[55]), "+r"(v[56]), "+r"(v[57]), "+r"(v[58]), "+r"(v[59]), "+r"(v[60]), "+r"(v[61]), "+r"(v[62]), "+r"(v[63])
-                 :
-                 : "memory");
-}
-
 // 32 lanes x 32 consecutive 32-bit columns: thread t gets lane (base lane + t).
 __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&v)[32])
 {
@@ -337,6 +313,8 @@ __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&v)
         : "memory");
 }
 
+// Wait for this thread's tcgen05.ld operations; the registers are tied to the
+// wait so that no use of the loaded values can be scheduled before it.
 __device__ __forceinline__ void tmem_ld_wait_regs(uint32_t (&v)[32])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -344,20 +322,5 @@ __device__ __forceinline__ void tmem_ld_wait_regs(uint32_t (&v)[32])
                  :
                  : "memory");
 }
-
-// Asynchronous global -> shared copies (cp.async, no registers held while in flight).
-__device__ __forceinline__ void cp_async_16(void *smem, const void *gmem)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_8(void *smem, const void *gmem)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 }  // namespace dl
