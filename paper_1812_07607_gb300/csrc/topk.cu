@@ -69,18 +69,21 @@ __global__ void __launch_bounds__(256) k_rowpar_topk(const double *__restrict__ 
 // (T - slack) - E (-inf with fewer than k groups). Padding rows (+inf) list nothing. One warp per row,
 // 32 values a lane (groups folded by maximum past 1,024: disjoint groups stay disjoint), no barriers;
 // T is found bit by bit from the values' common prefix on and cut off after kTkBits bits, downwards,
-// which lets in about one column more in 2^kTkBits. 4,096 rows of 1,953 groups, k = 100: 66 us,
-// 105 with a CTA a row and all 32 bits.
+// which lets in about one column more in 2^kTkBits. A row's groups are loaded all at once: what bounds
+// a few rows is that latency (one row of 976 groups: 4 us, 18 with a load at a time), what bounds many
+// the counting steps (4,096 rows of 1,953 groups, k = 100: 54 us; 66 so, 105 with a CTA a row and all
+// 32 bits besides). It also empties the rows' lists.
 constexpr int kTkBits = 14;
 
 __global__ void __launch_bounds__(256) k_topk_theta(const float4 *__restrict__ rowpar, const float *__restrict__ gmax, int n_groups,
                                                     int64_t row0, int64_t nQ, int64_t rows_tot, int k, const int *__restrict__ row_k,
-                                                    float4 *__restrict__ thr)
+                                                    float4 *__restrict__ thr, int *__restrict__ cnt)
 {
     const int lane = threadIdx.x & 31;
     const int64_t lr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int64_t i = row0 + lr;
     if (i >= rows_tot) return;
+    if (lane == 0 && i < nQ) cnt[lr] = 0;   // the row's list, empty
     const float inf = __int_as_float(0x7f800000);
     if (i >= nQ) {
         if (lane == 0) thr[i] = make_float4(inf, inf, 0.f, 0.f);
@@ -94,9 +97,15 @@ __global__ void __launch_bounds__(256) k_topk_theta(const float4 *__restrict__ r
         const float *g = gmax + (size_t)lr * n_groups;
         unsigned lo = 0xffffffffu, hi = 0u;
 #pragma unroll
+        for (int s = 0; s < kTkGroups / 32; ++s)   // every load in flight
+            v[s] = __float_as_uint(s * 32 + lane < n_groups ? __ldg(g + s * 32 + lane) : -inf);
+        for (int j0 = kTkGroups; j0 < n_groups; j0 += kTkGroups)
+#pragma unroll
+            for (int s = 0; s < kTkGroups / 32; ++s)
+                if (j0 + s * 32 + lane < n_groups) v[s] = __float_as_uint(fmaxf(__uint_as_float(v[s]), __ldg(g + j0 + s * 32 + lane)));
+#pragma unroll
         for (int s = 0; s < kTkGroups / 32; ++s) {
-            float m = -inf;
-            for (int j = s * 32 + lane; j < n_groups; j += kTkGroups) m = fmaxf(m, __ldg(g + j));
+            const float m = __uint_as_float(v[s]);
             v[s] = float_order_code(m);
             hi = max(hi, v[s]);
             if (m > -inf) lo = min(lo, v[s]);
@@ -737,10 +746,9 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                         L.p.tile_stride = 1;
                     }
                     if (!rc && nS > 0) {
-                        k_topk_theta<<<(unsigned)(cr_pad / 8), 256, 0, st>>>(rowpar, gmax, n_groups, row0, nQ, row0 + cr_pad, k, row_k, thr);
+                        k_topk_theta<<<(unsigned)(cr_pad / 8), 256, 0, st>>>(rowpar, gmax, n_groups, row0, nQ, row0 + cr_pad, k, row_k, thr, t.cnt);
                         rc = launched("k_topk_theta launch");
-                    }
-                    if (!rc) {
+                    } else if (!rc) {   // an empty store: empty lists
                         e = cudaMemsetAsync(t.cnt, 0, b_n, st);
                         if (e != cudaSuccess) rc = cuda_fail(e, "top-k memset");
                     }
