@@ -316,11 +316,11 @@ static int run_pass(const PassCfg &c, PassOut *po)
         nvtxRangePushA("exact recheck of the band (K6)");
         if (!rc && c.ip) {
             rc = launch_finalize_ip(band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2, jo, cnt + 3,
-                                    cnt + 2, sms * 8, st, (int)nR, (int)nS);
+                                    cnt + 2, sms * 5, st, (int)nR, (int)nS);
             ++launches;
         } else if (!rc && tc_prec(c.prec)) {
             rc = launch_finalize(band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2, c.t_acc,
-                                 c.t_rej, jo, cnt + 3, cnt + 2, sms * 8, st, (int)nR, (int)nS);
+                                 c.t_rej, jo, cnt + 3, cnt + 2, sms * 5, st, (int)nR, (int)nS);
             ++launches;
         } else if (!rc && c.prec == DL_PREC_FP32 && c.metric != 0) {
             rc = launch_hist_recheck(c.metric, band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2,

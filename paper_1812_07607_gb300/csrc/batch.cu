@@ -71,6 +71,9 @@ __global__ void __launch_bounds__(256)
                    unsigned long long *__restrict__ req_cnt,
                    unsigned long long *__restrict__ n_fp64, unsigned long long *__restrict__ n_band, int nQ, int nS)
 {
+    __shared__ unsigned s_cnt[2];   // the CTA's band pairs and canonical sums
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0u;
+    __syncthreads();
     const unsigned lane = threadIdx.x & 31;
     const unsigned long long n = min(*cand_cnt, cap);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -106,11 +109,16 @@ __global__ void __launch_bounds__(256)
         }
         const unsigned fm = __ballot_sync(0xffffffffu, f64);
         if (lane == 0) {
-            if (bm) atomicAdd(n_band, (unsigned long long)__popc(bm));
-            if (fm) atomicAdd(n_fp64, (unsigned long long)__popc(fm));
+            if (bm) atomicAdd(&s_cnt[0], (unsigned)__popc(bm));
+            if (fm) atomicAdd(&s_cnt[1], (unsigned)__popc(fm));
         }
         grouped_add(req_cnt, acc ? row_req[r] : 0, acc, 1u);
         if (valid) cand[i] = acc ? make_uint2((uint32_t)r, (uint32_t)c) : make_uint2((uint32_t)r, 0xffffffffu);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_cnt[0]) atomicAdd(n_band, (unsigned long long)s_cnt[0]);
+        if (s_cnt[1]) atomicAdd(n_fp64, (unsigned long long)s_cnt[1]);
     }
 }
 
