@@ -158,7 +158,10 @@ struct TopkRows {
 };
 
 // The listed candidates' FP32 distances (8-lane groups, 16-byte slices, four candidates a warp at a
-// time), each into its row's list. What bounds it: the rows' L2 reads, 8 d bytes a candidate.
+// time), each into its row's list. What bounds it: the rows' reads, 8 d bytes a candidate and past the
+// L2 for a store of its size. The grid is what is resident and windows are short until every warp has
+// many: 1.6 M candidates, d = 256, 299 us (413 with 32-wide windows over a grid of one and a third
+// times what is resident).
 __global__ void __launch_bounds__(256) k_topk_dist(const TopkRows f, const uint2 *__restrict__ cand,
                                                    const unsigned long long *__restrict__ cand_cnt, unsigned long long cand_cap)
 {
@@ -166,7 +169,8 @@ __global__ void __launch_bounds__(256) k_topk_dist(const TopkRows f, const uint2
     const unsigned long long n = min(*cand_cnt, cand_cap);
     const unsigned long long w0 = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-    const unsigned win = n <= nw * 4 ? 4u : 32u;   // few candidates: four a warp, one round trip each
+    // few candidates: four a warp, one round trip each; more: eight, until each warp has 256
+    const unsigned win = n <= nw * 4 ? 4u : n < nw * 256 ? 8u : 32u;
     const bool in = lane < win;
     uint2 nxt = in && w0 * win + lane < n ? cand[w0 * win + lane] : make_uint2(0u, 0u);
     for (unsigned long long base = w0 * win; base < n; base += nw * win) {
@@ -769,7 +773,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                     rc = launch_tc_join(L, st);
                     ++launches;
                     if (!rc) {
-                        const int64_t grid = std::min<int64_t>((cand_cap + 255) / 256, (int64_t)sms * 8);
+                        const int64_t grid = std::min<int64_t>((cand_cap + 255) / 256, (int64_t)sms * 6);   // 6 resident a SM
                         k_topk_dist<<<(unsigned)grid, 256, 0, st>>>(t, cand, misc + 4, (unsigned long long)cand_cap);
                         rc = launched("k_topk_dist launch");
                     }
