@@ -90,6 +90,35 @@ __device__ __forceinline__ double widen(float f)
     return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
+// The subtraction of abs_diff64 past its exponent range; out of line, or it would run under a predicate.
+static __device__ __noinline__ double abs_diff64_far(float q, float x) { return fabs(__dsub_rn((double)q, (double)x)); }
+
+// |RN64(q - x)| without the FP64 pipe (16 clocks of an SM a warp instruction there; these thirty integer
+// ones take 8): q - x = T 2^(e - 150) exactly, with T below 2^53 as long as the features' exponents lie
+// within 28 of each other. Farther apart, q - x itself rounds: the FP64 operation.
+__device__ __forceinline__ double abs_diff64(float q, float x)
+{
+    const unsigned uq = __float_as_uint(q), ux = __float_as_uint(x);
+    const int fq = (int)((uq >> 23) & 255u), fx = (int)((ux >> 23) & 255u);
+    const unsigned mq = (uq & 0x7fffffu) | (fq ? 0x800000u : 0u), mx = (ux & 0x7fffffu) | (fx ? 0x800000u : 0u);
+    const int eq = max(fq, 1), ex = max(fx, 1);
+    const bool q_up = eq >= ex;
+    const unsigned mb = q_up ? mq : mx, ms = q_up ? mx : mq;   // of the larger and the smaller exponent
+    int es = q_up ? ex : eq, gap = q_up ? eq - ex : ex - eq;
+    if (ms == 0u) {   // the other feature alone
+        es += gap;
+        gap = 0;
+    }
+    if (gap > 28) return abs_diff64_far(q, x);
+    const unsigned long long big = (unsigned long long)mb << gap;
+    const long long diff = ((uq ^ ux) >> 31) ? (long long)(big + ms) : (long long)(big - ms);
+    const unsigned long long T = (unsigned long long)(diff < 0 ? -diff : diff);   // gap 0: either may be the larger
+    if (T == 0ULL) return 0.0;
+    const int lz = __clzll((long long)T);   // 11 or more: the leading bit goes to bit 52
+    const unsigned long long man = T << (lz - 11);
+    return __longlong_as_double((long long)(man + ((unsigned long long)(1023 + 63 - lz + es - 150 - 1) << 52)));
+}
+
 // Float-float value S of sum_k (q_k - x_k)^2 by the whole warp (lane l takes k = l, l+32, ...;
 // a butterfly of commutative merges, so every lane returns the same S).
 __device__ __forceinline__ double warp_ff_sq(const float *__restrict__ q, const float *__restrict__ x, int d)

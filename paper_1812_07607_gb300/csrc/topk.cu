@@ -25,10 +25,10 @@
 //
 // Heaps of lower bounds kept by the epilogue's lanes in global memory did this in one pass over the
 // store; every insert sifted through dependent loads while the other lanes of its warp waited.
-// 4,096 queries against 1,000,003 x 256, k = 100: 18.6 ms then, 3.5 now; one query, k = 1: 0.53 ms, 0.21 (its 16
+// 4,096 queries against 1,000,003 x 256, k = 100: 18.6 ms then, 2.94 now; one query, k = 1: 0.53 ms, 0.195 (its 16
 // column splits left 136 SMs idle).
-// What bounds it now, of the 3.5 ms: the two tensor-core passes 0.33 + 1.45 ms, the candidates' rows 0.4,
-// the canonical sums 0.6; of the 0.21 ms: the store's 512 MB of FP16 rows, 76 us.
+// What bounds it now, of the 2.94 ms: the two tensor-core passes 0.30 + 1.17 ms, the candidates' rows 0.30,
+// the canonical sums 0.49; of the 0.195 ms: the store's 512 MB of FP16 rows, 76 us.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -318,8 +318,10 @@ __global__ void __launch_bounds__(256) k_topk_keep(const TopkRows f, int *__rest
 
 // The kept columns' canonical distances, up to 64 columns of any rows at a time: every thread forms
 // terms, a run of each column's, then a thread per column adds its own in ascending k. What bounds it:
-// the FP64 pipe, costed per warp instruction (16 cycles of an SM): three operations a term with every
-// lane busy, the conversions done by the integer units.
+// the FP64 pipe, costed per warp instruction (16 cycles of an SM): two operations a term with every
+// lane busy, the subtraction and the conversions done by the integer units (abs_diff64). The whole call
+// of 4,096 queries, k = 100, d = 256: 3.12 -> 2.94 ms against three operations; with the squares in
+// integers too (128-bit products, some 150 instructions) 3.13.
 __global__ void __launch_bounds__(128) k_topk_canon(const TopkRows f)
 {
     __shared__ double sh_t[kTkTerms];
@@ -345,7 +347,7 @@ __global__ void __launch_bounds__(128) k_topk_canon(const TopkRows f)
             for (int e = tid; e < na << sh; e += 128) {
                 const int a = e >> sh, k = e & (run - 1);
                 if (k < nk) {
-                    const double t = __dsub_rn(widen(__ldg(sh_q[a] + k0 + k)), widen(__ldg(sh_x[a] + k0 + k)));
+                    const double t = abs_diff64(__ldg(sh_q[a] + k0 + k), __ldg(sh_x[a] + k0 + k));
                     sh_t[a * ld + k] = __dmul_rn(t, t);
                 }
             }
