@@ -2,9 +2,8 @@
 
 A 32 x 32 chunk of a tile puts up to four hit rows aside and classifies them after the accumulator is
 released; more go through the many-row path. Cluster counts from one (every pair matches) to none take
-a chunk through every number of hit rows, with eight and sixteen epilogue warps. The pairs leave in
-batches of 128 a warp, so the full mode (two pairs a match) and a buffer too small for the pairs run
-over the same shapes. A 70,000-row clustered store has R tiles whose first columns lie past a block of
+a chunk through every number of hit rows, with eight and sixteen epilogue warps. The full mode (two
+pairs a match) and a buffer too small for the pairs run over clustered rows too. A 70,000-row clustered store has R tiles whose first columns lie past a block of
 tile tests, and features that start off a 16-byte line take the unaligned reads.
 """
 
