@@ -4,9 +4,8 @@
 // deduplication) are issued here many at a time against one resident store.
 // Every epsilon-join row of every request goes into ONE persistent tensor-core
 // launch: the per-row thresholds (k_rowpar) carry each row's own eps, so tiles
-// may mix requests freely. Every top-k row goes into one top-k launch with the
-// largest k as heap size and each row's own k in the finalize. Outputs are then
-// routed to their requests:
+// may mix requests freely. The top-k rows of each distinct k go into one top-k.
+// Outputs are then routed to their requests:
 //   k_batch_expand   request table -> per query row: caller row, eps^2 or k,
 //                    request index and output slot;
 //   tc_join_kernel   candidates (proven matches and band pairs) of all eps rows;
@@ -229,7 +228,7 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
             return DL_EINVAL;
         }
     }
-    // top-k rows are grouped by k (each group runs with its own heap size)
+    // top-k rows are grouped by k (each group's lists and thresholds follow its k)
     std::stable_sort(kr.begin(), kr.end(), [](const ReqDev &a, const ReqDev &b) { return a.k < b.k; });
     std::vector<std::pair<int, std::pair<int64_t, int64_t>>> kgroups;   // k -> [first row, end row)
     {
