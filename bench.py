@@ -635,7 +635,7 @@ def rows_leg(dl, sm_mhz=None, reps=5):
     Xs = dl.Store(torch.arange(n, device="cuda"), torch.from_numpy(X).cuda())
     P = n * (n - 1) // 2
     for metric, unit_ops, lanes, what in (("l1", 2, 128, "FP32 add (sub, add |t|) per term, 128 lanes/SM"),
-                                          ("chi2", 1, 16, "one MUFU reciprocal per term, 16 lanes/SM")):
+                                          ("chi2", 5, 128, "FP32 operations per term beside half a reciprocal, 128 lanes/SM")):
         st = {}
 
         def call():
