@@ -605,6 +605,15 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         return DL_EINVAL;
     }
     int code = (o.tile_n ? o.tile_n : 256) | (o.epilogue_warps == 16 ? kTuneWide : 0);
+    const int prec = !use_tc ? DL_PREC_FP32 : fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
+    if (nQ == 0) {   // no rows: nothing to run, time or tune
+        if (stats) {
+            stats->precision = prec;
+            stats->tile_n = use_tc ? tune_bn(code) : 0;
+            stats->epilogue_warps = !use_tc ? 0 : tune_wide(code) ? 16 : 8;
+        }
+        return DL_OK;
+    }
     if (use_tc && o.tile_n == 0 && o.epilogue_warps == 0) code = tune_pick(Q->dp, kTuneTopk, nQ, nS, &tune_trial);
     const int BN = tune_bn(code);
     const bool wide = use_tc && tune_wide(code);   // 16 epilogue warps
@@ -621,7 +630,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     const int64_t chunk_rows =
         use_tc ? std::min<int64_t>(rows, std::max<int64_t>(1, (1LL << 30) / (per_row * 128)) * 128) : rows;
 
-    const size_t b_rowpar = al256((size_t)rows * sizeof(float4)), b_frows = al256((size_t)std::max<int64_t>(nQ, 1) * sizeof(int));
+    const size_t b_rowpar = al256((size_t)rows * sizeof(float4)), b_frows = al256((size_t)nQ * sizeof(int));
     const bool timing = o.timing || tune_trial;
     void *ws = nullptr, *cws = nullptr;
     int rc = dev_alloc(&ws, 2 * b_rowpar + b_frows + 256, st);
@@ -687,7 +696,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     t.n_kept = misc + 5;
     int64_t flagged = 0;   // rows named in frows for the exact scan
     int64_t fp64 = 0;      // canonical distances of the other rows
-    if (nQ > 0 && (nS == 0 || use_tc)) {
+    if (nS == 0 || use_tc) {
         Half *hQ = nullptr, *hS = nullptr;
         const CUtensorMap *tmA = nullptr, *tmB = nullptr;
         if (nS > 0) {
@@ -824,7 +833,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                 rc = reset();
             }
         }
-    } else if (nQ > 0) {   // no tensor-core pass for this shape: every row takes the exact scan
+    } else {   // no tensor-core pass for this shape: every row takes the exact scan
         std::vector<int> every((size_t)nQ);
         for (int64_t i = 0; i < nQ; ++i) every[(size_t)i] = (int)i;
         e = cudaMemcpyAsync(frows, every.data(), (size_t)nQ * sizeof(int), cudaMemcpyHostToDevice, st);
@@ -888,7 +897,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         s.pairs_out = 0;
         s.band_pairs = flagged;   // rows re-solved by the exact scan
         s.fp64_pairs = fp64 + (int64_t)h[1];
-        s.precision = !use_tc ? DL_PREC_FP32 : fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
+        s.precision = prec;
         s.tile_n = use_tc ? BN : 0;
         s.epilogue_warps = use_tc ? (wide ? 16 : 8) : 0;
         s.kernels_launched = launches;
