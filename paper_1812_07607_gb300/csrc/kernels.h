@@ -118,8 +118,8 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
 int launch_diag(const int64_t *ids, int64_t n, int64_t *out_r, int64_t *out_s, unsigned long long *out_cnt,
                 unsigned long long cap, cudaStream_t st);
 
-// Workspace of one query row of a top-k against nS rows (topk.cu).
-int64_t topk_row_bytes(int64_t nS, int dp, int k);
+// What a top-k of nQ rows against nS takes at most for its group maxima, lists and candidates (topk.cu).
+int64_t topk_scratch_bytes(int64_t nQ, int64_t nS, int dp, int k);
 // ---- top-k core (topk.cu): every row of Q against S, outputs at row_off or caller row * k
 int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, const int64_t *row_off,
               int64_t *out_ids, double *out_d2, const dl_join_opts &o, cudaStream_t st, dl_join_stats *stats);

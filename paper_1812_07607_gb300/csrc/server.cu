@@ -75,7 +75,7 @@ static int64_t estimate_bytes(const dl_store *S, int32_t kind, int64_t nq, int32
     const int64_t d = S->d, dp = S->dp;
     int64_t b = nq * (d * 4 + dp * 2 + 64) * 2;           // uploaded + internal query store
     if (kind == DL_REQ_TOPK) {
-        b += nq * k * 16 + nq * topk_row_bytes(S->n, S->dp, k);   // output + group maxima, lists and candidates
+        b += nq * k * 16 + topk_scratch_bytes(nq, S->n, S->dp, k);   // output + group maxima, lists, candidates
     } else {
         b += nq * 16 * 1024 + (1 << 20);                   // output / candidates, grown on demand
     }

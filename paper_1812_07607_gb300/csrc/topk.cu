@@ -21,6 +21,10 @@
 // overflows again takes
 //   k_topk_fallback    an exact scan of the whole store for that row (FP32 bound + radix select +
 //                      FP64 + rank).
+// The candidates of all rows share one list, which never holds more than the rows' lists do together
+// (rows may list every column where the 16-bit bound exceeds the spread of the distances). When it
+// still overflows, some row holds more than its own list: those are tightened, or go to the exact scan
+// after kTkRefines times, and the others' candidates are listed again.
 // Store rows are in norm order; outputs are written at the caller's row order.
 //
 // Heaps of lower bounds kept by the epilogue's lanes in global memory did this in one pass over the
@@ -45,6 +49,9 @@ constexpr int kTkGroups = 1024;      // group maxima k_topk_theta keeps apart (m
 constexpr int kTkTermC = 64;         // candidates whose canonical terms are staged together
 constexpr int kTkTerms = kTkTermC * 33;   // staged terms, padding included
 constexpr int kTkRefines = 2;        // passes with tightened thresholds before the exact scan
+constexpr int kTkScan = 1 << 30;     // list count of a row that is left to the exact scan
+constexpr int kTkScanPasses = 4;     // passes that name such rows while the shared list overflows (then: all)
+constexpr int64_t kTkWorkspace = 1LL << 30;   // bytes of lists and candidates of a chunk of query rows, at most
 constexpr int kTkFallbackCap = 8192; // candidates a fallback block can rank
 
 // Per query row: {canonical slack of h, unused, ||q - q~|| up, ||q~|| up}; padding rows get zeros.
@@ -208,17 +215,28 @@ __device__ __forceinline__ float lower32(const TopkRows &f, float s)
 
 // Thresholds of another listing pass: an overflowed row's from the k-th smallest of the distances it
 // did list (at least k columns lie within its upper bound u, so a column with D > u (1 + slack) is not
-// in the top k: h < RD((||q||^2_dn - e2 (1 + 2 g64)) / 2) - E proves that, as in k_rowpar); every other
-// row lists nothing (its list stands). One CTA per row of the chunk.
+// in the top k: h < RD((||q||^2_dn - e2 (1 + 2 g64)) / 2) - E proves that, as in k_rowpar), or none and
+// the exact scan (`scan`; 2: every row); every other row lists nothing, its list stands -- or, when the
+// shared list was too short (`redo`), what its threshold admits once more. One CTA per row of the chunk.
 __global__ void __launch_bounds__(256) k_topk_refine(const TopkRows f, const double *__restrict__ nq64, int dp, double g64,
-                                                     int64_t rows_pad, const float4 *__restrict__ rowpar, float4 *__restrict__ thr)
+                                                     int64_t rows_pad, int redo, int scan, const float4 *__restrict__ rowpar,
+                                                     float4 *__restrict__ thr)
 {
     __shared__ unsigned s_cnt[2];
     const int64_t lr = blockIdx.x;
     const int64_t i = f.row0 + lr;
     const float inf = __int_as_float(0x7f800000);
-    if (lr >= f.rows || f.cnt[lr] <= f.cap) {
-        if (threadIdx.x == 0 && lr < rows_pad) thr[i] = make_float4(inf, inf, 0.f, 0.f);
+    const float4 none = make_float4(inf, inf, 0.f, 0.f);
+    const int m = lr >= f.rows || scan == 2 ? kTkScan : f.cnt[lr];
+    if (m <= f.cap && redo) {
+        if (threadIdx.x == 0) f.cnt[lr] = 0;
+        return;
+    }
+    if (m <= f.cap || m >= kTkScan || scan) {
+        if (threadIdx.x == 0) {
+            if (lr < rows_pad) thr[i] = none;
+            if (lr < f.rows && m > f.cap) f.cnt[lr] = kTkScan;
+        }
         return;
     }
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0u;
@@ -238,7 +256,8 @@ __global__ void __launch_bounds__(256) k_topk_refine(const TopkRows f, const dou
         const double nq_dn = __dmul_rd(nq64[i], 1.0 - (double)(dp + 2) * 2.220446049250313e-16);
         const double rej = __dsub_rd(nq_dn, __dmul_ru(e2, 1.0 + 2.0 * g64)) * 0.5;
         const float4 rp = rowpar[i];
-        thr[i] = make_float4(inf, __fsub_rd(__double2float_rd(rej), rp.x), rp.z, rp.w);
+        // never below the pass before: its candidates fitted the shared list, so will these
+        thr[i] = make_float4(inf, fmaxf(thr[i].y, __fsub_rd(__double2float_rd(rej), rp.x)), rp.z, rp.w);
         f.cnt[lr] = 0;
     }
 }
@@ -557,8 +576,8 @@ struct TopkShape {
     int cap;            // list capacity of a row
     int gran;           // columns of a group
     int n_groups;       // groups of a row (0: every column fits the list, no first pass)
-    int64_t per_cand;   // candidates of a row provided for
-    int64_t bytes() const { return 4LL * n_groups + 20LL * cap + 4 + 8 * per_cand; }
+    int64_t per_cand;   // candidates of a row provided for at first (never more than cap)
+    int64_t bytes() const { return 4LL * n_groups + 20LL * cap + 4 + 8LL * cap; }   // of a row, at most
 };
 
 static TopkShape topk_shape(int64_t nS, int dp, int k, int BN)
@@ -576,7 +595,17 @@ static TopkShape topk_shape(int64_t nS, int dp, int k, int BN)
     return s;
 }
 
-int64_t topk_row_bytes(int64_t nS, int dp, int k) { return topk_shape(nS, dp, k, 256).bytes(); }
+// Query rows whose lists and candidates stay within kTkWorkspace (whole 128-row tiles, at least one).
+static int64_t topk_chunk_rows(int64_t rows, int64_t per_row)
+{
+    return std::min<int64_t>(rows, std::max<int64_t>(1, kTkWorkspace / (per_row * 128)) * 128);
+}
+
+int64_t topk_scratch_bytes(int64_t nQ, int64_t nS, int dp, int k)
+{
+    const int64_t per_row = topk_shape(nS, dp, k, 256).bytes();
+    return std::min(nQ, topk_chunk_rows((nQ + 127) / 128 * 128, per_row)) * per_row + 65536 * 8;
+}
 
 // Top-k of every row of Q against S into out_ids / out_d2. k is the largest k of
 // any row; row_k (device, optional) gives each row's own k and
@@ -621,14 +650,12 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     const int64_t mt = (nQ + 127) / 128, rows = mt * 128;
     const int64_t nt = (nS + BN - 1) / BN;
 
-    // the two passes' shape, and query rows per chunk so that its workspace stays near 1 GB
+    // the two passes' shape, and the query rows of a chunk
     const TopkShape sh = topk_shape(nS, Q->dp, k, BN);
     const int f = sh.stride, cap = sh.cap, gran = sh.gran, n_groups = sh.n_groups;
     const int64_t nt_sub = (nt + f - 1) / f, per_cand = sh.per_cand;
     const bool all = n_groups == 0;   // every column fits a row's list: no first pass
-    const int64_t per_row = sh.bytes();
-    const int64_t chunk_rows =
-        use_tc ? std::min<int64_t>(rows, std::max<int64_t>(1, (1LL << 30) / (per_row * 128)) * 128) : rows;
+    const int64_t chunk_rows = topk_chunk_rows(rows, sh.bytes());
 
     const size_t b_rowpar = al256((size_t)rows * sizeof(float4)), b_frows = al256((size_t)nQ * sizeof(int));
     const bool timing = o.timing || tune_trial;
@@ -710,16 +737,21 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                 rc = launched("k_rowpar_topk launch");
             }
         }
-        int64_t cand_cap = std::min<int64_t>(chunk_rows, nQ) * per_cand + 65536;
+        const int64_t cand_max = chunk_rows * cap + 65536;
+        int64_t cand_cap = std::min<int64_t>(std::min<int64_t>(chunk_rows, nQ) * per_cand + 65536, cand_max);
         const size_t b_g = al256((size_t)chunk_rows * n_groups * 4), b_l = al256((size_t)chunk_rows * cap * 4),
                      b_n = al256((size_t)chunk_rows * 4), b_d = al256((size_t)chunk_rows * cap * 8);
-        for (int64_t row0 = 0; row0 < nQ && !rc; row0 += chunk_rows) {
-            const int64_t cr = std::min(chunk_rows, nQ - row0), cr_pad = (cr + 127) / 128 * 128;
-            for (int pass = 0, again = 0, grown = 0; !rc; ++pass) {   // listing passes over this chunk
+        for (int64_t row0 = 0; row0 < nQ && !rc;) {
+            int64_t cr = 0;
+            int refined = 0, scans = 0;
+            bool redo = false;   // the pass before overflowed the shared list
+            for (int pass = 0; !rc; ++pass) {   // listing passes over this chunk
                 if (!cws) {
                     rc = dev_alloc(&cws, b_g + 3 * b_l + b_n + b_d + (size_t)cand_cap * 8, st);
                     if (rc) break;
                 }
+                cr = std::min(chunk_rows, nQ - row0);
+                const int64_t cr_pad = (cr + 127) / 128 * 128;
                 float *gmax = (float *)cws;
                 t.col = (uint32_t *)((char *)cws + b_g);
                 t.d32 = (float *)((char *)cws + b_g + b_l);
@@ -767,12 +799,12 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                         e = cudaMemsetAsync(t.cnt, 0, b_n, st);
                         if (e != cudaSuccess) rc = cuda_fail(e, "top-k memset");
                     }
-                } else if (again) {   // tighter thresholds for the rows whose list overflowed
-                    k_topk_refine<<<(unsigned)cr_pad, 256, 0, st>>>(t, Q->nq64, Q->dp, g64, cr_pad, rowpar, thr);
+                } else {   // tighter thresholds for the rows whose list overflowed, then the exact scan
+                    const int scan = refined < kTkRefines ? 0 : ++scans <= kTkScanPasses ? 1 : 2;
+                    if (!scan) ++refined;
+                    k_topk_refine<<<(unsigned)cr_pad, 256, 0, st>>>(t, Q->nq64, Q->dp, g64, cr_pad, redo, scan, rowpar, thr);
                     rc = launched("k_topk_refine launch");
-                    if (!rc) {
-                        rc = reset();
-                    }
+                    if (!rc) rc = reset();
                 }
                 if (!rc && nS > 0) {
                     L.p.rowpar = thr;
@@ -802,36 +834,31 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                         rc = launched("k_topk_out launch");
                     }
                 }
-                if (timing && row0 + chunk_rows >= nQ && pass == 0) cudaEventRecord(ev[1], st);
+                if (timing && row0 + cr >= nQ && pass == 0) cudaEventRecord(ev[1], st);
                 if (!rc) rc = read_misc();
                 if (rc) break;
                 if (h[3]) {
                     set_error("top-k: a bounded device wait expired");
                     return done(DL_ETIMEOUT);
                 }
-                if (h[4] > (unsigned long long)cand_cap) {   // the candidate list was too short: its exact size, again
-                    cand_cap = (int64_t)h[4] + (int64_t)(h[4] / 8) + 1024;
+                redo = h[4] > (unsigned long long)cand_cap;   // lists short of candidates: what came of them is written again
+                if (redo && cand_cap < cand_max) {   // the shared list was too short: its exact size, again
+                    cand_cap = std::min<int64_t>((int64_t)(h[4] + h[4] / 8) + 1024, cand_max);
                     dev_free(cws, st);
                     cws = nullptr;
-                    if (++grown > 4) {
-                        set_error("top-k: the candidate list keeps overflowing");
-                        return done(DL_ENOMEM);
-                    }
                     pass = -1;
-                    again = 0;
+                    refined = scans = 0;
                     rc = reset();
                     continue;
                 }
-                if (h[0] == 0 || again == kTkRefines) {
+                if (!redo && (h[0] == 0 || refined == kTkRefines)) {
                     flagged += (int64_t)h[0];
                     fp64 += (int64_t)h[5];
                     break;
                 }
-                ++again;
             }
-            if (!rc && row0 + chunk_rows < nQ) {   // this chunk's named rows stay; its counters start over
-                rc = reset();
-            }
+            row0 += cr;
+            if (!rc && row0 < nQ) rc = reset();   // this chunk's named rows stay; its counters start over
         }
     } else {   // no tensor-core pass for this shape: every row takes the exact scan
         std::vector<int> every((size_t)nQ);

@@ -1,0 +1,69 @@
+"""The top-k's workspace is bounded whatever the data.
+
+Where the 16-bit bound exceeds the spread of the distances (rows with a large common offset), a row's
+threshold admits every column. The candidates then have to stay within the workspace's limit, the
+rows concerned take the exact scan, the others their lists, and ids and distances stay bit-exact.
+Memory is looked at from processes of their own: the pool keeps what earlier calls took.
+"""
+
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+from paper_1812_07607_gb300 import workloads as W
+from test_gpu_topk import _store, check_topk, dl, orc  # noqa: F401 (fixtures)
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def run(code):
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout.split()
+
+
+def offset(g, n, d):
+    return (1000 + 1e-3 * g.standard_normal((n, d))).astype(np.float32)
+
+
+def test_offset_cluster_memory_is_bounded():
+    """1,536 rows that each reach all of 200,000 columns: 2.5 GB as one list of 8-byte candidates."""
+    taken, = run("""
+import torch
+from paper_1812_07607_gb300 import dl
+g = torch.Generator(device="cuda"); g.manual_seed(5)
+st = lambda n: dl.Store(torch.arange(n, device="cuda"), 1000 + torch.randn(n, 16, generator=g, device="cuda") * 1e-3)
+Q, S = st(1536), st(200000)
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+dl.topk_join(Q, S, 10).free()
+print(free - torch.cuda.mem_get_info()[0])
+""")
+    # the lists' limit (2^30) and the exact scan's (2^28), in the pool's granularity
+    assert int(taken) <= (1 << 30) + (1 << 28) + (1 << 27)
+
+
+@pytest.mark.parametrize("k", [1, 40])
+@pytest.mark.parametrize("bad", [3, 150, 300])
+def test_rows_past_the_shared_list_exact(dl, orc, bad, k):
+    g = W.rng(8600 + bad + k)
+    S = np.concatenate([offset(g, 20_000, 16), W.dirichlet_histograms(g, 9000, 16)])
+    Q = np.concatenate([offset(g, bad, 16), W.dirichlet_histograms(g, 300 - bad, 16)])
+    st = check_topk(dl, orc, Q, S, k)
+    assert st["band_pairs"] <= bad
+
+
+def test_all_rows_past_the_shared_list_in_a_batch(dl, orc):
+    g = W.rng(8650)
+    S, Q = offset(g, 15_000, 24), offset(g, 260, 24)
+    res = dl.batch_join(_store(dl, np.arange(15_000), S), np.arange(260), Q,
+                        [{"kind": "topk", "q_begin": 0, "nq": 130, "k": 7}, {"kind": "topk", "q_begin": 130, "nq": 130, "k": 100}])
+    for i, k in ((0, 7), (1, 100)):
+        ids, d2 = res.request_topk(i)
+        oi, od = orc.topk(Q[130 * i:130 * i + 130], S, k)
+        assert (ids == oi).all() and (d2 == od).all()
+    res.free()
