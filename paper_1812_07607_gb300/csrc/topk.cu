@@ -655,7 +655,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     const int f = sh.stride, cap = sh.cap, gran = sh.gran, n_groups = sh.n_groups;
     const int64_t nt_sub = (nt + f - 1) / f, per_cand = sh.per_cand;
     const bool all = n_groups == 0;   // every column fits a row's list: no first pass
-    const int64_t chunk_rows = topk_chunk_rows(rows, sh.bytes());
+    int64_t chunk_rows = topk_chunk_rows(rows, sh.bytes());
 
     const size_t b_rowpar = al256((size_t)rows * sizeof(float4)), b_frows = al256((size_t)nQ * sizeof(int));
     const bool timing = o.timing || tune_trial;
@@ -737,19 +737,30 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                 rc = launched("k_rowpar_topk launch");
             }
         }
-        const int64_t cand_max = chunk_rows * cap + 65536;
-        int64_t cand_cap = std::min<int64_t>(std::min<int64_t>(chunk_rows, nQ) * per_cand + 65536, cand_max);
-        const size_t b_g = al256((size_t)chunk_rows * n_groups * 4), b_l = al256((size_t)chunk_rows * cap * 4),
-                     b_n = al256((size_t)chunk_rows * 4), b_d = al256((size_t)chunk_rows * cap * 8);
+        int64_t cand_cap = 0, cand_max = 0;
+        size_t b_g = 0, b_l = 0, b_n = 0, b_d = 0;
+        auto size_chunk = [&]() {
+            cand_max = chunk_rows * cap + 65536;
+            cand_cap = std::min<int64_t>(std::min<int64_t>(chunk_rows, nQ) * per_cand + 65536, cand_max);
+            b_g = al256((size_t)chunk_rows * n_groups * 4);
+            b_l = al256((size_t)chunk_rows * cap * 4);
+            b_n = al256((size_t)chunk_rows * 4);
+            b_d = al256((size_t)chunk_rows * cap * 8);
+        };
+        size_chunk();
         for (int64_t row0 = 0; row0 < nQ && !rc;) {
             int64_t cr = 0;
             int refined = 0, scans = 0;
             bool redo = false;   // the pass before overflowed the shared list
             for (int pass = 0; !rc; ++pass) {   // listing passes over this chunk
-                if (!cws) {
+                while (!cws) {
                     rc = dev_alloc(&cws, b_g + 3 * b_l + b_n + b_d + (size_t)cand_cap * 8, st);
-                    if (rc) break;
+                    if (rc != DL_ENOMEM || chunk_rows <= 128) break;
+                    chunk_rows = std::max<int64_t>(128, chunk_rows / 256 * 128);   // memory is short: fewer rows at a time
+                    size_chunk();
+                    clear_error();
                 }
+                if (rc) break;
                 cr = std::min(chunk_rows, nQ - row0);
                 const int64_t cr_pad = (cr + 127) / 128 * 128;
                 float *gmax = (float *)cws;

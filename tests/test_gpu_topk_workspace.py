@@ -1,4 +1,4 @@
-"""The top-k's workspace is bounded whatever the data.
+"""The top-k's workspace is bounded whatever the data, and follows what the device has left.
 
 Where the 16-bit bound exceeds the spread of the distances (rows with a large common offset), a row's
 threshold admits every column. The candidates then have to stay within the workspace's limit, the
@@ -67,3 +67,24 @@ def test_all_rows_past_the_shared_list_in_a_batch(dl, orc):
         oi, od = orc.topk(Q[130 * i:130 * i + 130], S, k)
         assert (ids == oi).all() and (d2 == od).all()
     res.free()
+
+
+def test_short_memory_takes_fewer_rows_at_a_time():
+    """A call whose lists would take a gigabyte, on a device with a third of one left."""
+    same, = run("""
+import torch
+from paper_1812_07607_gb300 import dl
+g = torch.Generator(device="cuda"); g.manual_seed(6)
+X = torch.rand(60000, 16, generator=g, device="cuda")
+st = lambda x: dl.Store(torch.arange(len(x), device="cuda"), x)
+Q, S = st(X[:16000].contiguous()), st(X)
+def call(Q):
+    r = dl.topk_join(Q, S, 512); a = r.topk_host(); r.free(); return a
+small = call(st(X[:200].contiguous()))          # modules loaded, little in the pool
+free = torch.cuda.mem_get_info()[0]
+out = 16000 * 512 * 16
+hold = torch.empty(free - out - (340 << 20), dtype=torch.uint8, device="cuda")
+ids, d2 = call(Q)
+print(bool((ids[:200] == small[0]).all() and (d2[:200] == small[1]).all() and (ids >= 0).all()))
+""")
+    assert same == "True"
