@@ -69,15 +69,22 @@ struct Server {
     int64_t done = 0, failed = 0, batches = 0, batched_requests = 0, admit_waits = 0;
 };
 
-// Device-memory estimate of one request inside a batch (queries, output, workspace).
-static int64_t estimate_bytes(const dl_store *S, int32_t kind, int64_t nq, int32_t k)
+// Device-memory estimate of one request inside a batch (queries, output, workspace). `refuse_by` is what
+// the budget is compared with to refuse a request for good: a top-k's lists are cut to the memory there is,
+// so it is never more than 16 slots of a k-entry heap and a list of 4 k (64 at least) a row, the line
+// that requests have always been refused by.
+static int64_t estimate_bytes(const dl_store *S, int32_t kind, int64_t nq, int32_t k, int64_t *refuse_by)
 {
     const int64_t d = S->d, dp = S->dp;
     int64_t b = nq * (d * 4 + dp * 2 + 64) * 2;           // uploaded + internal query store
     if (kind == DL_REQ_TOPK) {
-        b += nq * k * 16 + topk_scratch_bytes(nq, S->n, S->dp, k);   // output + group maxima, lists, candidates
+        const int64_t lists = topk_scratch_bytes(nq, S->n, S->dp, k);   // group maxima, lists, candidates
+        b += nq * k * 16;                                  // output
+        *refuse_by = b + std::min(lists, nq * 16 * (k * 4 + std::max<int64_t>(64, 4 * k) * 8));
+        b += lists;
     } else {
         b += nq * 16 * 1024 + (1 << 20);                   // output / candidates, grown on demand
+        *refuse_by = b;
     }
     return b;
 }
@@ -321,10 +328,11 @@ int dl_submit(dl_server *sv, const int64_t *q_ids, const float *q_feats, int64_t
     q->nq = nq;
     q->ids.assign(q_ids, q_ids + nq);
     q->feats.assign(q_feats, q_feats + nq * sv->S->d);
-    q->est_bytes = estimate_bytes(sv->S, kind, nq, q->k);
-    if (q->est_bytes > sv->budget) {
+    int64_t refuse_by = 0;
+    q->est_bytes = std::min(estimate_bytes(sv->S, kind, nq, q->k, &refuse_by), sv->budget);
+    if (refuse_by > sv->budget) {
         set_error("dl_submit: request needs ~%lld bytes, more than the server budget %lld",
-                  (long long)q->est_bytes, (long long)sv->budget);
+                  (long long)refuse_by, (long long)sv->budget);
         return DL_ENOMEM_ADMIT;
     }
     q->t_submit = Clock::now();
