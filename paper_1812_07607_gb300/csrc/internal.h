@@ -119,6 +119,7 @@ struct Store {
         const int *nseg = nullptr;       // [tiles] balls of each tile
     } balls[2];
     std::mutex mu;           // guards tmaps and hints
+    float x_max = 0.f;       // largest |x_k| of the store
     float nq_max = 0.f;      // largest ||x||^2 of the store (FP32 sum; used only inside slack terms)
     int64_t hint_pairs = 0;  // last output size seen with this store as R (capacity hint)
     int64_t hint_band = 0;

@@ -5,6 +5,7 @@
 
 #include "emit.cuh"
 #include "internal.h"
+#include "simt_tile.cuh"
 
 namespace dl {
 
@@ -85,6 +86,7 @@ struct SimtParams {
     int exact;          // 0 plain, 1 exact (band output)
     int metric;         // 0 squared L2, 1 L1, 2 chi-square (distances compared with t_acc / t_rej)
     float t_acc, t_rej; // exact thresholds; plain uses t_acc only
+    Chi2Scale chi2;     // metric 2: the features' scale
     JoinOut out;
 };
 int launch_simt_join(SimtParams p, cudaStream_t st);

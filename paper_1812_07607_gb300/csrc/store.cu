@@ -919,6 +919,7 @@ int store_create_impl(dl_store **out, const int64_t *ids, const float *feats, in
         return fail(DL_EINVAL);
     }
     std::memcpy(&s->nq_max, &h_back[5], sizeof s->nq_max);
+    std::memcpy(&s->x_max, &h_back[6], sizeof s->x_max);
     s->h.fmt = half_format(h_back[6], ~h_back[7], &s->h.scale);
     dev_free(tmp, st);
     *out = s;
