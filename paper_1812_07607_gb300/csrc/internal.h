@@ -127,6 +127,12 @@ struct Store {
     bool unit = false;       // rows are the unit-normalized rows of another store (cosine metric)
     int nonneg = 0;          // 0 not checked yet, 1 every feature >= 0, 2 some feature < 0 (chi-square)
     int32_t *clabel = nullptr;   // [n] cluster of each store row (stores from dl_store_cluster), else NULL
+    struct SearchCopy {          // a clustered store's 16-bit rows in norm order, per format (get_search)
+        void *blk = nullptr;
+        Half h;
+        float *beta = nullptr;   // [n_pad]
+        int32_t *row = nullptr;  // [n] store row of each
+    } search[2];
 };
 
 // Create a store; gather == NULL orders rows by norm, else store row i is caller row gather[i].
@@ -161,6 +167,9 @@ int prune_units(const dl_store *R, const dl_store *S, bool upper, int BN, double
 // The store's 16-bit copy in the given format: FP16 only where the store holds it (DL_EUNSUPPORTED
 // otherwise), BF16 always (built on first use where the store holds FP16).
 int get_half(Store *s, int fmt, cudaStream_t st, Half **out);
+// A clustered store's rows once more, in the given format and in norm order (built on first use): what the
+// top-k runs on, whose thresholds want rows that are near each other to lie apart in the store.
+int get_search(Store *s, int fmt, cudaStream_t st, Store::SearchCopy **out);
 // Build (or fetch from the copy's cache) a 2-D tensor map over a 16-bit copy with a box of 64
 // columns x box_rows rows and the 128-byte swizzle.
 int get_tmap(Store *s, Half *h, int box_rows, const CUtensorMap **out);

@@ -1,0 +1,102 @@
+"""Top-k against a store in cluster order does what it does against the same rows in norm order.
+
+Views of one object lie side by side there, and thresholds from maxima of neighbouring columns would let
+most of a cluster into every row's list. As many listing passes have to do as in norm order, no more rows
+may need the exact scan (but for chance: which rows a list misses by little depends on their order), and
+ids and distances stay bit-exact: k from 1 to 100, both 16-bit formats, unit rows (equal norms), a batch,
+and a device without the memory for the copy that the passes run on.
+"""
+
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+from paper_1812_07607_gb300 import workloads as W
+from test_gpu_topk import _store, dl, orc  # noqa: F401 (fixtures)
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def data():
+    g = W.rng(8900)
+    X, label = W.clustered_histograms(g, 70_000, 64, 70, 0.01)
+    X = X[np.argsort(label, kind="stable")]   # 1,000 views an object, side by side for the caller too
+    return X, X[g.choice(70_000, 700, replace=False)] * np.float32(1.0001)
+
+
+def call(dl, Q, S, k, **kw):
+    res = dl.topk_join(Q, S, k, **kw)
+    out = res.topk_host() + (res.stats(),)
+    res.free()
+    return out
+
+
+@pytest.mark.parametrize("precision", ["fp16", "bf16"])
+@pytest.mark.parametrize("k", [1, 10, 100])
+def test_as_in_norm_order(dl, orc, data, k, precision):
+    X, Qh = data
+    sid = np.arange(70_000) * 3 + 7
+    Q, S = _store(dl, np.arange(700), Qh), _store(dl, sid, X).clustered(280, iters=3)
+    ids, d2, st = call(dl, Q, S, k, precision=precision)
+    ids, d2, st = call(dl, Q, S, k, precision=precision)
+    oi, od = orc.topk(Qh[:60], X, k)
+    assert (ids[:60] == sid[oi]).all() and (d2[:60] == od).all()
+    ni, nd, nst = call(dl, Q, _store(dl, sid, X), k, precision=precision)
+    assert (ids == ni).all() and (d2 == nd).all()
+    assert st["band_pairs"] <= 2 * nst["band_pairs"] and st["kernels_launched"] <= nst["kernels_launched"]
+
+
+@pytest.mark.parametrize("k", [1, 10, 100])
+def test_unit_rows(dl, data, k):
+    X, Qh = data
+    Q = _store(dl, np.arange(700), Qh).normalized()
+    N = _store(dl, np.arange(70_000), X).normalized()
+    S = N.clustered(280, iters=3)
+    ids, d2, st = call(dl, Q, S, k, metric="cosine")
+    ni, nd, nst = call(dl, Q, N, k, metric="cosine")
+    assert (ids == ni).all() and (d2 == nd).all()
+    assert st["band_pairs"] <= 2 * nst["band_pairs"] and st["kernels_launched"] <= nst["kernels_launched"]
+
+
+def test_batch(dl, orc, data):
+    X, Qh = data
+    S = _store(dl, np.arange(70_000), X).clustered(280, iters=3)
+    res = dl.batch_join(S, np.arange(700), Qh, [{"kind": "topk", "q_begin": 0, "nq": 300, "k": 10},
+                                                {"kind": "topk", "q_begin": 300, "nq": 400, "k": 100}])
+    for i, (a, n, k) in enumerate(((0, 300, 10), (300, 400, 100))):
+        ids, d2 = res.request_topk(i)
+        oi, od = orc.topk(Qh[a:a + 40], X, k)
+        assert (ids[:40] == oi).all() and (d2[:40] == od).all()
+    res.free()
+
+
+def test_without_memory_for_the_copy():
+    same, = subprocess.run([sys.executable, "-c", """
+import torch
+from paper_1812_07607_gb300 import dl
+g = torch.Generator(device="cuda"); g.manual_seed(6)
+X = torch.rand(1 << 20, 128, generator=g, device="cuda")
+st = lambda x: dl.Store(torch.arange(len(x), device="cuda"), x)
+N, Q = st(X), st(X[:16].contiguous())
+del X
+def call(S):
+    r = dl.topk_join(Q, S, 3); a = r.topk_host(); r.free(); return a
+want = call(N)
+S = N.clustered(4, iters=0)
+free = torch.cuda.mem_get_info()[0]
+hold = torch.empty(free - (160 << 20), dtype=torch.uint8, device="cuda")   # the copy takes 280 MB
+keep = []
+try:   # and what the pool has left over
+    while True:
+        keep.append(dl.Store(torch.arange(1 << 17, device="cuda"), torch.zeros(1 << 17, 128, device="cuda")))
+except Exception:
+    keep = keep[:-1]
+got = call(S)
+print(bool((got[0] == want[0]).all() and (got[1] == want[1]).all()))
+"""], cwd=ROOT, capture_output=True, text=True, timeout=600, check=True).stdout.split()
+    assert same == "True"
