@@ -120,7 +120,8 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
 int launch_diag(const int64_t *ids, int64_t n, int64_t *out_r, int64_t *out_s, unsigned long long *out_cnt,
                 unsigned long long cap, cudaStream_t st);
 
-// What a top-k of nQ rows against nS takes at most for its group maxima, lists and candidates (topk.cu).
+// What a top-k of nQ rows against nS takes for its group maxima, lists and candidates (topk.cu; when the
+// candidates do not fit, a gigabyte in all at most).
 int64_t topk_scratch_bytes(int64_t nQ, int64_t nS, int dp, int k);
 // ---- top-k core (topk.cu): every row of Q against S, outputs at row_off or caller row * k
 int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, const int64_t *row_off,

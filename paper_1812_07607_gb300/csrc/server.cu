@@ -78,7 +78,7 @@ static int64_t estimate_bytes(const dl_store *S, int32_t kind, int64_t nq, int32
     const int64_t d = S->d, dp = S->dp;
     int64_t b = nq * (d * 4 + dp * 2 + 64) * 2;           // uploaded + internal query store
     if (kind == DL_REQ_TOPK) {
-        const int64_t lists = topk_scratch_bytes(nq, S->n, S->dp, k);   // group maxima, lists, candidates
+        const int64_t lists = topk_scratch_bytes(nq, S->n, S->dp, k);   // group maxima, lists, candidates (more: on demand)
         b += nq * k * 16;                                  // output
         *refuse_by = b + std::min(lists, nq * 16 * (k * 4 + std::max<int64_t>(64, 4 * k) * 8));
         b += lists;

@@ -21,10 +21,13 @@
 // overflows again takes
 //   k_topk_fallback    an exact scan of the whole store for that row (FP32 bound + radix select +
 //                      FP64 + rank).
-// The candidates of all rows share one list, which never holds more than the rows' lists do together
-// (rows may list every column where the 16-bit bound exceeds the spread of the distances). When it
-// still overflows, some row holds more than its own list: those are tightened, or go to the exact scan
-// after kTkRefines times, and the others' candidates are listed again.
+// The candidates of all rows share one list, which grows to what is left of kTkWorkspace (and holds at
+// least as much as the rows' lists do together). Where the 16-bit bound exceeds the spread of the
+// distances rows may list every column, and it overflows all the same: then fewer rows are taken at a
+// time, down to 128 (a million candidates each). Past that some row holds more than its own list: those
+// are tightened kTkRedos times, or go to the exact scan, and the others' candidates are listed again.
+// (Bounded by the rows' lists alone, ordinary overflows took that way, with thresholds from the columns
+// listed first: 512 rows, k = 10, against 1,000,000 x 128 in tight clusters 1.7 -> 520 ms.)
 // Store rows are in norm order; outputs are written at the caller's row order. Thresholds from maxima of
 // neighbouring columns of every f-th tile need near rows to be spread over the store. A store in cluster
 // order puts them side by side: the passes over it run on a copy of its 16-bit rows in norm order
@@ -54,8 +57,9 @@ constexpr int kTkTermC = 64;         // candidates whose canonical terms are sta
 constexpr int kTkTerms = kTkTermC * 33;   // staged terms, padding included
 constexpr int kTkRefines = 2;        // passes with tightened thresholds before the exact scan
 constexpr int kTkScan = 1 << 30;     // list count of a row that is left to the exact scan
-constexpr int kTkScanPasses = 4;     // passes that name such rows while the shared list overflows (then: all)
-constexpr int64_t kTkWorkspace = 1LL << 30;   // bytes of lists and candidates of a chunk of query rows, at most
+constexpr int kTkRedos = 2;          // passes with tightened thresholds while the shared list overflows
+constexpr int kTkScanPasses = 4;     // then passes that name rows for the scan while it does (then: all)
+constexpr int64_t kTkWorkspace = 1LL << 30;   // bytes of lists and candidates of a chunk of query rows
 constexpr int kTkFallbackCap = 8192; // candidates a fallback block can rank
 
 // Per query row: {canonical slack of h, unused, ||q - q~|| up, ||q~|| up}; padding rows get zeros.
@@ -270,7 +274,8 @@ __global__ void __launch_bounds__(256) k_topk_refine(const TopkRows f, const dou
 
 // One warp per query row: the columns of its list that can still be in the top k, moved to the list's
 // front (their count becomes the row's) and named in the chunk's kept list. A row whose list
-// overflowed is named in over_rows instead.
+// overflowed is named in over_rows instead (n_over: how many, and above bit 32 those not yet left to the
+// exact scan).
 __global__ void __launch_bounds__(256) k_topk_keep(const TopkRows f, int *__restrict__ over_rows, unsigned long long *__restrict__ n_over)
 {
     constexpr int kReg = 8;   // distances a lane keeps in registers
@@ -280,7 +285,7 @@ __global__ void __launch_bounds__(256) k_topk_keep(const TopkRows f, int *__rest
     for (int64_t lr = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; lr < f.rows; lr += nw) {
         const int m0 = f.cnt[lr];
         if (m0 > f.cap) {
-            if (lane == 0) over_rows[atomicAdd(n_over, 1ULL)] = (int)(f.row0 + lr);
+            if (lane == 0) over_rows[(unsigned)atomicAdd(n_over, m0 < kTkScan ? 1ULL | 1ULL << 32 : 1ULL)] = (int)(f.row0 + lr);
             continue;
         }
         const unsigned kk = (unsigned)(f.row_k ? f.row_k[f.row0 + lr] : f.k);
@@ -583,7 +588,7 @@ struct TopkShape {
     int gran;           // columns of a group
     int n_groups;       // groups of a row (0: every column fits the list, no first pass)
     int64_t per_cand;   // candidates of a row provided for at first (never more than cap)
-    int64_t bytes() const { return 4LL * n_groups + 20LL * cap + 4 + 8LL * cap; }   // of a row, at most
+    int64_t bytes() const { return 4LL * n_groups + 20LL * cap + 4 + 8LL * cap; }   // of a row, its list's candidates included
 };
 
 static TopkShape topk_shape(int64_t nS, int dp, int k, int BN)
@@ -670,7 +675,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     if (rc) return rc;
     float4 *rowpar = (float4 *)ws, *thr = (float4 *)((char *)ws + b_rowpar);
     int *frows = (int *)((char *)ws + 2 * b_rowpar);
-    // [0] rows named in frows [1] fp64 evals [2] more near-ties than the fallback ranks [3] wait expired
+    // [0] rows named in frows (k_topk_keep) [1] fp64 evals [2] more near-ties than the fallback ranks [3] wait expired
     // [4] candidates of a pass [5] columns kept by it
     unsigned long long *misc = (unsigned long long *)((char *)ws + 2 * b_rowpar + b_frows);
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -761,6 +766,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         auto size_chunk = [&]() {
             cand_max = chunk_rows * cap + 65536;
             cand_cap = std::min<int64_t>(std::min<int64_t>(chunk_rows, nQ) * per_cand + 65536, cand_max);
+            cand_max = std::max<int64_t>(cand_max, (kTkWorkspace - chunk_rows * (sh.bytes() - 8LL * cap)) / 8);
             b_g = al256((size_t)chunk_rows * n_groups * 4);
             b_l = al256((size_t)chunk_rows * cap * 4);
             b_n = al256((size_t)chunk_rows * 4);
@@ -769,14 +775,21 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         size_chunk();
         for (int64_t row0 = 0; row0 < nQ && !rc;) {
             int64_t cr = 0;
-            int refined = 0, scans = 0;
+            int refined = 0, redos = 0;
             bool redo = false;   // the pass before overflowed the shared list
             for (int pass = 0; !rc; ++pass) {   // listing passes over this chunk
                 while (!cws) {
                     rc = dev_alloc(&cws, b_g + 3 * b_l + b_n + b_d + (size_t)cand_cap * 8, st);
-                    if (rc != DL_ENOMEM || chunk_rows <= 128) break;
-                    chunk_rows = std::max<int64_t>(128, chunk_rows / 256 * 128);   // memory is short: fewer rows at a time
-                    size_chunk();
+                    if (rc != DL_ENOMEM) break;
+                    // memory is short: a list that is no larger than it must be, then fewer rows at a time
+                    if (cand_cap > chunk_rows * cap + 65536) {
+                        cand_cap = cand_max = chunk_rows * cap + 65536;
+                    } else if (chunk_rows > 128) {
+                        chunk_rows = std::max<int64_t>(128, chunk_rows / 256 * 128);
+                        size_chunk();
+                    } else {
+                        break;
+                    }
                     clear_error();
                 }
                 if (rc) break;
@@ -830,8 +843,8 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                         if (e != cudaSuccess) rc = cuda_fail(e, "top-k memset");
                     }
                 } else {   // tighter thresholds for the rows whose list overflowed, then the exact scan
-                    const int scan = refined < kTkRefines ? 0 : ++scans <= kTkScanPasses ? 1 : 2;
-                    if (!scan) ++refined;
+                    redo ? ++redos : ++refined;
+                    const int scan = !redo || redos <= kTkRedos ? 0 : redos <= kTkRedos + kTkScanPasses ? 1 : 2;
                     k_topk_refine<<<(unsigned)cr_pad, 256, 0, st>>>(t, Q->nq64, Q->dp, g64, cr_pad, redo, scan, rowpar, thr);
                     rc = launched("k_topk_refine launch");
                     if (!rc) rc = reset();
@@ -872,17 +885,24 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                     return done(DL_ETIMEOUT);
                 }
                 redo = h[4] > (unsigned long long)cand_cap;   // lists short of candidates: what came of them is written again
-                if (redo && cand_cap < cand_max) {   // the shared list was too short: its exact size, again
-                    cand_cap = std::min<int64_t>((int64_t)(h[4] + h[4] / 8) + 1024, cand_max);
+                if (redo && (cand_cap < cand_max || chunk_rows > 128)) {   // again, with the list's exact size or fewer rows
+                    const int64_t want = (int64_t)(h[4] + h[4] / 8) + 1024;
+                    if (cand_cap < cand_max) {
+                        cand_cap = std::min(want, cand_max);
+                    } else {
+                        chunk_rows = std::max<int64_t>(128, (int64_t)((double)cr * (double)cand_max / (double)want) / 128 * 128);
+                        size_chunk();
+                        cand_cap = cand_max;
+                    }
                     dev_free(cws, st);
                     cws = nullptr;
                     pass = -1;
-                    refined = scans = 0;
+                    refined = redos = 0;
                     rc = reset();
                     continue;
                 }
-                if (!redo && (h[0] == 0 || refined == kTkRefines)) {
-                    flagged += (int64_t)h[0];
+                if (!redo && ((h[0] >> 32) == 0 || refined == kTkRefines)) {
+                    flagged += (int64_t)(h[0] & 0xffffffffULL);
                     fp64 += (int64_t)h[5];
                     break;
                 }

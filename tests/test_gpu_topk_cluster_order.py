@@ -75,7 +75,7 @@ def test_batch(dl, orc, data):
     res.free()
 
 
-def test_without_memory_for_the_copy():
+def test_without_memory_for_the_copy(dl):
     same, = subprocess.run([sys.executable, "-c", """
 import torch
 from paper_1812_07607_gb300 import dl

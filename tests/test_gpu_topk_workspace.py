@@ -30,7 +30,7 @@ def offset(g, n, d):
     return (1000 + 1e-3 * g.standard_normal((n, d))).astype(np.float32)
 
 
-def test_offset_cluster_memory_is_bounded():
+def test_offset_cluster_memory_is_bounded(dl):
     """1,536 rows that each reach all of 200,000 columns: 2.5 GB as one list of 8-byte candidates."""
     taken, = run("""
 import torch
@@ -57,6 +57,19 @@ def test_rows_past_the_shared_list_exact(dl, orc, bad, k):
     assert st["band_pairs"] <= bad
 
 
+def test_more_columns_than_the_list_ever_holds(dl, orc):
+    """One tile of rows that reach 1.2 million columns each: more than a gigabyte of candidates."""
+    g = W.rng(8640)
+    S = np.concatenate([offset(g, 1_200_000, 8), W.dirichlet_histograms(g, 1000, 8)])
+    Q = np.concatenate([offset(g, 126, 8), W.dirichlet_histograms(g, 4, 8)])
+    res = dl.topk_join(_store(dl, np.arange(130), Q), _store(dl, np.arange(len(S)), S), 3)
+    ids, d2 = res.topk_host()
+    res.free()
+    rows = [0, 1, 60, 125, 126, 129]
+    oi, od = orc.topk(Q[rows], S, 3)
+    assert (ids[rows] == oi).all() and (d2[rows] == od).all()
+
+
 def test_all_rows_past_the_shared_list_in_a_batch(dl, orc):
     g = W.rng(8650)
     S, Q = offset(g, 15_000, 24), offset(g, 260, 24)
@@ -69,7 +82,7 @@ def test_all_rows_past_the_shared_list_in_a_batch(dl, orc):
     res.free()
 
 
-def test_short_memory_takes_fewer_rows_at_a_time():
+def test_short_memory_takes_fewer_rows_at_a_time(dl):
     """A call whose lists would take a gigabyte, on a device with a third of one left."""
     same, = run("""
 import torch
