@@ -87,7 +87,6 @@ __global__ void __launch_bounds__(256) k_hist_dist_few(const HistTk f)
     const int lane = threadIdx.x & 31;
     const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
     const float *Q = f.Q + (size_t)f.row0 * f.d;
-    auto scaled = [&](float x) { return M == 2 ? x * f.cs.up : x; };
     for (int j = w; j < f.nS; j += nw) {
         const float *x = f.S + (size_t)j * f.d;
         for (int r = 0; r < f.rows; ++r) {
@@ -97,14 +96,13 @@ __global__ void __launch_bounds__(256) k_hist_dist_few(const HistTk f)
                 for (int k = lane * 4; k < f.d; k += 128) {
                     const float4 a = __ldg(reinterpret_cast<const float4 *>(q + k));
                     const float4 b = __ldg(reinterpret_cast<const float4 *>(x + k));
-                    dist_terms<M>(scaled(a.x), scaled(a.y), scaled(b.x), scaled(b.y), s);
-                    dist_terms<M>(scaled(a.z), scaled(a.w), scaled(b.z), scaled(b.w), s);
+                    dist_terms<M>(a.x, a.y, b.x, b.y, f.cs, s);
+                    dist_terms<M>(a.z, a.w, b.z, b.w, f.cs, s);
                 }
             } else {
                 for (int k = lane * 2; k < f.d; k += 64) {
                     const bool two = k + 1 < f.d;   // an absent second feature is 0 in both rows: a zero term
-                    dist_terms<M>(scaled(__ldg(q + k)), two ? scaled(__ldg(q + k + 1)) : 0.f, scaled(__ldg(x + k)),
-                                  two ? scaled(__ldg(x + k + 1)) : 0.f, s);
+                    dist_terms<M>(__ldg(q + k), two ? __ldg(q + k + 1) : 0.f, __ldg(x + k), two ? __ldg(x + k + 1) : 0.f, f.cs, s);
                 }
             }
 #pragma unroll

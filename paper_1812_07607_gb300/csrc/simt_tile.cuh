@@ -59,27 +59,6 @@ inline Chi2Scale chi2_scale(float x_max)
 inline double chi2_g32(int d) { return (d + 16) * 1.1920928955078125e-07; }
 inline double chi2_abs32(int d, Chi2Scale c) { return d * 3.552713678800501e-15 * c.down + 1.401298464324817e-45; }
 
-// Adds the terms k and k + 1 of metric M for a pair (a, b) of feature values to acc:
-//   M = 0: squared L2; M = 1: L1; M = 2: chi-square on non-negative features. One reciprocal
-//   serves two chi-square terms: the MUFU unit (16 lanes an SM) would otherwise bound the loop.
-template <int M>
-__device__ __forceinline__ void dist_terms(float a0, float a1, float b0, float b1, float &acc)
-{
-    const float t0 = a0 - b0, t1 = a1 - b1;
-    if constexpr (M == 0) {
-        acc = fmaf(t0, t0, acc);
-        acc = fmaf(t1, t1, acc);
-    } else if constexpr (M == 1) {
-        acc += fabsf(t0);
-        acc += fabsf(t1);
-    } else {
-        const float u0 = fmaxf(a0 + b0, kChi2Floor), u1 = fmaxf(a1 + b1, kChi2Floor);
-        float r;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(u0 * u1));
-        acc = fmaf(fmaf(t1 * t1, u0, (t0 * t0) * u1), r, acc);
-    }
-}
-
 // Packed pairs of floats (add / mul / fma.f32x2): each half rounds as the scalar operation does.
 __device__ __forceinline__ uint64_t pack2(float x, float y)
 {
@@ -105,6 +84,35 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     uint64_t r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+
+// Adds the terms k and k + 1 of metric M for a pair (a, b) of feature values to acc:
+//   M = 0: squared L2; M = 1: L1; M = 2: chi-square on non-negative features, times c.up. One reciprocal
+//   serves two chi-square terms: the MUFU unit (16 lanes an SM) would otherwise bound the loop. Packed:
+//   the two features' scaling, sum and difference take three instructions.
+template <int M>
+__device__ __forceinline__ void dist_terms(float a0, float a1, float b0, float b1, const Chi2Scale c, float &acc)
+{
+    if constexpr (M == 2) {
+        const uint64_t b = pack2(b0, b1), as = mul2(pack2(a0, a1), pack2(c.up, c.up));
+        const uint64_t t = fma2(b, pack2(-c.up, -c.up), as);
+        float u0, u1, s0, s1, r;
+        unpack2(fma2(b, pack2(c.up, c.up), as), u0, u1);
+        u0 = fmaxf(u0, kChi2Floor);
+        u1 = fmaxf(u1, kChi2Floor);
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(u0 * u1));
+        unpack2(mul2(t, t), s0, s1);
+        acc = fmaf(fmaf(s1, u0, s0 * u1), r, acc);
+    } else {
+        const float t0 = a0 - b0, t1 = a1 - b1;
+        if constexpr (M == 0) {
+            acc = fmaf(t0, t0, acc);
+            acc = fmaf(t1, t1, acc);
+        } else {
+            acc += fabsf(t0);
+            acc += fabsf(t1);
+        }
+    }
 }
 
 // dist_terms for two neighbouring columns at once: the row's features twice in a0 / a1, the
