@@ -667,7 +667,7 @@ def rows_leg(dl, sm_mhz=None, reps=5):
         Qs.close()
     Xs.close()
 
-    # the inner-product threshold join on rows of any norm (BF16 tensor cores, exact)
+    # the inner-product threshold join on rows of any norm (16-bit tensor cores, exact)
     g = W.rng(W.SEED_BASE + 120)
     nip, dip = 65536, 128
     Rip = (g.standard_normal((nip, dip)) * 2.0 ** g.uniform(-1.0, 1.0, (nip, 1))).astype(np.float32)
@@ -696,7 +696,7 @@ def rows_leg(dl, sm_mhz=None, reps=5):
                             "roofline": {"bound": "tensor", "achieved": 2.0 * dip * P / (kern_ms / 1e3) / 1e12,
                                          "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
                                          "frac": 2.0 * dip * P / (kern_ms / 1e3) / 1e12 / pk["bf16_tflops"],
-                                         "kernel": "tc_join_kernel<256> (BF16, zero column term)"}}
+                                         "kernel": "tc_join_kernel<256> (FP16, zero column term)"}}
     Rs_ip.close()
     Ss_ip.close()
     del Rip, Sip

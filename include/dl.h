@@ -71,7 +71,8 @@ typedef enum dl_precision {
     DL_PREC_AUTO = 0,       /* ε-join: FP16 tensor-core path when d <= 512 (BF16 when a store's features
                                span too wide a range), else FP8 e4m3, or FP16 for large joins;
                                top-k: FP16 or BF16 when d <= 512, else FP32 */
-    DL_PREC_BF16 = 1,       /* -2 q.x on tcgen05 tensor cores in BF16, FP32 accumulate; exact result */
+    DL_PREC_BF16 = 1,       /* -2 q.x on tcgen05 tensor cores in BF16, FP32 accumulate; exact result
+                               (a store whose 16-bit copy is FP16 adds a BF16 one on first use) */
     DL_PREC_FP8E4M3 = 2,    /* as BF16 but FP8 e4m3 with power-of-two scales (per 32-row chunk of
                                each store); exact result */
     DL_PREC_FP32 = 3,       /* FP32 SIMT distances + bound + FP64 recheck; exact result */
@@ -230,9 +231,10 @@ int dl_dedup(const dl_store *X, int32_t metric, double eps, const int32_t *label
  * run with DL_PREC_FP32 (AUTO picks it) or DL_PREC_FP32_PLAIN (BF16 / FP8 give
  * DL_EUNSUPPORTED), and CHI2 gives DL_EINVAL when a feature is negative. With
  * DL_METRIC_IP, eps is the inner-product threshold t (any value but NaN; -inf returns
- * every pair, +inf none); it runs on the BF16 tensor-core path (AUTO picks it), for
- * R x S and the upper self mode, without pruning (FP32 / FP8 precisions, the full self
- * mode and opts->prune give DL_EUNSUPPORTED). opts may be
+ * every pair, +inf none); it runs on the 16-bit tensor-core path (AUTO: FP16 where both
+ * stores hold it and one has more than 1,024 rows, else BF16; or DL_PREC_BF16), d <= 512, for R x S and the upper self mode,
+ * without pruning (other precisions, the full self mode and opts->prune give
+ * DL_EUNSUPPORTED). opts may be
  * NULL (defaults). On success *out holds the result (free with
  * dl_result_free); on DL_EOVERFLOW *out is also set so that the required
  * count can be read. The pair order is unspecified (the result is a set).

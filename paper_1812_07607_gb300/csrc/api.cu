@@ -243,7 +243,8 @@ static int run_pass(const PassCfg &c, PassOut *po)
                 rc = get_half(const_cast<dl_store *>(R), fmt, st, &hR);
                 if (!rc) rc = get_half(const_cast<dl_store *>(S), fmt, st, &hS);
             }
-            if (!rc && c.ip) rc = ensure_ip(const_cast<dl_store *>(S), st);
+            const Store::IpColumns *ipc = nullptr;
+            if (!rc && c.ip) rc = get_ip(const_cast<dl_store *>(S), hS, st, &ipc);
             if (!rc && c.ip)
                 rc = launch_rowpar_ip(hR->rowb, nR, rows_pad, R->dp, c.e2, rowpar, st);
             else if (!rc)
@@ -285,8 +286,8 @@ static int run_pass(const PassCfg &c, PassOut *po)
                 tc_plan(c.BN, L.p.kc, &L.p.stages, &L.p.a_slots, fp8, c.cg2, c.wide, !c.pruned);
                 L.p.upper = c.self ? 1 : 0;
                 L.p.rowpar = rowpar;
-                L.p.beta = c.ip ? S->beta_ip : S->beta;
-                L.p.cstat = fp8 ? S->cstat8 : (c.ip ? S->cstat_ip : hS->cstat);
+                L.p.beta = c.ip ? ipc->beta : S->beta;
+                L.p.cstat = fp8 ? S->cstat8 : (c.ip ? ipc->cstat : hS->cstat);
                 L.p.sc_r = fp8 ? R->sc8 : nullptr;
                 L.p.sc_s = fp8 ? S->scc8 : nullptr;
                 L.p.cand = band;                 // candidates share the band buffer and counter
@@ -381,6 +382,12 @@ static double g_rate_out = 0.0, g_rate_band = 0.0;
 // 700, d = 640: 63 us, FP8 86; 2,000 x 2,000: 64 and 199), but small joins keep the FP8 path that AUTO
 // has always documented and reported for these widths; here it costs 20 us, further up milliseconds.
 constexpr double kWideF16Pairs = 262144.0;   // 2^18
+
+// The inner-product join under AUTO takes FP16 when a store has more rows than this. BF16 makes a store that
+// holds FP16 build and keep a second copy, 2 d_p bytes a row and a pass over its rows (256 rows against n x
+// 128, first call: FP16 67, 67 and 82 us at n = 8,192, 65,536 and 262,144, BF16 104, 166 and 362). Below the
+// line that is 30 us once, and small joins keep the format that AUTO has always reported for them.
+constexpr int64_t kIpF16Rows = 1024;
 
 static int check_device(const dl_store *s)
 {
@@ -490,15 +497,15 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
         if (hmetric)
             prec = DL_PREC_FP32;
         else if (ip)
-            prec = DL_PREC_BF16;
+            prec = f16 && R->dp <= 512 && std::max(R->n, Sx->n) > kIpF16Rows ? DL_PREC_FP16 : DL_PREC_BF16;
         else if (R->dp <= 512)
             prec = f16 ? DL_PREC_FP16 : DL_PREC_BF16;
         else
             prec = f16 && !o.prune && o.cta_pair != 2 && (double)R->n * (double)Sx->n >= kWideF16Pairs ? DL_PREC_FP16
                                                                                                        : DL_PREC_FP8E4M3;
     }
-    if (ip && (prec != DL_PREC_BF16 || (self && o.self_mode == DL_SELF_FULL) || o.prune)) {
-        set_error("dl_sim_join: the inner-product join runs in BF16, R x S or the upper self mode, without pruning");
+    if (ip && ((o.precision != DL_PREC_AUTO && prec != DL_PREC_BF16) || (self && o.self_mode == DL_SELF_FULL) || o.prune)) {
+        set_error("dl_sim_join: the inner-product join runs in DL_PREC_AUTO or BF16, R x S or the upper self mode, without pruning");
         return DL_EUNSUPPORTED;
     }
     if (hmetric && tc_prec(prec)) {

@@ -739,19 +739,18 @@ int get_search(Store *s, int fmt, cudaStream_t st, Store::SearchCopy **out)
     return DL_OK;
 }
 
-// The inner-product join's column term is 0: h = q.x. Its chunk stats are those of the BF16 copy, so
-// P1 and P2 (the encoding and accumulation terms of the bound) are the store's own and P3 keeps the
+// The inner-product join's column term is 0: h = q.x. Its chunk stats are those of the 16-bit copy, so
+// P1 and P2 (the encoding and accumulation terms of the bound) are the copy's own and P3 keeps the
 // L2 beta error (a conservative extra); padding rows get +inf, so they never match.
-int ensure_ip(Store *s, cudaStream_t st)
+int get_ip(Store *s, const Half *h, cudaStream_t st, const Store::IpColumns **out)
 {
-    Half *h = nullptr;
-    int rc = get_half(s, kHalfBF16, st, &h);
-    if (rc) return rc;
     std::lock_guard<std::mutex> lk(s->mu);
-    if (s->ip_block) return DL_OK;
+    Store::IpColumns &c = s->ip[h->fmt];
+    *out = &c;
+    if (c.blk) return DL_OK;
     const size_t b_b = align256(sizeof(float) * s->n_pad), b_cs = align256(sizeof(float4) * (s->n_pad / 32));
     void *blk = nullptr;
-    rc = dev_alloc(&blk, b_b + b_cs, st);
+    const int rc = dev_alloc(&blk, b_b + b_cs, st);
     if (rc) return rc;
     float *beta_ip = (float *)blk;
     float4 *cstat_ip = (float4 *)((char *)blk + b_b);
@@ -765,9 +764,9 @@ int ensure_ip(Store *s, cudaStream_t st)
         dev_free(blk, st);
         return cuda_fail(e, "inner-product column arrays");
     }
-    s->beta_ip = beta_ip;
-    s->cstat_ip = cstat_ip;
-    s->ip_block = blk;
+    c.beta = beta_ip;
+    c.cstat = cstat_ip;
+    c.blk = blk;
     return DL_OK;
 }
 
@@ -1185,7 +1184,8 @@ int dl_store_destroy(dl_store *s)
     dev_free(s->ids, 0);   // ids is the base of the store's single allocation
     if (s->fp8_block) dev_free(s->fp8_block, 0);
     if (s->alt_block) dev_free(s->alt_block, 0);
-    if (s->ip_block) dev_free(s->ip_block, 0);
+    for (auto &c : s->ip)
+        if (c.blk) dev_free(c.blk, 0);
     if (s->clabel) dev_free(s->clabel, 0);
     for (auto &c : s->search)
         if (c.blk) dev_free(c.blk, 0);
