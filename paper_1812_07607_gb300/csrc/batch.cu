@@ -378,7 +378,8 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
         }
         stats.precision = fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
         bool tune_trial = false;
-        const int code = o.tile_n ? o.tile_n : tune_pick(Qe->dp, kTuneBatch, ne, S->n, &tune_trial);
+        const int tune_kind = fmt == kHalfF16 ? kTuneBatch16 : kTuneBatch;
+        const int code = o.tile_n ? o.tile_n : tune_pick(Qe->dp, tune_kind, ne, S->n, &tune_trial);
         const int BN = tune_bn(code);
         const bool wide = tune_wide(code);
         stats.tile_n = BN;   // the epsilon rows' configuration (the autotuner's choice once decided)
@@ -511,7 +512,7 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
             if (!rc && tune_trial && attempt == 0) {
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, tev[0], tev[1]);
-                tune_record(Qe->dp, kTuneBatch, ne, S->n, code, ms, (double)ne * (double)S->n);
+                tune_record(Qe->dp, tune_kind, ne, S->n, code, ms, (double)ne * (double)S->n);
             }
             dev_free(ws, st);
             break;

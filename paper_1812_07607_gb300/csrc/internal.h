@@ -202,7 +202,7 @@ int pinned_counters(unsigned long long **p);
 constexpr int kTunePair = 1 << 12;
 constexpr int kTuneWide = 1 << 13;
 enum TuneKind { kTuneEpsRxS = 0, kTuneEpsSelf = 1, kTuneTopk = 2, kTuneEpsRxS8 = 3, kTuneEpsSelf8 = 4, kTuneBatch = 5,
-                kTuneEpsRxS16 = 6, kTuneEpsSelf16 = 7 };
+                kTuneEpsRxS16 = 6, kTuneEpsSelf16 = 7, kTuneTopk16 = 8, kTuneBatch16 = 9 };   // 16: FP16; 8: FP8; else BF16
 inline int tune_bn(int code) { return code & 0xfff; }
 inline bool tune_pair(int code) { return (code & kTunePair) != 0; }
 inline bool tune_wide(int code) { return (code & kTuneWide) != 0; }

@@ -645,6 +645,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         return DL_EINVAL;
     }
     int code = (o.tile_n ? o.tile_n : 256) | (o.epilogue_warps == 16 ? kTuneWide : 0);
+    const int tune_kind = fmt == kHalfF16 ? kTuneTopk16 : kTuneTopk;
     const int prec = !use_tc ? DL_PREC_FP32 : fmt == kHalfF16 ? DL_PREC_FP16 : DL_PREC_BF16;
     if (nQ == 0) {   // no rows: nothing to run, time or tune
         if (stats) {
@@ -654,7 +655,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
         }
         return DL_OK;
     }
-    if (use_tc && o.tile_n == 0 && o.epilogue_warps == 0) code = tune_pick(Q->dp, kTuneTopk, nQ, nS, &tune_trial);
+    if (use_tc && o.tile_n == 0 && o.epilogue_warps == 0) code = tune_pick(Q->dp, tune_kind, nQ, nS, &tune_trial);
     const int BN = tune_bn(code);
     const bool wide = use_tc && tune_wide(code);   // 16 epilogue warps
     const int sms = device_sm_count();
@@ -987,7 +988,7 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
     if (tune_trial && flagged == 0) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, ev[0], ev[1]);
-        tune_record(Q->dp, kTuneTopk, nQ, nS, code, ms, (double)nQ * (double)nS);
+        tune_record(Q->dp, tune_kind, nQ, nS, code, ms, (double)nQ * (double)nS);
     }
     return done(DL_OK);
 }

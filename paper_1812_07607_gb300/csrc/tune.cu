@@ -3,14 +3,15 @@
 // A configuration is a code: the tile width (128 or 256 columns) plus kTunePair when the tile
 // runs on a pair of SMs (tcgen05 cta_group::2, 256-row tiles) or kTuneWide for the 16-warp
 // epilogue (which wins when many chunks hold candidates). A tuning key is a shape class:
-// (device SMs, padded d, join kind, log2 |R|, log2 |S|). Each kind has its own candidate list;
+// (device SMs, padded d, join kind and operand format, log2 |R|, log2 |S|). Each kind has its own candidate list;
 // the first calls of a class run every candidate once, then the first candidate again (its
 // first run is the class's cold call), with CUDA-event timing of the tensor-core kernel. A
 // candidate's best kernel milliseconds per 10^9 pairs counts, and from then on the fastest is
 // used. The shared-memory plan (stages, resident R-tile slots) follows from the configuration
-// and d (tc_plan); top-k's S-split count follows from the grid. Decisions are kept for the
+// and d (tc_plan), the work units from the grid (tc_grid_units). Decisions are kept for the
 // process and, when the environment variable DL_TUNE_CACHE names a file, loaded from and
-// appended to it as lines "key code".
+// appended to it as lines "key code". The key starts with a version: what older kernels were timed
+// with does not decide for these.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -51,6 +52,7 @@ std::vector<int> candidates(int kind)
     case kTuneEpsSelf16:
         return {256, 256 | kTuneWide, 128};
     case kTuneBatch:
+    case kTuneBatch16:
         return {256, 256 | kTuneWide};
     default:   // top-k: single-SM tiles
         return {256, 128, 256 | kTuneWide};
@@ -73,8 +75,9 @@ int ilog2(int64_t x)
 std::string make_key(int dp, int kind, int64_t nR, int64_t nS)
 {
     char buf[96];
-    const int lr = (kind == kTuneBatch || kind == kTuneTopk) ? ilog2(nR) / 2 * 2 : ilog2(nR);
-    std::snprintf(buf, sizeof buf, "sm%d:dp%d:k%d:r%d:s%d", device_sm_count(), dp, kind, lr, ilog2(nS));
+    const bool wide = kind == kTuneBatch || kind == kTuneBatch16 || kind == kTuneTopk || kind == kTuneTopk16;
+    const int lr = wide ? ilog2(nR) / 2 * 2 : ilog2(nR);
+    std::snprintf(buf, sizeof buf, "v2:sm%d:dp%d:k%d:r%d:s%d", device_sm_count(), dp, kind, lr, ilog2(nS));
     return buf;
 }
 
