@@ -355,7 +355,8 @@ typedef struct dl_request {
  * epsilon-join rows run in one persistent tensor-core launch (each row with its
  * request's eps), all top-k rows in another (each row with its request's k),
  * then the outputs are routed per request. Each request's result is the set (or
- * ordered list) the single-request call would return. On success *out holds a
+ * ordered list) the single-request call would return. DL_PREC_FP16 is taken as AUTO
+ * (FP16 where the store and the batch's rows hold it, else BF16). On success *out holds a
  * batch result; read it with dl_result_request_pairs / dl_result_request_topk.
  */
 int dl_batch_join(const dl_store *S, const int64_t *q_ids, const float *q_feats, int64_t nq_total, int32_t d,

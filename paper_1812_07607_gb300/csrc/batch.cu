@@ -527,6 +527,8 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
         }
     }
     // ---- top-k part
+    dl_join_opts tko = o;   // FP16 where both stores hold it: one request's rows refuse no other's
+    if (tko.precision == DL_PREC_FP16) tko.precision = DL_PREC_AUTO;
     for (const auto &grp : kgroups) {
         const int kg = grp.first;
         const int64_t g0 = grp.second.first, g1 = grp.second.second;
@@ -537,7 +539,7 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
             stores.push_back(Qk);
             dl_join_stats ts{};
             rc = topk_core(Qk, S, kg, row_k + g0, row_off + g0, (int64_t *)tk_block,
-                           (double *)((char *)tk_block + al(slots * 8)), o, st, &ts);
+                           (double *)((char *)tk_block + al(slots * 8)), tko, st, &ts);
             stats.fp64_pairs += ts.fp64_pairs;
         }
         if (rc) {
