@@ -541,6 +541,7 @@ extern "C" int dl_batch_join(const dl_store *S, const int64_t *q_ids, const floa
             rc = topk_core(Qk, S, kg, row_k + g0, row_off + g0, (int64_t *)tk_block,
                            (double *)((char *)tk_block + al(slots * 8)), tko, st, &ts);
             stats.fp64_pairs += ts.fp64_pairs;
+            if (ne == 0 || S->n == 0) stats.precision = ts.precision;   // otherwise the epsilon rows'
         }
         if (rc) {
             dev_free(tk_block, st);

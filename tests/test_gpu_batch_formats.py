@@ -32,3 +32,14 @@ def test_fp16_server_answers_wide_rows_beside_others(dl, orc):
         assert (ids == oi).all() and (d2 == od).all()
         res.free()
     sv.close()
+
+
+@pytest.mark.parametrize("rows,want", [("near", "DL_PREC_FP16"), ("wide", "DL_PREC_BF16")])
+@pytest.mark.parametrize("kinds", [("topk",), ("eps",), ("eps", "topk")])
+def test_reported_precision(dl, rows, want, kinds):
+    S, near, wide = data()
+    Q = near if rows == "near" else wide
+    res = dl.batch_join(_store(dl, np.arange(3000), S), np.arange(30), Q,
+                        [{"kind": kind, "q_begin": 0, "nq": 30, "k": 4, "eps": 0.1} for kind in kinds])
+    assert res.stats()["precision"] == getattr(dl, want)
+    res.free()
