@@ -341,11 +341,20 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
     // rows per chunk: about 256 MB of distances (rows padded to whole 128-column tiles)
     f.ld = (nS + kSimtTile - 1) / kSimtTile * kSimtTile;
     const int64_t per_row = std::max<int64_t>(f.ld * 4, 256);
-    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(nQ, std::min<int64_t>((256LL << 20) / per_row, 65535LL * kSimtTile)));
-    const int sel = (int)std::min<int64_t>(rows, (int64_t)device_sm_count() * 4);   // CTAs of k_hist_select
+    int64_t rows = std::max<int64_t>(1, std::min<int64_t>(nQ, std::min<int64_t>((256LL << 20) / per_row, 65535LL * kSimtTile)));
+    int sel = 1;   // CTAs of k_hist_select
     void *blk = nullptr;
-    const size_t b_v = al256((size_t)rows * f.ld * 4), b_c = al256((size_t)sel * kHtCap * 4), b_d = al256((size_t)sel * kHtCap * 8);
-    int rc = dev_alloc(&blk, b_v + 2 * b_c + b_d + 256, st);
+    size_t b_v = 0, b_c = 0, b_d = 0;
+    int rc = DL_OK;
+    for (;; rows = (rows + 1) / 2) {   // fewer where memory is short
+        sel = (int)std::min<int64_t>(rows, (int64_t)device_sm_count() * 4);
+        b_v = al256((size_t)rows * f.ld * 4);
+        b_c = al256((size_t)sel * kHtCap * 4);
+        b_d = al256((size_t)sel * kHtCap * 8);
+        rc = dev_alloc(&blk, b_v + 2 * b_c + b_d + 256, st);
+        if (rc != DL_ENOMEM || rows == 1) break;
+        clear_error();
+    }
     if (rc) return rc;
     f.dist = (float *)blk;
     f.scr_c = (uint32_t *)((char *)blk + b_v);
