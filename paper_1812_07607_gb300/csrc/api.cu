@@ -156,7 +156,7 @@ struct PassCfg {
     bool pruned = false;           // the pruned join (units may be empty: every tile pair skipped)
     bool ip = false;               // inner-product join: e2 holds the threshold t of q.x >= t
     float t_acc, t_rej;     // FP32 thresholds (exact: recheck/SIMT; plain: SIMT only)
-    Chi2Scale chi2;         // chi-square: the features' scale
+    float up = 1.f;         // chi-square: the features' scale, and that of t_acc and t_rej
     int64_t cap, band_cap;
     bool timing;
     cudaStream_t st;
@@ -308,7 +308,7 @@ static int run_pass(const PassCfg &c, PassOut *po)
             sp.tiles_m = 0;
             sp.exact = (c.prec == DL_PREC_FP32) ? 1 : 0;
             sp.metric = c.metric;
-            sp.chi2 = c.chi2;
+            sp.up = c.up;
             sp.t_acc = c.t_acc;
             sp.t_rej = c.t_rej;
             sp.out = jo;
@@ -582,9 +582,9 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
     c.metric = hmetric;
     c.ip = ip;
     c.ids = emit_ids;
-    c.chi2 = chi2_scale(std::max(R->x_max, Sx->x_max));
+    if (hmetric == 2) c.up = chi2_scale(std::max(R->x_max, Sx->x_max));
     if (prec == DL_PREC_FP32_PLAIN && hmetric) {
-        c.t_acc = (float)eps;
+        c.t_acc = (float)eps * c.up;
         c.t_rej = c.t_acc;
     } else if (prec == DL_PREC_FP32_PLAIN) {
         const float ef = (float)std::sqrt(e2);
@@ -594,9 +594,10 @@ int sim_join_impl(const dl_store *R, const dl_store *S, int32_t metric, double e
         // |D32 - D| <= g32 D + abs32 for the SIMT evaluation, |D64 - D| <= g64 D for the canonical sum
         const double g64 = (hmetric == 1) ? gamma64(d) : gamma64(d + 4);
         const double g32 = (hmetric == 1) ? (d + 4) * 1.1920928955078125e-07 : chi2_g32(d);
-        const double abs32 = (hmetric == 1) ? d * 7.52316384526264e-37 : chi2_abs32(d, c.chi2);   // L1: d 2^-120
-        c.t_acc = f32_rd(eps * (1.0 - g64) * (1.0 - g32) * (1.0 - 8.881784197001252e-16) - abs32);
-        c.t_rej = f32_ru(eps * (1.0 + 2.0 * g64) * (1.0 + g32) * (1.0 + 8.881784197001252e-16) + abs32);
+        const double abs32 = (hmetric == 1) ? d * 7.52316384526264e-37 : chi2_abs32(d);   // L1: d 2^-120
+        const double t = eps * c.up;
+        c.t_acc = f32_rd(t * (1.0 - g64) * (1.0 - g32) * (1.0 - 8.881784197001252e-16) - abs32);
+        c.t_rej = f32_ru(t * (1.0 + 2.0 * g64) * (1.0 + g32) * (1.0 + 8.881784197001252e-16) + abs32);
     } else {
         const double g64 = gamma64(d), g32 = gamma32(d);
         const double abs32 = (double)(d + 8) * 1.401298464324817e-45 * 2.0;

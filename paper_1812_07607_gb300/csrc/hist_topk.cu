@@ -54,7 +54,7 @@ struct HistTk {
     int64_t *out_ids;
     double *out_d;
     float g32, a32, slack;
-    Chi2Scale cs;             // chi-square: the features' scale
+    float up;                 // chi-square: the features' scale, and that of `dist`
     int *err;
     unsigned long long *n_fp64;
 };
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(256, 2) k_hist_dist(const HistTk f)
     __shared__ __align__(16) SimtSmem sm;
     const int r0 = blockIdx.y * kSimtTile, c0 = blockIdx.x * kSimtTile;
     float acc[8][8];
-    simt_tile<M, VEC>(f.Q + (size_t)f.row0 * f.d, f.S, f.rows, f.nS, f.d, r0, c0, f.cs, sm, acc);
+    simt_tile<M, VEC>(f.Q + (size_t)f.row0 * f.d, f.S, f.rows, f.nS, f.d, r0, c0, f.up, sm, acc);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -96,18 +96,18 @@ __global__ void __launch_bounds__(256) k_hist_dist_few(const HistTk f)
                 for (int k = lane * 4; k < f.d; k += 128) {
                     const float4 a = __ldg(reinterpret_cast<const float4 *>(q + k));
                     const float4 b = __ldg(reinterpret_cast<const float4 *>(x + k));
-                    dist_terms<M>(a.x, a.y, b.x, b.y, f.cs, s);
-                    dist_terms<M>(a.z, a.w, b.z, b.w, f.cs, s);
+                    dist_terms<M>(a.x, a.y, b.x, b.y, f.up, s);
+                    dist_terms<M>(a.z, a.w, b.z, b.w, f.up, s);
                 }
             } else {
                 for (int k = lane * 2; k < f.d; k += 64) {
                     const bool two = k + 1 < f.d;   // an absent second feature is 0 in both rows: a zero term
-                    dist_terms<M>(__ldg(q + k), two ? __ldg(q + k + 1) : 0.f, __ldg(x + k), two ? __ldg(x + k + 1) : 0.f, f.cs, s);
+                    dist_terms<M>(__ldg(q + k), two ? __ldg(q + k + 1) : 0.f, __ldg(x + k), two ? __ldg(x + k + 1) : 0.f, f.up, s);
                 }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) f.dist[(size_t)r * f.ld + j] = M == 2 ? s * f.cs.down : s;
+            if (lane == 0) f.dist[(size_t)r * f.ld + j] = s;
         }
     }
 }
@@ -320,8 +320,7 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
     if (nQ == 0) return DL_OK;
     // the SIMT join's bounds (|D32 - D| <= g32 D + a32) and the canonical sum's relative error g64
     const double g32 = metric == 1 ? (d + 4) * 1.1920928955078125e-07 : chi2_g32(d);
-    const Chi2Scale cs = chi2_scale(std::max(Q->x_max, S->x_max));
-    const double a32 = metric == 1 ? d * 7.52316384526264e-37 : chi2_abs32(d, cs);   // L1: d 2^-120
+    const double a32 = metric == 1 ? d * 7.52316384526264e-37 : chi2_abs32(d);   // L1: d 2^-120
     const double g64 = (metric == 1 ? d + 4 : d + 8) * 1.1102230246251565e-16;
     HistTk f{};
     f.Q = Q->x32;
@@ -336,7 +335,7 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
     f.out_d = out_d;
     f.g32 = f32_ru(g32);
     f.a32 = f32_ru(a32);
-    f.cs = cs;
+    f.up = chi2_scale(std::max(Q->x_max, S->x_max));
     f.slack = f32_ru(4.0 * g64 + 1e-12);   // (1 + g64) / (1 - g64) and this product's roundings
     // rows per chunk: about 256 MB of distances (rows padded to whole 128-column tiles)
     f.ld = (nS + kSimtTile - 1) / kSimtTile * kSimtTile;

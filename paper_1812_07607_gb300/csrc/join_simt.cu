@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256, 2) k8_simt_join(const SimtParams p)
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 
     float acc[8][8];
-    simt_tile<M, VEC>(p.R, p.S, p.nR, p.nS, p.d, r0, c0, p.chi2, sm, acc);
+    simt_tile<M, VEC>(p.R, p.S, p.nR, p.nS, p.d, r0, c0, p.up, sm, acc);
 
     // classify: the common case is "no candidate anywhere in this thread's 64 pairs"
     bool any = false;

@@ -86,7 +86,7 @@ struct SimtParams {
     int exact;          // 0 plain, 1 exact (band output)
     int metric;         // 0 squared L2, 1 L1, 2 chi-square (distances compared with t_acc / t_rej)
     float t_acc, t_rej; // exact thresholds; plain uses t_acc only
-    Chi2Scale chi2;     // metric 2: the features' scale
+    float up;           // metric 2: the features' scale, and the thresholds'
     JoinOut out;
 };
 int launch_simt_join(SimtParams p, cudaStream_t st);

@@ -35,29 +35,26 @@ constexpr float kChi2Floor = 8.8817841970012523e-16f;   // 2^-50
 
 // Chi-square distances scale with the features, the clamp does not: the features enter the tile times a
 // power of two that brings the two stores' largest just below 2^40 (the domain's end, so nothing grows
-// past it), and distances are scaled back. The clamp then lies 2^90 below the largest feature. Without
+// past it), and distances are compared at that scale. The clamp then lies 2^90 below the largest feature. Without
 // it rows that sum to 1e-12, or rows of any sum that differ by 1e-6 of it, lay within the clamp's error
-// of each other. Sixteen multiplications a thread and slice: chi-square top-10 of 1,000 rows against
-// 65,536 x 128 1,765 us without, 1,769 with (runs of one side differ by 0.3%).
-struct Chi2Scale {
-    float up = 1.f, down = 1.f;
-};
-inline Chi2Scale chi2_scale(float x_max)
+// of each other. The rows' features are scaled when they are staged, the columns' within the FMAs that
+// form a difference and a sum: chi-square top-10 of 1,000 rows against 65,536 x 128 1,752 us without any
+// scaling, 1,747 so, 1,764 with both scaled when staged.
+inline float chi2_scale(float x_max)
 {
     int e = 0;
     std::frexp(x_max, &e);   // x_max < 2^e
     const int s = x_max > 0.f ? std::min(std::max(40 - e, 0), 126) : 0;
-    return {std::ldexp(1.f, s), std::ldexp(1.f, -s)};
+    return std::ldexp(1.f, s);
 }
 
-// FP32 error of a chi-square distance: |D32 - D| <= chi2_g32(d) D + chi2_abs32(d, scale).
+// FP32 error of a chi-square distance of scaled features: |D32 - D| <= chi2_g32(d) D + chi2_abs32(d).
 //   Relative: a pair of terms, (t1^2 u2 + t2^2 u1) / (u1 u2), has at most 11 roundings of 2^-24 on
 //   any path (rcp.approx counted as two) and d / 2 accumulations follow: below (d + 16) 2^-23.
-//   Absolute, per pair of terms of scaled features: the clamp (2 x 2^-50) and what underflows below the
-//   normal range (2^-150 / (u1 u2) <= 2^-50 for each product, u >= 2^-50): below 2^-47, so d 2^-48 in
-//   all; scaled back, and half a subnormal step for the rounding of that.
+//   Absolute, per pair of terms: the clamp (2 x 2^-50) and what underflows below the normal range
+//   (2^-150 / (u1 u2) <= 2^-50 for each product, u >= 2^-50): below 2^-47, so d 2^-48 in all.
 inline double chi2_g32(int d) { return (d + 16) * 1.1920928955078125e-07; }
-inline double chi2_abs32(int d, Chi2Scale c) { return d * 3.552713678800501e-15 * c.down + 1.401298464324817e-45; }
+inline double chi2_abs32(int d) { return d * 3.552713678800501e-15; }
 
 // Packed pairs of floats (add / mul / fma.f32x2): each half rounds as the scalar operation does.
 __device__ __forceinline__ uint64_t pack2(float x, float y)
@@ -87,17 +84,17 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 }
 
 // Adds the terms k and k + 1 of metric M for a pair (a, b) of feature values to acc:
-//   M = 0: squared L2; M = 1: L1; M = 2: chi-square on non-negative features, times c.up. One reciprocal
+//   M = 0: squared L2; M = 1: L1; M = 2: chi-square on non-negative features, times `up`. One reciprocal
 //   serves two chi-square terms: the MUFU unit (16 lanes an SM) would otherwise bound the loop. Packed:
 //   the two features' scaling, sum and difference take three instructions.
 template <int M>
-__device__ __forceinline__ void dist_terms(float a0, float a1, float b0, float b1, const Chi2Scale c, float &acc)
+__device__ __forceinline__ void dist_terms(float a0, float a1, float b0, float b1, float up, float &acc)
 {
     if constexpr (M == 2) {
-        const uint64_t b = pack2(b0, b1), as = mul2(pack2(a0, a1), pack2(c.up, c.up));
-        const uint64_t t = fma2(b, pack2(-c.up, -c.up), as);
+        const uint64_t b = pack2(b0, b1), as = mul2(pack2(a0, a1), pack2(up, up));
+        const uint64_t t = fma2(b, pack2(-up, -up), as);
         float u0, u1, s0, s1, r;
-        unpack2(fma2(b, pack2(c.up, c.up), as), u0, u1);
+        unpack2(fma2(b, pack2(up, up), as), u0, u1);
         u0 = fmaxf(u0, kChi2Floor);
         u1 = fmaxf(u1, kChi2Floor);
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(u0 * u1));
@@ -117,10 +114,11 @@ __device__ __forceinline__ void dist_terms(float a0, float a1, float b0, float b
 
 // dist_terms for two neighbouring columns at once: the row's features twice in a0 / a1, the
 // columns' in b0 / b1, the same operations and roundings (b (-1) + a rounds once, as a - b).
+// Chi-square: the rows' features come scaled, the columns' are scaled here, within those two FMAs.
 template <int M>
-__device__ __forceinline__ void dist_terms2(uint64_t a0, uint64_t a1, uint64_t b0, uint64_t b1, float &c0, float &c1)
+__device__ __forceinline__ void dist_terms2(uint64_t a0, uint64_t a1, uint64_t b0, uint64_t b1, float up, float &c0, float &c1)
 {
-    const uint64_t m1 = pack2(-1.f, -1.f);
+    const uint64_t m1 = M == 2 ? pack2(-up, -up) : pack2(-1.f, -1.f);
     const uint64_t t0 = fma2(b0, m1, a0), t1 = fma2(b1, m1, a1);
     if constexpr (M == 0) {
         uint64_t c = pack2(c0, c1);
@@ -137,8 +135,8 @@ __device__ __forceinline__ void dist_terms2(uint64_t a0, uint64_t a1, uint64_t b
         c1 += fabsf(y);
     } else {
         float x, y, z, w, p, q, rp, rq;
-        unpack2(add2(a0, b0), x, y);
-        unpack2(add2(a1, b1), z, w);
+        unpack2(fma2(b0, pack2(up, up), a0), x, y);
+        unpack2(fma2(b1, pack2(up, up), a1), z, w);
         const uint64_t u0 = pack2(fmaxf(x, kChi2Floor), fmaxf(y, kChi2Floor)), u1 = pack2(fmaxf(z, kChi2Floor), fmaxf(w, kChi2Floor));
         unpack2(mul2(u0, u1), p, q);
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(p));
@@ -170,14 +168,14 @@ __device__ __forceinline__ void load_slice8(const float *__restrict__ x, bool ro
 }
 
 // acc[i][j] = distance of rows r0 + simt_sub(ty, i) of R and c0 + simt_sub(tx, j) of S, with
-// tx = tid & 15 and ty = tid >> 4 (cs: chi-square only). Every thread of the CTA (256) calls it.
+// tx = tid & 15 and ty = tid >> 4; chi-square: times `up`. Every thread of the CTA (256) calls it.
 __device__ __forceinline__ int simt_sub(int t, int i) { return (i < 4) ? t * 4 + i : 64 + t * 4 + i - 4; }
 
 template <int M, bool VEC>
 __device__ __forceinline__ void simt_tile(const float *__restrict__ R, const float *__restrict__ S, int nR, int nS, int d,
-                                          int r0, int c0, const Chi2Scale cs, SimtSmem &sm, float (&acc)[8][8])
+                                          int r0, int c0, float up, SimtSmem &sm, float (&acc)[8][8])
 {
-    auto staged = [&](float x) { return M == 2 ? x * cs.up : x; };
+    auto staged = [&](float x) { return M == 2 ? x * up : x; };
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int row = tid & 127, kh = (tid >> 7) * 8;   // this thread stages features kh .. kh + 7 of a slice
     const bool a_ok = r0 + row < nR, b_ok = c0 + row < nS;
@@ -194,7 +192,7 @@ __device__ __forceinline__ void simt_tile(const float *__restrict__ R, const flo
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         sm.a[0][kh + e][row] = staged(va[e]);
-        sm.b[0][kh + e][row] = staged(vb[e]);
+        sm.b[0][kh + e][row] = vb[e];
     }
     __syncthreads();
     for (int k0 = 0; k0 < d; k0 += kSimtK) {
@@ -218,23 +216,17 @@ __device__ __forceinline__ void simt_tile(const float *__restrict__ R, const flo
 #pragma unroll
                 for (int j = 0; j < 8; j += 2)
                     dist_terms2<M>(pack2(a[0][i], a[0][i]), pack2(a[1][i], a[1][i]), pack2(b[0][j], b[0][j + 1]), pack2(b[1][j], b[1][j + 1]),
-                                   acc[i][j], acc[i][j + 1]);
+                                   up, acc[i][j], acc[i][j + 1]);
         }
         if (more) {
             buf ^= 1;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 sm.a[buf][kh + e][row] = staged(va[e]);
-                sm.b[buf][kh + e][row] = staged(vb[e]);
+                sm.b[buf][kh + e][row] = vb[e];
             }
             __syncthreads();
         }
-    }
-    if constexpr (M == 2) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] *= cs.down;
     }
 }
 
