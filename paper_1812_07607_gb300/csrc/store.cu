@@ -2,9 +2,9 @@
 //
 // A store keeps a patch collection resident on the GPU (the in-memory form of
 // "materialize", Sec. 3.2 / Sec. 4.1 of the paper): int64 ids, the FP32
-// feature rows (the ground truth), a zero-padded BF16 copy for the tensor
-// cores, and per-row / per-32-row-chunk statistics from which the join
-// kernels derive sound error bounds.
+// feature rows (the ground truth), a zero-padded 16-bit copy (FP16 with one
+// scale, or BF16) for the tensor cores, and per-row / per-32-row-chunk
+// statistics from which the join kernels derive sound error bounds.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

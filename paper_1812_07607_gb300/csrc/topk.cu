@@ -15,8 +15,10 @@
 //                      that can still be in the top k;
 //   k_topk_canon       their canonical FP64 distances;
 //   k_topk_out         per row: an exact rank by (D64, caller's store row index).
-// About k f columns of a row are listed: f balances the first pass against them (topk_stride). A row
-// with more than its list holds (near-duplicates side by side in the store) gets a tighter threshold
+// About k f columns of a row are listed: f balances the first pass against them (topk_stride). (While k
+// stays well below the 1,024 maxima that k_topk_theta keeps apart: 256 rows against 262,144 x 128 take
+// 0.98 ms at k = 700, and 24 at k = 1,024, with some 8,000 columns a row, more passes and a seventh of the
+// rows scanned; the heaps below took 83 and 87.) A row with more than its list holds (near-duplicates side by side in the store) gets a tighter threshold
 // from the distances it did list and the rows like it another pass (k_topk_refine); one that
 // overflows again takes
 //   k_topk_fallback    an exact scan of the whole store for that row (FP32 bound + radix select +
@@ -83,11 +85,12 @@ __global__ void __launch_bounds__(256) k_rowpar_topk(const double *__restrict__ 
 // column of the top k has h + E + slack >= T, so the row lists the columns whose h~ reaches
 // (T - slack) - E (-inf with fewer than k groups). Padding rows (+inf) list nothing. One warp per row,
 // 32 values a lane (groups folded by maximum past 1,024: disjoint groups stay disjoint), no barriers;
-// T is found bit by bit from the values' common prefix on and cut off after kTkBits bits, downwards,
-// which lets in about one column more in 2^kTkBits. A row's groups are loaded all at once: what bounds
-// a few rows is that latency (one row of 976 groups: 4 us, 18 with a load at a time), what bounds many
-// the counting steps (4,096 rows of 1,953 groups, k = 100: 54 us; 66 so, 105 with a CTA a row and all
-// 32 bits besides). It also empties the rows' lists.
+// T is found bit by bit from the values' common prefix on and cut off after kTkBits bits, downwards. That
+// resolves T to 2^-14 of its octave where the maxima share one, and to 2^-5 of it where they have both
+// signs (the sign and the exponent take nine of the bits), which lets more columns in. A row's groups are
+// loaded all at once: what bounds a few rows is that latency (one row of 976 groups: 4 us, 18 with a load
+// at a time), what bounds many the counting steps (4,096 rows of 1,953 groups, k = 100: 54 us; 66 with a
+// load at a time, 105 with a CTA a row and all 32 bits besides). It also empties the rows' lists.
 constexpr int kTkBits = 14;
 
 __global__ void __launch_bounds__(256) k_topk_theta(const float4 *__restrict__ rowpar, const float *__restrict__ gmax, int n_groups,
@@ -574,8 +577,8 @@ static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Every how many-th tile the first pass takes. That pass costs 2 d nS / f operations a row, and about
 // k f columns of a row are listed at some 0.2 ns each (a slow-path visit and an 8 d byte recheck):
-// the sum is least at f = sqrt(d nS / (1.6e5 k)). At most 16 (a row's list grows with f), and at
-// least 8 k groups of 16 columns stay.
+// the sum is least at f = sqrt(d nS / (1.6e5 k)). At most 16 (a row's list grows with f), and above 1
+// only as far as 8 k groups of 16 columns stay.
 static int topk_stride(int64_t nS, int dp, int k)
 {
     const double f = std::sqrt((double)nS * dp / (1.6e5 * k));

@@ -1,9 +1,9 @@
 """Top-k against a store in cluster order does what it does against the same rows in norm order.
 
 Views of one object lie side by side there, and thresholds from maxima of neighbouring columns would let
-most of a cluster into every row's list. As many listing passes have to do as in norm order, no more rows
-may need the exact scan (but for chance: which rows a list misses by little depends on their order), and
-ids and distances stay bit-exact: k from 1 to 100, both 16-bit formats, unit rows (equal norms), a batch,
+most of a cluster into every row's list. As many listing passes have to do as in norm order and no more
+rows may need the exact scan, but for chance: a row or two whose list overflows by little, which depends
+on the rows' order, cost a pass (six kernels). Ids and distances stay bit-exact: k from 1 to 100, both 16-bit formats, unit rows (equal norms), a batch,
 and a device without the memory for the copy that the passes run on.
 """
 
@@ -36,6 +36,10 @@ def call(dl, Q, S, k, **kw):
     return out
 
 
+def as_good(st, norm):
+    return st["band_pairs"] <= 2 * norm["band_pairs"] + 2 and st["kernels_launched"] <= norm["kernels_launched"] + 6
+
+
 @pytest.mark.parametrize("precision", ["fp16", "bf16"])
 @pytest.mark.parametrize("k", [1, 10, 100])
 def test_as_in_norm_order(dl, orc, data, k, precision):
@@ -48,7 +52,7 @@ def test_as_in_norm_order(dl, orc, data, k, precision):
     assert (ids[:60] == sid[oi]).all() and (d2[:60] == od).all()
     ni, nd, nst = call(dl, Q, _store(dl, sid, X), k, precision=precision)
     assert (ids == ni).all() and (d2 == nd).all()
-    assert st["band_pairs"] <= 2 * nst["band_pairs"] and st["kernels_launched"] <= nst["kernels_launched"]
+    assert as_good(st, nst)
 
 
 @pytest.mark.parametrize("k", [1, 10, 100])
@@ -60,7 +64,7 @@ def test_unit_rows(dl, data, k):
     ids, d2, st = call(dl, Q, S, k, metric="cosine")
     ni, nd, nst = call(dl, Q, N, k, metric="cosine")
     assert (ids == ni).all() and (d2 == nd).all()
-    assert st["band_pairs"] <= 2 * nst["band_pairs"] and st["kernels_launched"] <= nst["kernels_launched"]
+    assert as_good(st, nst)
 
 
 def test_batch(dl, orc, data):
