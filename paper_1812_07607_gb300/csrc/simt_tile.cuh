@@ -11,7 +11,7 @@
 // Additions and FMAs run as packed pairs (two columns an instruction), half the issue slots. The
 // K loop is not unrolled: its body is 200 to 500 instructions already, and unrolled eight times it
 // left the instruction cache (L1: 29 ms). Measured, 65,536 x 128 self-join (2.1 G pairs): 18.2 ms
-// under L1, 47.4 under chi-square, 16.9 under squared L2; with single instead of packed operations
+// under L1, 46.7 under chi-square, 16.9 under squared L2; with single instead of packed operations
 // 20.8, 55.8 and 20.9; with, besides, one 32-wide buffer and a reciprocal a term 22.0, 70.6, 22.1.
 #pragma once
 

@@ -112,7 +112,9 @@ __host__ __device__ inline int half_format(unsigned max_bits, unsigned min_bits,
 // bound by the tensor cores under the power cap, where fewer toggling bits mean higher clocks:
 // 131,072^2 unit-norm rows, d = 512, back to back, 11 bits 11.87 ms, 10 bits 11.71, 9 bits 11.52, BF16
 // 11.53, with 0.51, 0.75, 1.24 and 2.29 M undecided pairs. Narrower joins are bound by their epilogue
-// (d = 128: 3.33 ms at any width), wider ones by the recheck's longer rows.
+// (d = 128: 3.33 ms at any width), wider ones by the recheck's longer rows. A small call at such a d is not
+// at the cap and settles more pairs than with 11 bits, but one copy serves every call on a store; it still
+// has about half of BF16's undecided pairs.
 static int f16_bits(int dp) { return dp > 256 && dp <= 512 ? 9 : 11; }
 
 struct BuildParams {
