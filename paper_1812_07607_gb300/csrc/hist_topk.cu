@@ -267,18 +267,23 @@ __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
                     for (int k = 0; k < nk; ++k) s = __dadd_rn(s, sh_t[tid][k]);
                 __syncthreads();
             }
-            if (tid < na) cd[a0 + tid] = s;
+            if (tid < na) {
+                cd[a0 + tid] = s;
+                cv[a0 + tid] = __int_as_float(f.s_orig[cl[a0 + tid]]);   // the FP32 distances are done with
+            }
         }
         __syncthreads();
         // 4. exact rank by (canonical distance, caller's store row)
         const int64_t base = (int64_t)f.q_orig[f.row0 + row] * f.k;
         for (int a = tid; a < m; a += 256) {
             const double da = cd[a];
-            const int32_t oa = f.s_orig[cl[a]];
+            const int32_t oa = __float_as_int(cv[a]);
             int rank = 0;
-            for (int bb = 0; bb < m; ++bb) {
+#pragma unroll 4
+            for (int bb = 0; bb < m; ++bb) {   // every load unconditional: ties by the thousand wait for none
                 const double db = cd[bb];
-                rank += (db < da) || (db == da && f.s_orig[cl[bb]] < oa);
+                const int32_t ob = __float_as_int(cv[bb]);
+                rank += (db < da) | ((db == da) & (ob < oa));
             }
             if (rank < f.k) {
                 f.out_ids[base + rank] = f.s_ids[cl[a]];
