@@ -5,7 +5,8 @@
 //
 // Query rows are taken in chunks that bound the scratch memory. For each chunk:
 //   k_hist_dist (many query rows) or k_hist_dist_few (a few)
-//                   the FP32 distance D32 of every (query, store) pair of the chunk;
+//                   the FP32 distance D32 of every (query, store) pair of the chunk (against a few
+//                   store rows: k_hist_select itself);
 //   k_hist_select   one CTA per query row at a time: with |D32 - D| <= g32 D + a32 (the SIMT
 //                   join's bound, which holds for any summation order of the non-negative terms),
 //                   1. a bound T on the row's k-th smallest D32: the k-th smallest of the minima
@@ -33,6 +34,11 @@ constexpr int kHtCap = 8192;     // candidates a row can rank (more: DL_EOVERFLO
 constexpr int kHtShared = 1024;  // candidates kept in shared memory (more: the CTA's global scratch)
 constexpr int kHtGroups = 8;     // column groups of each of the 256 threads
 constexpr int kHtTermK = 32;     // canonical terms of a candidate staged at a time
+// Up to this many store rows a row's CTA forms its distances itself: a launch less, and no tile padded
+// to 128 columns. Whole calls, one kernel against two: L1, d = 64, k = 100, 300 rows against 11, 115 and
+// 500: 52 / 70, 90 / 107 and 115 / 105 us; chi-square 53 / 93, 127 / 157 and 141 / 158; 3,000 rows, d = 11,
+// k = 3, L1, against 32, 115 and 200: 94 / 98, 114 / 100 and 126 / 104.
+constexpr int kHtOwn = 128;
 // Up to this many query rows the distances come from k_hist_dist_few: a warp's lanes share one
 // pair's features (16-byte slices, a shuffle tree per pair), so no work goes into padding a query
 // tile to 128 rows. Whole calls against 65,536 x 128, few against tile: L1 112 / 175 us at 1 row,
@@ -80,34 +86,41 @@ __global__ void __launch_bounds__(256, 2) k_hist_dist(const HistTk f)
     }
 }
 
+// The FP32 distance of one pair by a warp.
+template <int M, bool VEC>
+__device__ __forceinline__ float warp_hist_dist(const float *q, const float *x, int d, float up)
+{
+    const int lane = threadIdx.x & 31;
+    float s = 0.f;
+    if constexpr (VEC) {
+        for (int k = lane * 4; k < d; k += 128) {
+            const float4 a = __ldg(reinterpret_cast<const float4 *>(q + k));
+            const float4 b = __ldg(reinterpret_cast<const float4 *>(x + k));
+            dist_terms<M>(a.x, a.y, b.x, b.y, up, s);
+            dist_terms<M>(a.z, a.w, b.z, b.w, up, s);
+        }
+    } else {
+        for (int k = lane * 2; k < d; k += 64) {
+            const bool two = k + 1 < d;   // an absent second feature is 0 in both rows: a zero term
+            dist_terms<M>(__ldg(q + k), two ? __ldg(q + k + 1) : 0.f, __ldg(x + k), two ? __ldg(x + k + 1) : 0.f, up, s);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 // The same for a few rows: a warp takes store rows in turn and every query row against each.
 template <int M, bool VEC>
 __global__ void __launch_bounds__(256) k_hist_dist_few(const HistTk f)
 {
-    const int lane = threadIdx.x & 31;
     const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
     const float *Q = f.Q + (size_t)f.row0 * f.d;
     for (int j = w; j < f.nS; j += nw) {
         const float *x = f.S + (size_t)j * f.d;
         for (int r = 0; r < f.rows; ++r) {
-            const float *q = Q + (size_t)r * f.d;
-            float s = 0.f;
-            if constexpr (VEC) {
-                for (int k = lane * 4; k < f.d; k += 128) {
-                    const float4 a = __ldg(reinterpret_cast<const float4 *>(q + k));
-                    const float4 b = __ldg(reinterpret_cast<const float4 *>(x + k));
-                    dist_terms<M>(a.x, a.y, b.x, b.y, f.up, s);
-                    dist_terms<M>(a.z, a.w, b.z, b.w, f.up, s);
-                }
-            } else {
-                for (int k = lane * 2; k < f.d; k += 64) {
-                    const bool two = k + 1 < f.d;   // an absent second feature is 0 in both rows: a zero term
-                    dist_terms<M>(__ldg(q + k), two ? __ldg(q + k + 1) : 0.f, __ldg(x + k), two ? __ldg(x + k + 1) : 0.f, f.up, s);
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) f.dist[(size_t)r * f.ld + j] = s;
+            const float s = warp_hist_dist<M, VEC>(Q + (size_t)r * f.d, x, f.d, f.up);
+            if ((threadIdx.x & 31) == 0) f.dist[(size_t)r * f.ld + j] = s;
         }
     }
 }
@@ -140,8 +153,9 @@ __device__ __forceinline__ unsigned cta_kth_bits(int k, unsigned *s_cnt, int &tu
 }
 
 // One query row at a time. What bounds it: reading the row's distances twice (the minima, then the
-// columns under the bound), from L2 or HBM; what follows touches about k columns.
-template <int M>
+// columns under the bound), from L2 or HBM; what follows touches about k columns. OWN: the row's
+// distances are formed here first (stores of up to kHtOwn rows; VEC as in the distance kernels).
+template <int M, bool VEC, bool OWN>
 __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
 {
     __shared__ uint32_t sh_c[kHtShared];
@@ -155,8 +169,15 @@ __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
     __syncthreads();
     int turn = 0;
     for (int row = blockIdx.x; row < f.rows; row += gridDim.x) {
-        const float *D = f.dist + (size_t)row * f.ld;
+        float *D = f.dist + (size_t)row * f.ld;
         const float *q = f.Q + (size_t)(f.row0 + row) * f.d;
+        if constexpr (OWN) {
+            for (int j = tid >> 5; j < f.nS; j += 8) {
+                const float s = warp_hist_dist<M, VEC>(q, f.S + (size_t)j * f.d, f.d, f.up);
+                if ((tid & 31) == 0) D[j] = s;
+            }
+            __syncthreads();
+        }
         auto upper = [&](float v) { return __fmul_ru(__fadd_ru(__fmul_ru(v, 1.0f + f.g32), f.a32), 1.0f + f.slack); };
         auto lower = [&](float v) { return __fsub_rd(__fmul_rd(v, 1.0f - f.g32), f.a32); };
         // 1. the k-th smallest group minimum
@@ -301,15 +322,17 @@ __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
 template <int M, bool VEC>
 void launch_hist_chunk(const HistTk &f, int grid_sel, cudaStream_t st)
 {
-    if (f.nS > 0) {
+    if (f.nS <= kHtOwn) {
+        k_hist_select<M, VEC, true><<<(unsigned)grid_sel, 256, 0, st>>>(f);
+    } else {
         if (f.rows <= few_rows(M))
             k_hist_dist_few<M, VEC><<<(unsigned)std::min((f.nS + 7) / 8, device_sm_count() * 8), 256, 0, st>>>(f);
         else
             k_hist_dist<M, VEC><<<dim3((unsigned)((f.nS + kSimtTile - 1) / kSimtTile), (unsigned)((f.rows + kSimtTile - 1) / kSimtTile)),
                                   256, 0, st>>>(f);
         count_launch();
+        k_hist_select<M, false, false><<<(unsigned)grid_sel, 256, 0, st>>>(f);
     }
-    k_hist_select<M><<<(unsigned)grid_sel, 256, 0, st>>>(f);
     count_launch();
 }
 
@@ -395,7 +418,7 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
         stats->pairs_evaluated = nQ * nS;
         stats->fp64_pairs = (int64_t)hf;
         stats->precision = DL_PREC_FP32;
-        stats->kernels_launched = (int32_t)((nQ + rows - 1) / rows) * (nS > 0 ? 2 : 1);
+        stats->kernels_launched = (int32_t)((nQ + rows - 1) / rows) * (nS > kHtOwn ? 2 : 1);
     }
     return DL_OK;
 }
