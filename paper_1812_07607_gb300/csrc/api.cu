@@ -317,13 +317,17 @@ static int run_pass(const PassCfg &c, PassOut *po)
         }
         if (c.timing) cudaEventRecord(ev[1], st);
         nvtxRangePushA("exact recheck of the band (K6)");
+        // as many CTAs as are resident; more where rows are read feature by feature (d no multiple of 4), whose
+        // warps diverge: 199 M undecided pairs, 8 against 5 an SM: 41.3 and 47 ms at d = 422, 29 and 27 at 424,
+        // 10.5 and 11.0 at 128, 15.6 and 15.4 at 256 (a pruned self-join of 131,072 rows gains at 5)
+        const int fin_grid = sms * ((d & 3) ? 8 : 5);
         if (!rc && c.ip) {
             rc = launch_finalize_ip(band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2, jo, cnt + 3,
-                                    cnt + 2, sms * 5, st, (int)nR, (int)nS);
+                                    cnt + 2, fin_grid, st, (int)nR, (int)nS);
             ++launches;
         } else if (!rc && tc_prec(c.prec)) {
             rc = launch_finalize(band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2, c.t_acc,
-                                 c.t_rej, jo, cnt + 3, cnt + 2, sms * 5, st, (int)nR, (int)nS);
+                                 c.t_rej, jo, cnt + 3, cnt + 2, fin_grid, st, (int)nR, (int)nS);
             ++launches;
         } else if (!rc && c.prec == DL_PREC_FP32 && c.metric != 0) {
             rc = launch_hist_recheck(c.metric, band, cnt + 1, (unsigned long long)c.band_cap, R->x32, S->x32, d, c.e2,
