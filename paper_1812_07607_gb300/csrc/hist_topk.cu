@@ -34,6 +34,10 @@ constexpr int kHtCap = 8192;     // candidates a row can rank (more: DL_EOVERFLO
 constexpr int kHtShared = 1024;  // candidates kept in shared memory (more: the CTA's global scratch)
 constexpr int kHtGroups = 8;     // column groups of each of the 256 threads
 constexpr int kHtTermK = 32;     // canonical terms of a candidate staged at a time
+// Up to this many features, and with more than 32 candidates, a thread forms and adds its candidate's terms
+// alone: staged, 32 - d of 32 threads would wait. Chi-square, 3,000 rows against 147, k = 100, whole
+// calls, a thread alone against staged: d = 3 253 / 431 us, 8 293 / 438, 16 366 / 441; d = 32 no gain.
+constexpr int kHtChain = 16;
 // Up to this many store rows a row's CTA forms its distances itself: a launch less, and no tile padded
 // to 128 columns. Whole calls, one kernel against two: L1, d = 64, k = 100, 300 rows against 11, 115 and
 // 500: 52 / 70, 90 / 107 and 115 / 105 us; chi-square 53 / 93, 127 / 157 and 141 / 158; 3,000 rows, d = 11,
@@ -272,9 +276,19 @@ __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
             m = kept;
         }
         // 3. canonical distances, 32 candidates at a time: every thread forms terms, one per candidate
-        // adds them in order
+        // adds them in order (few features: see kHtChain)
         if (tid == 0 && m) atomicAdd(f.n_fp64, (unsigned long long)m);
-        for (int a0 = 0; a0 < m; a0 += 32) {
+        const bool chain = f.d <= kHtChain && m > 32;   // a thread a candidate
+        if (chain) {
+            for (int a = tid; a < m; a += 256) {
+                const float *x = f.S + (size_t)cl[a] * f.d;
+                double s = 0.0;
+                for (int k = 0; k < f.d; ++k) s = __dadd_rn(s, canon_term<M>(__ldg(q + k), __ldg(x + k)));
+                cd[a] = s;
+                cv[a] = __int_as_float(f.s_orig[cl[a]]);
+            }
+        }
+        for (int a0 = chain ? m : 0; a0 < m; a0 += 32) {
             const int na = min(32, m - a0);
             double s = 0.0;
             for (int k0 = 0; k0 < f.d; k0 += kHtTermK) {
