@@ -41,8 +41,10 @@ constexpr int kHtChain = 16;
 // Up to this many store rows a row's CTA forms its distances itself: a launch less, and no tile padded
 // to 128 columns. Whole calls, one kernel against two: L1, d = 64, k = 100, 300 rows against 11, 115 and
 // 500: 52 / 70, 90 / 107 and 115 / 105 us; chi-square 53 / 93, 127 / 157 and 141 / 158; 3,000 rows, d = 11,
-// k = 3, L1, against 32, 115 and 200: 94 / 98, 114 / 100 and 126 / 104.
-constexpr int kHtOwn = 128;
+// k = 3, L1, against 32, 115 and 200: 94 / 98, 114 / 100 and 126 / 104. Where query rows leave SMs idle the
+// line lies higher: 40 rows, d = 64, k = 100, against 200 and 500: L1 81 / 95 and 104 / 106, chi-square
+// 101 / 132 and 120 / 144; d = 11, k = 3, L1, 57 / 58 and 68 / 55.
+constexpr int own_rows(int rows) { return rows <= 256 ? 200 : 128; }
 // Up to this many query rows the distances come from k_hist_dist_few: a warp's lanes share one
 // pair's features (16-byte slices, a shuffle tree per pair), so no work goes into padding a query
 // tile to 128 rows. Whole calls against 65,536 x 128, few against tile: L1 112 / 175 us at 1 row,
@@ -158,7 +160,7 @@ __device__ __forceinline__ unsigned cta_kth_bits(int k, unsigned *s_cnt, int &tu
 
 // One query row at a time. What bounds it: reading the row's distances twice (the minima, then the
 // columns under the bound), from L2 or HBM; what follows touches about k columns. OWN: the row's
-// distances are formed here first (stores of up to kHtOwn rows; VEC as in the distance kernels).
+// distances are formed here first (stores of up to own_rows; VEC as in the distance kernels).
 template <int M, bool VEC, bool OWN>
 __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
 {
@@ -334,9 +336,10 @@ __global__ void __launch_bounds__(256) k_hist_select(const HistTk f)
 }
 
 template <int M, bool VEC>
-void launch_hist_chunk(const HistTk &f, int grid_sel, cudaStream_t st)
+int launch_hist_chunk(const HistTk &f, int grid_sel, cudaStream_t st)   // kernels launched
 {
-    if (f.nS <= kHtOwn) {
+    const bool own = f.nS <= own_rows(f.rows);
+    if (own) {
         k_hist_select<M, VEC, true><<<(unsigned)grid_sel, 256, 0, st>>>(f);
     } else {
         if (f.rows <= few_rows(M))
@@ -348,6 +351,7 @@ void launch_hist_chunk(const HistTk &f, int grid_sel, cudaStream_t st)
         k_hist_select<M, false, false><<<(unsigned)grid_sel, 256, 0, st>>>(f);
     }
     count_launch();
+    return own ? 1 : 2;
 }
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -405,6 +409,7 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
     unsigned long long *nf = (unsigned long long *)(err + 2);
     f.err = err;
     f.n_fp64 = nf;
+    int launches = 0;
     cudaError_t e = cudaMemsetAsync(err, 0, 16, st);
     for (int64_t r0 = 0; r0 < nQ && e == cudaSuccess; r0 += rows) {
         f.row0 = r0;
@@ -412,9 +417,9 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
         const bool vec = (d & 3) == 0;   // store rows start on 16 bytes
         const int gs = std::min(f.rows, sel);
         if (metric == 1)
-            vec ? launch_hist_chunk<1, true>(f, gs, st) : launch_hist_chunk<1, false>(f, gs, st);
+            launches += vec ? launch_hist_chunk<1, true>(f, gs, st) : launch_hist_chunk<1, false>(f, gs, st);
         else
-            vec ? launch_hist_chunk<2, true>(f, gs, st) : launch_hist_chunk<2, false>(f, gs, st);
+            launches += vec ? launch_hist_chunk<2, true>(f, gs, st) : launch_hist_chunk<2, false>(f, gs, st);
         e = cudaGetLastError();
     }
     int herr = 0;
@@ -432,7 +437,7 @@ int hist_topk(const dl_store *Q, const dl_store *S, int metric, int k, int64_t *
         stats->pairs_evaluated = nQ * nS;
         stats->fp64_pairs = (int64_t)hf;
         stats->precision = DL_PREC_FP32;
-        stats->kernels_launched = (int32_t)((nQ + rows - 1) / rows) * (nS > kHtOwn ? 2 : 1);
+        stats->kernels_launched = launches;
     }
     return DL_OK;
 }
