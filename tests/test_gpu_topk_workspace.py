@@ -57,6 +57,14 @@ def test_rows_past_the_shared_list_exact(dl, orc, bad, k):
     assert st["band_pairs"] <= bad
 
 
+def test_rows_that_no_threshold_helps_are_scanned_at_once(dl, orc):
+    """Every row reaches every column: a first listing, one with the list's size, no tightened ones."""
+    g = W.rng(8630)
+    S, Q = offset(g, 20_000, 16), offset(g, 300, 16)
+    st = check_topk(dl, orc, Q, S, 10)
+    assert st["band_pairs"] == 300 and st["kernels_launched"] <= 1 + 7 + 7 + 1   # setup, passes, the scan
+
+
 def test_more_columns_than_the_list_ever_holds(dl, orc):
     """One tile of rows that reach 1.2 million columns each: more than a gigabyte of candidates."""
     g = W.rng(8640)
