@@ -275,6 +275,12 @@ __global__ void __launch_bounds__(256) k_topk_refine(const TopkRows f, const dou
     }
 }
 
+__global__ void __launch_bounds__(256) k_topk_name(int *__restrict__ rows, int row0, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) rows[i] = row0 + i;
+}
+
 // One warp per query row: the columns of its list that can still be in the top k, moved to the list's
 // front (their count becomes the row's) and named in the chunk's kept list. A row whose list
 // overflowed is named in over_rows instead (n_over: how many, and above bit 32 those not yet left to the
@@ -890,6 +896,13 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                     return done(DL_ETIMEOUT);
                 }
                 redo = h[4] > (unsigned long long)cand_cap;   // lists short of candidates: what came of them is written again
+                // nearly every column of nearly every row: no lists, the chunk's rows all take the scan
+                if (redo && 4 * n_groups >= 5 * k && 8 * h[4] > 7ULL * (unsigned long long)cr * (unsigned long long)nS) {
+                    k_topk_name<<<(unsigned)((cr + 255) / 256), 256, 0, st>>>(frows + flagged, (int)row0, (int)cr);
+                    rc = launched("k_topk_name launch");
+                    flagged += cr;
+                    break;
+                }
                 if (redo && (cand_cap < cand_max || chunk_rows > 128)) {   // again, with the list's exact size or fewer rows
                     const int64_t want = (int64_t)(h[4] + h[4] / 8) + 1024;
                     if (cand_cap < cand_max) {
@@ -910,9 +923,9 @@ int topk_core(const dl_store *Q, const dl_store *S, int k, const int *row_k, con
                 // rows that no threshold helps, the bound being as wide as the distances lie apart: three
                 // quarters of all columns past one from enough groups, or a tighter one that left nearly
                 // every row and candidate. 3,000 rows against 3,737 x 76 with an offset, k = 100: 4.2 ms with
-                // every row tightened twice and scanned in the end, 2.9 so (3.0 with the heaps).
+                // every row tightened twice and scanned in the end, 2.9 so, 2.2 without lists at all (3.0 with the heaps).
                 const bool stuck = refined > 0 ? 10 * (h[0] >> 32) > 9 * open && 4 * h[4] > 3 * listed
-                                               : n_groups >= 2 * k && 4 * h[4] > 3ULL * (unsigned long long)cr * (unsigned long long)nS;
+                                               : 4 * n_groups >= 5 * k && 4 * h[4] > 3ULL * (unsigned long long)cr * (unsigned long long)nS;
                 if (!redo && ((h[0] >> 32) == 0 || refined == kTkRefines || stuck)) {
                     flagged += (int64_t)(h[0] & 0xffffffffULL);
                     fp64 += (int64_t)h[5];

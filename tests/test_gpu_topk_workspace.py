@@ -65,6 +65,15 @@ def test_rows_that_no_threshold_helps_are_scanned_at_once(dl, orc):
     assert st["band_pairs"] == 300 and st["kernels_launched"] <= 1 + 7 + 7 + 1   # setup, passes, the scan
 
 
+def test_no_lists_where_every_column_passes(dl, orc):
+    """Known after the first listing: no second one, and rows with near columns are still exact."""
+    g = W.rng(8635)
+    S = np.concatenate([offset(g, 20_000, 16), W.dirichlet_histograms(g, 50, 16)])
+    Q = np.concatenate([offset(g, 300, 16), W.dirichlet_histograms(g, 3, 16)])
+    st = check_topk(dl, orc, Q, S, 10)
+    assert st["band_pairs"] == 303 and st["kernels_launched"] <= 1 + 7 + 1 + 1   # setup, passes, the names, the scan
+
+
 def test_more_columns_than_the_list_ever_holds(dl, orc):
     """One tile of rows that reach 1.2 million columns each: more than a gigabyte of candidates."""
     g = W.rng(8640)
